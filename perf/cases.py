@@ -4,8 +4,11 @@ Every case goes through the public binding (paper_2602_19873_gb300.nl).  The
 inputs are drawn on the GPU with torch, in the distributions of the framework's
 own workload generators: uniform periodic cubes, the Evrard sphere, the
 jittered-lattice fluid with and without charges, mixtures of Plummer spheres,
-and batches of uneven systems.  Smoothing lengths come from the analytic
-number density of each distribution, masses are equal.
+and batches of uneven systems.  Masses are equal.  Smoothing lengths come from
+the analytic number density of each distribution; where that is far from the
+particles' own counts, in the halos of Plummer spheres, they are then brought
+to the target count (within 2) by the framework's h iteration, as its users do
+before a run.
 
 A case is a dict with
   op         what one pass does (see RUN)
@@ -175,7 +178,13 @@ _DIST = {"uniform": _uniform, "evrard": _evrard, "fluid": _fluid, "plummer": _pl
 
 def _system(c, seed):
     p, h, (lo, hi, per) = _DIST[c["dist"]](_gen(seed), c["n"], c["neighbors"])
-    return p.contiguous(), h.contiguous(), {"lo": lo, "hi": hi, "periodic": per}
+    p, h, box = p.contiguous(), h.contiguous(), {"lo": lo, "hi": hi, "periodic": per}
+    if c["dist"] == "plummer" and c["op"] != "iterate_h":
+        tmp = nl.NeighborList()
+        tmp.iterate_h(p[0], p[1], p[2], h, box, nl.make_params(), c["neighbors"], tol=2.0,
+                      start=nl.NL_HSTART_GIVEN, check=False)
+        tmp.free()
+    return p, h, box
 
 
 def _sizes(c):
@@ -195,7 +204,12 @@ def _batch(c, seed):
         hs.append(h)
         boxes.append({"lo": lo, "hi": hi, "periodic": per})
         offs.append(offs[-1] + n)
-    return torch.cat(ps, 1).contiguous(), torch.cat(hs), boxes, offs
+    p, h = torch.cat(ps, 1).contiguous(), torch.cat(hs)
+    tmp = nl.NeighborList()
+    tmp.iterate_h_batch(p[0], p[1], p[2], h, offs, boxes, nl.make_params(), c["neighbors"], tol=2.0,
+                        start=nl.NL_HSTART_GIVEN, check=False)
+    tmp.free()
+    return p, h, boxes, offs
 
 
 def _charges(g, n):
