@@ -1,26 +1,35 @@
 // Cluster-pair search and list encoding (Sec. II-A, II-B, II-C).
 //
 // One warp per super-cluster (8 i-clusters of M particles), taken from an
-// atomic work counter by a persistent grid.  The warp walks the pre-order
-// octree without a stack (skip indices), reading nodes in coalesced chunks
-// of 32 staged in shared memory.  Every particle of the super-cluster (1 to
-// 4 per lane) is tested against the node box inflated by the larger of its
-// radius and the node's maximum radius, with monotone round-to-nearest gaps
-// so that no pair accepted by the FP32 predicate can be pruned.  Accepted leaves append
-// their j-clusters (MJ particles each, MJ = M or M / 2: the M x MJ tiles of
-// Sec. II-A / III-A) to a per-warp queue, drained 4 j-clusters at a time:
-// their particles are staged in shared memory, 4 x 8 (i-cluster, j-cluster)
-// box pairs are tested in one round (one lane each), and each candidate tile
-// is decided by the exact FP32 predicate on its M x MJ pairs, stopping at the
-// first pair found.  (Finer filters between the two, every i particle against
-// the j-cluster box and a test for tiles whose pairs are all neighbors, cost
-// more than the tile tests they saved.)  Depth-first order yields
-// ascending j-clusters (Sec. II-A), so the (J, mask) list is produced
-// sorted; it is staged per warp (L2 resident) and then encoded:
+// atomic work counter by a persistent grid.  Every step works on 32 items at
+// once, one per lane, and hands the survivors to the next:
+//   1. the pre-order octree without a stack (skip indices), 32 consecutive
+//      nodes at a time against the super-cluster's box inflated by the larger
+//      of its radius and the node's (a half search starts at the leaf of its
+//      own first particle); where the box is wide against the radii, every
+//      particle against the nodes that the box reaches;
+//   2. the j-clusters of the leaves reached (MJ particles each, MJ = M or M / 2:
+//      the M x MJ tiles of Sec. II-A / III-A), 32 at a time against the boxes of
+//      the 8 i-clusters;
+//   3. a few single pairs of each candidate tile by the exact FP32 predicate;
+//   4. all M x MJ pairs of the tiles still undecided, 32 / M tiles at a time.
+// All box tests use monotone round-to-nearest gaps, so that no pair accepted by
+// the FP32 predicate can be pruned.  Depth-first order yields ascending
+// j-clusters (Sec. II-A), so the (J, mask) list is produced sorted; it is staged
+// per warp (L2 resident) and then encoded:
 // u32 count | u8 masks | nibble blocks of 32 differences (Sec. II-B, the
 // layout of Sec. II-C with w = 32), reserved with one atomicAdd in the list
 // buffer.  Super-clusters whose list exceeds the staging capacity or the
 // list buffer are queued in a redo list and re-run by the host after growth.
+//
+// What bounds it: instruction issue (75 % of cycles) and shared-memory wavefronts
+// (60 %), not DRAM.  The lane-per-item steps replaced a walk that tested one node,
+// four j-clusters and one tile at a time with the whole warp: 78.7k -> 20k warp
+// instructions per super-cluster on the Evrard sphere at 2^21; search stage (half
+// lists, CUDA events) 1.18 -> 0.75 ms there, 15.9 -> 9.2 ms on 2^24 particles in
+// 64 Plummer spheres, 3.36 -> 2.20 ms on the 4M-particle fluid.
+#include <type_traits>
+
 #include "nl_internal.cuh"
 
 namespace nlg {
@@ -28,7 +37,18 @@ namespace nlg {
 constexpr int SR_THREADS = 256;
 constexpr int SR_WARPS = SR_THREADS / 32;
 constexpr int WIN_WORDS = 64;
-constexpr uint32_t SR_QCAP = 128;   // j-cluster queue entries per warp (multiple of 4)
+// A super-cluster is wide, and its particles are tested against the nodes, when
+// its box widened by its largest radius exceeds kLoose of its smallest radii, or
+// when the boxes alone have reached more than kLooseMin + kLooseRate j-clusters
+// per entry found.  Typical lists reach 2.5 to 4 j-clusters per entry; kLoose 3 /
+// 5 / 8 gave a search of 9.67 / 9.23 / 9.28 ms on 2^24 particles in 64 Plummer
+// spheres and 0.78 / 0.75 / 0.81 ms on a 2^21-particle Evrard sphere; without the
+// second condition single super-clusters of the halos ran for 10 ms.
+constexpr float kLoose = 5.f;
+constexpr uint32_t kLooseMin = 256, kLooseRate = 6;
+// Single pairs of every candidate tile that are tested first (search stage on
+// the Evrard sphere with 0 / 1 / 2 of them: 0.88 / 0.78 / 0.75 ms).
+constexpr int kProbes = 2;
 
 struct SearchCtl {
     const uint32_t *work;   // NULL: super-clusters 0..count-1, else ids
@@ -235,25 +255,64 @@ __device__ bool half_output(uint32_t cnt, const uint32_t *stJ, const uint8_t *st
     return ok;
 }
 
-// Shared memory of one warp: the super-cluster's particles, a chunk of 32
-// consecutive octree nodes, the queue of candidate j-clusters, the particles
-// and boxes of the 4 j-clusters being tested, and the encoder window.
-// The tile operands are laid out for packed (two-pair) arithmetic: an i
-// particle as (x, y, z, r^2), one 16-byte load per tile (the tile tests are
-// bound by shared-memory bandwidth); the j particles of a lane's two pairs a
-// and b as (xa, xb, ya, yb) and (za, zb, ra^2, rb^2), loaded once per
-// j-cluster.  Squared radii suffice: fl(max(ri, rj)^2) = max(fl(ri^2),
-// fl(rj^2)), squaring being monotone.
+// j-clusters tested together: one per lane, at most 256 particles staged
+template <int MJ>
+constexpr uint32_t sr_batch() { return MJ > 8 ? 256 / MJ : 32; }
+
+// Shared memory of one warp: the super-cluster's particles and the boxes of
+// its 8 i-clusters, the queue of j-clusters that the walk reached, the staged
+// particles of one batch of them, its list of candidate tiles, the masks of
+// the tiles found to hold a pair, and the encoder window.  Particles are
+// (x, y, z, r^2); squared radii suffice: fl(max(ri, rj)^2) = max(fl(ri^2),
+// fl(rj^2)), squaring being monotone.  The boxes are laid out in pairs of
+// clusters for packed arithmetic: (lo.x, lo.x', lo.y, lo.y'), (lo.z, lo.z',
+// r^2, r'^2), (hi.x, hi.x', hi.y, hi.y'), (hi.z, hi.z', 0, 0).
 template <int M, int MJ>
 struct SearchSmem {
-    float4 ip[kSC * M];            // i particles
-    float4 nlo[32], nhi[32];       // node chunk
-    int2 nrg[32];
-    uint32_t jq[SR_QCAP];          // candidate j-clusters, ascending
-    float4 jpA[4 * MJ], jpB[4 * MJ];  // particles of the 4 j-clusters under test
-    float4 ilo[kSC], ihi[kSC];     // boxes of the 8 i-clusters
+    float4 ip[kSC * M];                 // i particles
+    float4 jp[sr_batch<MJ>() * MJ];     // j particles of the batch
+    float4 ibox[kSC / 2][4];            // boxes of the i-clusters, in pairs
+    uint32_t jq[64];                    // j-clusters to test, ascending (ring)
+    uint32_t found[32];                 // per batch slot: tiles holding a pair
+    uint8_t tl[32 * kSC];               // candidate tiles: slot * 8 + i-cluster
     uint32_t win[WIN_WORDS];
 };
+
+// Could some particle of i-cluster box c (pair layout, half e) be a symmetric
+// neighbor of one in box B (b squared radius brr)?  The monotone gaps of
+// boxes_near.
+template <bool PER>
+__device__ __forceinline__ void box_pair_near(const float4 *ib, const float4 &blo, const float4 &bhi,
+                                              float brr, const PerLen &L, bool &n0, bool &n1)
+{
+    const float4 A = ib[0], B = ib[1], C = ib[2], D = ib[3];
+    float g[3][2];
+    if constexpr (PER) {
+        g[0][0] = axis_gap_len<true>(A.x, C.x, blo.x, bhi.x, L.x);
+        g[0][1] = axis_gap_len<true>(A.y, C.y, blo.x, bhi.x, L.x);
+        g[1][0] = axis_gap_len<true>(A.z, C.z, blo.y, bhi.y, L.y);
+        g[1][1] = axis_gap_len<true>(A.w, C.w, blo.y, bhi.y, L.y);
+        g[2][0] = axis_gap_len<true>(B.x, D.x, blo.z, bhi.z, L.z);
+        g[2][1] = axis_gap_len<true>(B.y, D.y, blo.z, bhi.z, L.z);
+    } else {
+        const f32x2 up[3] = {sub2_rn(pk2(blo.x, blo.x), pk2(C.x, C.y)), sub2_rn(pk2(blo.y, blo.y), pk2(C.z, C.w)),
+                             sub2_rn(pk2(blo.z, blo.z), pk2(D.x, D.y))};
+        const f32x2 dn[3] = {sub2_rn(pk2(A.x, A.y), pk2(bhi.x, bhi.x)), sub2_rn(pk2(A.z, A.w), pk2(bhi.y, bhi.y)),
+                             sub2_rn(pk2(B.x, B.y), pk2(bhi.z, bhi.z))};
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            float u0, u1, d0, d1;
+            unpk2(up[ax], u0, u1);
+            unpk2(dn[ax], d0, d1);
+            g[ax][0] = fmaxf(0.f, fmaxf(u0, d0));
+            g[ax][1] = fmaxf(0.f, fmaxf(u1, d1));
+        }
+    }
+    float da, db;
+    sum_sq_x2(pk2(g[0][0], g[0][1]), pk2(g[1][0], g[1][1]), pk2(g[2][0], g[2][1]), da, db);
+    n0 = da <= fmaxf(B.z, brr);
+    n1 = db <= fmaxf(B.w, brr);
+}
 
 // MODE 0: full list.  MODE 1: half search, upper entries and transposed
 // tuples for the record assembly.  MODE 2: half list (each pair stored once,
@@ -262,10 +321,9 @@ template <int M, int MJ, bool PER, int MODE>
 __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCtl ctl)
 {
     constexpr bool HALF = MODE != 0;  // only j-clusters from the own first one on
-    constexpr int NP = (M * MJ) / 32 > 0 ? (M * MJ) / 32 : 1;  // pairs per lane per tile
-    constexpr int JSTEP = 32 / M;
-    constexpr uint32_t R = M / MJ;        // j-clusters per i-cluster
-    constexpr int NPI = (kSC * M) / 32;   // i particles per lane for the pruning tests
+    constexpr uint32_t NB = sr_batch<MJ>();
+    constexpr uint32_t G = 32 / M;        // tiles tested together, M lanes each
+    constexpr int NPI = (kSC * M) / 32;   // i particles per lane
     extern __shared__ __align__(16) unsigned char search_smem[];
     SearchSmem<M, MJ> &S = reinterpret_cast<SearchSmem<M, MJ> *>(search_smem)[threadIdx.x >> 5];
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
@@ -275,9 +333,11 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
     if (slot >= a.stage_slots) return;
     uint32_t *stJ = a.stageJ + (size_t)slot * a.stage_cap;
     uint8_t *stM = a.stageM + (size_t)slot * a.stage_cap;
-    const uint32_t II = lane % M;
-    const uint32_t JJ0 = (lane / M) % MJ;
-    const uint32_t grp = lane >> 3;       // j-cluster slot of this lane in the box round
+    const uint32_t II = lane % M, grp = lane / M;
+    // order in which a group of lanes reads the j particles of its tile: the
+    // groups read different 16-byte columns of the staged clusters (banks)
+    const uint32_t swz = (MJ >= 8 ? 2u * grp : grp) & (uint32_t)(MJ - 1);
+    const uint32_t gbits = (M == 32 ? 0xffffffffu : ((1u << M) - 1u)) << (grp * M);
     const uint32_t count = ctl.count_dev ? min(ctl.count, *ctl.count_dev) : ctl.count;
 
     for (;;) {
@@ -295,219 +355,247 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
         const uint32_t vroot = min(a.sys.root[sy], a.nnodes - 1);
         const uint32_t vend = min((uint32_t)__float_as_int(a.nhi[vroot].w), a.nnodes);
 
-        // i-cluster box of this lane's cluster (lane & 7)
-        if (lane < kSC) {
-            S.ilo[lane] = a.clo[s * kSC + lane];
-            S.ihi[lane] = a.chi[s * kSC + lane];
-        }
-        // pruning particles base + lane + 32 t, staged as (x, y, z, r) for
-        // the tile tests.  Dummies sit at infinity, which no open axis comes
-        // near; on periodic systems they are flagged off as well (a point at
-        // infinity has no meaningful periodic gap).  Per-particle tests, not boxes of several particles:
-        // particles adjacent on the curve can lie far apart in sparse
-        // regions, and a box around them would admit far too many nodes.
-        float4 qp[NPI];
-        float qr[NPI];
-        uint32_t qok = 0;  // bit t: particle t of this lane is real
+        // i-cluster boxes (lane & 7) and the box around all of them
+        float4 slo = a.clo[s * kSC + (lane & 7)], shi = a.chi[s * kSC + (lane & 7)];
         __syncwarp();
+        if (lane < kSC) {
+            float *ib = reinterpret_cast<float *>(&S.ibox[lane >> 1][0]) + (lane & 1);
+            ib[0] = slo.x; ib[2] = slo.y; ib[4] = slo.z; ib[6] = __fmul_rn(slo.w, slo.w);
+            ib[8] = shi.x; ib[10] = shi.y; ib[12] = shi.z; ib[14] = 0.f;
+        }
+#pragma unroll
+        for (int o = 1; o < kSC; o <<= 1) {
+            slo.x = fminf(slo.x, __shfl_xor_sync(0xffffffffu, slo.x, o));
+            slo.y = fminf(slo.y, __shfl_xor_sync(0xffffffffu, slo.y, o));
+            slo.z = fminf(slo.z, __shfl_xor_sync(0xffffffffu, slo.z, o));
+            slo.w = fmaxf(slo.w, __shfl_xor_sync(0xffffffffu, slo.w, o));
+            shi.x = fmaxf(shi.x, __shfl_xor_sync(0xffffffffu, shi.x, o));
+            shi.y = fmaxf(shi.y, __shfl_xor_sync(0xffffffffu, shi.y, o));
+            shi.z = fmaxf(shi.z, __shfl_xor_sync(0xffffffffu, shi.z, o));
+            shi.w = fminf(shi.w, __shfl_xor_sync(0xffffffffu, shi.w, o));
+        }
 #pragma unroll
         for (int t = 0; t < NPI; ++t) {
             const float4 p = a.pos[base + lane + 32 * t];
             const float r = __fmul_rn(a.support, p.w);
-            const float rr = __fmul_rn(r, r);
-            S.ip[lane + 32 * t] = make_float4(p.x, p.y, p.z, rr);
-            const bool real = p.x == p.x;
-            qp[t] = real ? p : make_float4(INFINITY, INFINITY, INFINITY, 0.f);
-            qr[t] = real ? r : 0.f;
-            qok |= real ? 1u << t : 0u;
+            S.ip[lane + 32 * t] = make_float4(p.x, p.y, p.z, __fmul_rn(r, r));
         }
+        // a super-cluster whose box is wide against its radii (particles
+        // adjacent on the curve can lie far apart in sparse regions) would
+        // reach far too many nodes by its box alone: its particles are tested
+        // against every node that its box reaches
+        const float ext = fmaxf(fmaxf(shi.x - slo.x, shi.y - slo.y), shi.z - slo.z);
+        bool loose = !(ext + 2.f * slo.w <= kLoose * shi.w);
+        __syncwarp();
 
-        // open systems, two pruning particles per lane: their coordinates as
-        // packed pairs for the node tests
-        f32x2 qx2 = 0, qy2 = 0, qz2 = 0;
-        if constexpr (!PER && NPI == 2) {
-            qx2 = pk2(qp[0].x, qp[1].x);
-            qy2 = pk2(qp[0].y, qp[1].y);
-            qz2 = pk2(qp[0].z, qp[1].z);
-        }
-        uint32_t cnt = 0, tiles = 0, nvis = 0, lvis = 0, jex = 0, ttests = 0, qn = 0;
+        uint32_t cnt = 0, tiles = 0, nvis = 0, lvis = 0, jex = 0, ttests = 0;
+        uint32_t qh = 0, qt = 0;  // queue of j-clusters, ring positions
         // the half search takes only j-clusters from its own first one on
         int lastJ = HALF ? (int)(base / MJ) - 1 : -1;
 
-        // Test the queued j-clusters, 4 per round, and stage the hits.
-        auto flush = [&]() {
-            for (uint32_t b = 0; b < qn; b += 4) {
-                const uint32_t nq = min(4u, qn - b);
-                // stage the particles and boxes of up to 4 j-clusters
-                __syncwarp();
-                bool cand = false;
-                if (grp < nq) {
-                    const uint32_t Jl = S.jq[b + grp];
+        // Test a batch of up to NB queued j-clusters.
+        auto batch = [&]() {
+            const uint32_t nq = min(NB, qt - qh);
+            // 1. box tests, one j-cluster per lane against the 8 i-clusters
+            const uint32_t J = lane < nq ? S.jq[(qh + lane) & 63u] : 0u;
+            uint32_t cm = 0;
+            if (lane < nq) {
+                const float4 blo = a.jlo[J], bhi = a.jhi[J];
+                const float brr = __fmul_rn(blo.w, blo.w);
 #pragma unroll
-                    for (uint32_t jl = lane & 7; jl < (uint32_t)MJ; jl += 8) {
-                        const float4 p = a.pos[Jl * MJ + jl];
-                        const float r = __fmul_rn(a.support, p.w);
-                        // slot of the lane's pair (a, b) holding jl, and its half
-                        uint32_t slot = jl, half = 0;
-                        if constexpr (NP >= 2) {
-                            const uint32_t t = jl / JSTEP;
-                            slot = (jl - t * JSTEP) + (t >> 1) * 2u * JSTEP;
-                            half = t & 1u;
-                        }
-                        float *pa = reinterpret_cast<float *>(&S.jpA[grp * MJ + slot]);
-                        float *pb = reinterpret_cast<float *>(&S.jpB[grp * MJ + slot]);
-                        pa[half] = p.x;
-                        pa[2 + half] = p.y;
-                        pb[half] = p.z;
-                        pb[2 + half] = __fmul_rn(r, r);
-                    }
-                    // 4 j-clusters x 8 i-cluster boxes, one per lane: may some
-                    // pair be neighbors?
-                    cand = boxes_near<PER>(S.ilo[lane & 7], S.ihi[lane & 7], a.jlo[Jl], a.jhi[Jl],
-                                           box);
-                }
-                const uint32_t bal = __ballot_sync(0xffffffffu, cand);
-                __syncwarp();
-                for (uint32_t q = 0; q < nq; ++q) {
-                    const uint32_t cm = (bal >> (8 * q)) & 0xffu;
-                    if (!cm) continue;
-                    const uint32_t J = S.jq[b + q];
-                    // exact FP32 test of the candidate M x MJ tiles; the j
-                    // operands of the first two pairs stay in registers
-                    uint32_t mask = 0;
-                    ttests += __popc(cm);
-                    const float4 jA0 = S.jpA[q * MJ + JJ0], jB0 = S.jpB[q * MJ + JJ0];
-                    for (uint32_t bits = cm; bits; bits &= bits - 1u) {
-                        const int k = __ffs(bits) - 1;  // candidate tiles only, ascending
-                        const float4 pi = S.ip[k * M + II];
-                        // pair (i, j) is a self pair iff II - jl == delta
-                        const int delta = (int)(J * MJ) - (int)(base + k * M);
-                        bool hit = false;
-                        if constexpr (NP >= 2) {
-                            const f32x2 ix = pk2(pi.x, pi.x), iy = pk2(pi.y, pi.y);
-                            const f32x2 iz = pk2(pi.z, pi.z);
-#pragma unroll
-                            for (int u = 0; u < NP / 2; ++u) {  // stops at the first hit
-                                const uint32_t slot = JJ0 + 2u * u * JSTEP;
-                                const float4 jA = u == 0 ? jA0 : S.jpA[q * MJ + slot];
-                                const float4 jB = u == 0 ? jB0 : S.jpB[q * MJ + slot];
-                                float d2a, d2b;
-                                pair_d2_x2<PER>(pk2(jA.x, jA.y), pk2(jA.z, jA.w), pk2(jB.x, jB.y), ix, iy,
-                                                iz, box, d2a, d2b);
-                                const int ca = (int)II - (int)slot, cb = ca - JSTEP;
-                                const bool h = (d2a < fmaxf(pi.w, jB.z) && ca != delta) ||
-                                               (d2b < fmaxf(pi.w, jB.w) && cb != delta);
-                                if (__any_sync(0xffffffffu, h)) {
-                                    hit = true;
-                                    break;
-                                }
-                            }
-                        } else {
-                            const float d2 = pair_d2<PER>(pi, make_float4(jA0.x, jA0.z, jB0.x, 0.f), box);
-                            hit = __any_sync(0xffffffffu, d2 < fmaxf(pi.w, jB0.z) &&
-                                                              (int)II - (int)JJ0 != delta);
-                        }
-                        if (hit) mask |= 1u << k;
-                    }
-                    if (mask) {
-                        if (lane == 0 && cnt < a.stage_cap) {
-                            stJ[cnt] = J;
-                            stM[cnt] = (uint8_t)mask;
-                        }
-                        ++cnt;
-                        tiles += __popc(mask);
-                    }
+                for (int k = 0; k < kSC; k += 2) {
+                    bool n0, n1;
+                    box_pair_near<PER>(S.ibox[k >> 1], blo, bhi, brr, box, n0, n1);
+                    cm |= (n0 ? 1u << k : 0u) | (n1 ? 2u << k : 0u);
                 }
             }
-            qn = 0;
+            if (__any_sync(0xffffffffu, cm != 0u)) {
+                // 2. stage the j particles
+                for (uint32_t q = lane; q < nq * MJ; q += 32) {
+                    const float4 p = a.pos[S.jq[(qh + q / MJ) & 63u] * MJ + q % MJ];
+                    const float r = __fmul_rn(a.support, p.w);
+                    S.jp[q] = make_float4(p.x, p.y, p.z, __fmul_rn(r, r));
+                }
+                __syncwarp();
+                // 3. single pairs of every candidate tile, one j-cluster per
+                // lane: most tiles that hold a pair are found here (about half
+                // of all pairs of such tiles are neighbors)
+                uint32_t mask = 0;
+                if (cm) {
+#pragma unroll
+                    for (int q = 0; q < kProbes; ++q) {
+                        const float4 pj = S.jp[lane * MJ + ((lane + q * (MJ / 2)) & (MJ - 1))];
+#pragma unroll
+                        for (int k = 0; k < kSC; ++k) {
+                            const float4 pi = S.ip[k * M + (q * (M / 2) + M / 4)];
+                            const float d2 = pair_d2<PER>(pi, pj, box);
+                            // (a self pair has d2 = 0)
+                            if (d2 < fmaxf(pi.w, pj.w) && d2 > 0.f) mask |= 1u << k;
+                        }
+                    }
+                    cm &= ~mask;
+                }
+                S.found[lane] = mask;
+                // list of the other candidate tiles
+                const uint32_t pc = __popc(cm);
+                const uint32_t incl = warp_incl_scan(pc);
+                const uint32_t T = __shfl_sync(0xffffffffu, incl, 31);
+                uint32_t at = incl - pc;
+                for (uint32_t b = cm; b; b &= b - 1u) S.tl[at++] = (uint8_t)(lane * kSC + __ffs(b) - 1);
+                __syncwarp();
+                // 4. exact FP32 test of these tiles, G at a time: a lane holds
+                // one i particle of its group's tile and takes the MJ j
+                // particles in turn
+                auto tiles_test = [&](auto own) {
+                    for (uint32_t t0 = 0; t0 < T; t0 += G) {
+                        const uint32_t e = S.tl[min(t0 + grp, T - 1u)];
+                        const uint32_t sl = e >> 3, k = e & 7u;
+                        const float4 pi = S.ip[k * M + II];
+                        const float4 *jb = S.jp + sl * MJ;
+                        // pair (i, j) is a self pair iff jj == delta
+                        const uint32_t delta = own ? base + k * M + II - S.jq[(qh + sl) & 63u] * MJ : 0u;
+                        const f32x2 ixy = pk2(pi.x, pi.y);
+                        bool hit = false;
+#pragma unroll
+                        for (uint32_t t = 0; t < (uint32_t)MJ; ++t) {
+                            const uint32_t jj = t ^ swz;
+                            const float4 pj = jb[jj];
+                            float d2;
+                            if constexpr (PER) {
+                                d2 = pair_d2<true>(pi, pj, box);
+                            } else {
+                                const f32x2 dxy = sub2_rn(pk2(pj.x, pj.y), ixy);
+                                const float dz = __fsub_rn(pj.z, pi.z);
+                                float x2, y2;
+                                unpk2(mul2_rn(dxy, dxy), x2, y2);
+                                d2 = __fadd_rn(__fadd_rn(x2, y2), __fmul_rn(dz, dz));
+                            }
+                            hit |= d2 < fmaxf(pi.w, pj.w) && (!own || jj != delta);
+                        }
+                        const uint32_t hb = __ballot_sync(0xffffffffu, hit) & gbits;
+                        if (II == 0 && hb) atomicOr(&S.found[sl], 1u << k);
+                    }
+                };
+                const uint32_t J0 = S.jq[qh & 63u];
+                if (J0 * MJ < base + kSC * M && S.jq[(qh + nq - 1u) & 63u] * MJ >= base)
+                    tiles_test(std::true_type{});
+                else
+                    tiles_test(std::false_type{});
+                __syncwarp();
+                // 5. j-clusters with a tile holding a pair
+                mask = S.found[lane];
+                const uint32_t has = __ballot_sync(0xffffffffu, mask != 0u);
+                const uint32_t o = cnt + __popc(has & lanemask_lt());
+                if (mask && o < a.stage_cap) {
+                    stJ[o] = J;
+                    stM[o] = (uint8_t)mask;
+                }
+                cnt += __popc(has);
+                tiles += __popc(mask);
+                ttests += T;
+                __syncwarp();
+            }
+            qh += nq;
         };
 
-        // Stackless pre-order walk of the system's subtree; nodes are read in
-        // coalesced chunks of 32 consecutive nodes staged in shared memory.
-        uint32_t v = vroot, cb = 0;
-        bool have = false, past = false;
-        while (v < vend) {
-            if (!have || v - cb >= 32u) {
-                cb = v;
-                have = true;
-                __syncwarp();
-                const uint32_t u = cb + lane;
-                if (u < vend) {
-                    S.nlo[lane] = a.nlo[u];
-                    S.nhi[lane] = a.nhi[u];
-                    S.nrg[lane] = a.nrng[u];
-                }
-                __syncwarp();
+        // Stackless pre-order walk of the system's subtree, 32 consecutive
+        // nodes at a time: each lane tests one node against the
+        // super-cluster's box (the descendants of a node that fails fail too,
+        // the gaps being monotone), and the walk continues after the subtree
+        // of the last failing node that reaches beyond the chunk.  The
+        // j-clusters of the leaves that pass are queued until a batch is full.
+        uint32_t v = vroot, leaves = 0;  // leaves: of the current chunk, not queued yet
+        if constexpr (HALF) {
+            // start at the leaf that holds the first own particle: the last
+            // node in pre-order whose range begins at or before it (the range
+            // starts ascend in pre-order); 32 probes a round
+            uint32_t hi = vend;  // nodes [v, hi) may be it; v itself begins early enough
+            while (hi - v > 1) {
+                const uint32_t step = (hi - v + 31u) >> 5;
+                const uint32_t u = v + lane * step;
+                const uint32_t m = __ballot_sync(0xffffffffu, u < hi && (uint32_t)a.nrng[min(u, vend - 1)].x <= base);
+                const uint32_t last = 31u - __clz(m | 1u);
+                v += last * step;
+                hi = min(hi, v + step);
             }
-            const float4 nlo = S.nlo[v - cb];
-            const float4 nhi = S.nhi[v - cb];
-            const uint32_t skip = (uint32_t)__float_as_int(nhi.w);
-            // wholly before the own particles: only nodes ahead of the first
-            // accepted leaf can be (that leaf holds particle base, and every
-            // later node in pre-order holds later particles)
-            if (HALF && !past && (uint32_t)S.nrg[v - cb].y <= base) {
-                v = skip > v ? skip : v + 1;
-                continue;
-            }
-            ++nvis;
-            bool near = false;
-            if constexpr (!PER && NPI == 2) {
-                // the gap of each particle to the node box per axis, packed
-                float g[3][2];
-                const f32x2 lo2[3] = {pk2(nlo.x, nlo.x), pk2(nlo.y, nlo.y), pk2(nlo.z, nlo.z)};
-                const f32x2 hi2[3] = {pk2(nhi.x, nhi.x), pk2(nhi.y, nhi.y), pk2(nhi.z, nhi.z)};
-                const f32x2 q2[3] = {qx2, qy2, qz2};
-#pragma unroll
-                for (int ax = 0; ax < 3; ++ax) {
-                    float a0, a1, b0, b1;
-                    unpk2(sub2_rn(lo2[ax], q2[ax]), a0, a1);
-                    unpk2(sub2_rn(q2[ax], hi2[ax]), b0, b1);
-                    g[ax][0] = fmaxf(0.f, fmaxf(a0, b0));
-                    g[ax][1] = fmaxf(0.f, fmaxf(a1, b1));
-                }
-                const f32x2 gx = pk2(g[0][0], g[0][1]), gy = pk2(g[1][0], g[1][1]);
-                const f32x2 gz = pk2(g[2][0], g[2][1]);
-                float d2a, d2b, rra, rrb;
-                sum_sq_x2(gx, gy, gz, d2a, d2b);
-                const float ra = fmaxf(qr[0], nlo.w), rb = fmaxf(qr[1], nlo.w);
-                unpk2(mul2_rn(pk2(ra, rb), pk2(ra, rb)), rra, rrb);
-                near = d2a <= rra || d2b <= rrb;
-            } else {
-#pragma unroll
-                for (int t = 0; t < NPI; ++t)
-                    near |= (!PER || ((qok >> t) & 1u)) && point_near<PER>(qp[t], qr[t], nlo, nhi, box);
-            }
-            if (!__any_sync(0xffffffffu, near)) {
-                v = skip > v ? skip : v + 1;  // always advances
-                continue;
-            }
-            if (skip != v + 1) {  // internal node: descend to its first child
-                ++v;
-                continue;
-            }
-            // leaf: queue its j-clusters not queued yet (leaves can share one)
-            const int2 rg = S.nrg[v - cb];
-            past = true;
-            int Jlo = max(rg.x / MJ, lastJ + 1);
-            const int Jhi = (rg.y - 1) / MJ;
-            ++lvis;
-            if (Jhi >= Jlo) {
-                jex += (uint32_t)(Jhi - Jlo + 1);
-                lastJ = Jhi;
-                while (Jlo <= Jhi) {
-                    if (qn == SR_QCAP) flush();
-                    const uint32_t c = min((uint32_t)(Jhi - Jlo + 1), SR_QCAP - qn);
-                    __syncwarp();
-                    for (uint32_t e = lane; e < c; e += 32) S.jq[qn + e] = (uint32_t)Jlo + e;
-                    __syncwarp();
-                    qn += c;
-                    Jlo += (int)c;
-                }
-            }
-            ++v;
         }
-        flush();
+        int2 rg = make_int2(0, 0);       // particle range of this lane's node
+        int Jlo = 0, Jhi = -1;           // j-clusters of the current leaf, not queued yet
+        for (;;) {
+            while (qt - qh < NB) {
+                if (Jlo <= Jhi) {
+                    const uint32_t c = min((uint32_t)(Jhi - Jlo + 1), 32u);
+                    if (lane < c) S.jq[(qt + lane) & 63u] = (uint32_t)Jlo + lane;
+                    qt += c;
+                    Jlo += 32;
+                    continue;
+                }
+                if (leaves) {  // (leaves can share a j-cluster)
+                    const int b = __ffs(leaves) - 1;
+                    leaves &= leaves - 1u;
+                    Jlo = max(__shfl_sync(0xffffffffu, rg.x, b) / MJ, lastJ + 1);
+                    Jhi = (__shfl_sync(0xffffffffu, rg.y, b) - 1) / MJ;
+                    lastJ = max(lastJ, Jhi);
+                    ++lvis;
+                    jex += (uint32_t)max(Jhi - Jlo + 1, 0);
+                    continue;
+                }
+                if (v >= vend) break;
+                const uint32_t u = v + lane;
+                float4 nlo = make_float4(0.f, 0.f, 0.f, 0.f), nhi = nlo;
+                bool near = false;
+                uint32_t skip = 0;
+                if (u < vend) {
+                    nlo = a.nlo[u];
+                    nhi = a.nhi[u];
+                    rg = a.nrng[u];
+                    skip = (uint32_t)__float_as_int(nhi.w);
+                    // (wholly before the own particles: not for a half search)
+                    near = (!HALF || (uint32_t)rg.y > base) && boxes_near<PER>(slo, shi, nlo, nhi, box);
+                }
+                uint32_t next = max(v + 32u, __reduce_max_sync(0xffffffffu, near ? 0u : skip));
+                leaves = __ballot_sync(0xffffffffu, near && skip == u + 1u);
+                nvis += min(32u, vend - v);
+                // (also when few of the j-clusters reached by boxes hold a pair)
+                loose = loose || jex > kLooseMin + kLooseRate * cnt;
+                if (loose) {
+                    // particles against the leaves and the nodes reaching beyond the chunk
+                    const uint32_t big = __ballot_sync(0xffffffffu, near && skip > v + 32u);
+                    for (uint32_t todo = leaves | big; todo;) {
+                        const int b = __ffs(todo) - 1;
+                        todo &= todo - 1u;
+                        const float4 lo = make_float4(__shfl_sync(0xffffffffu, nlo.x, b), __shfl_sync(0xffffffffu, nlo.y, b),
+                                                      __shfl_sync(0xffffffffu, nlo.z, b), 0.f);
+                        const float4 hi = make_float4(__shfl_sync(0xffffffffu, nhi.x, b), __shfl_sync(0xffffffffu, nhi.y, b),
+                                                      __shfl_sync(0xffffffffu, nhi.z, b), 0.f);
+                        const float nr = __shfl_sync(0xffffffffu, nlo.w, b), nrr = __fmul_rn(nr, nr);
+                        bool any = false;
+#pragma unroll
+                        for (int t = 0; t < NPI; ++t) {
+                            const float4 p = S.ip[lane + 32 * t];
+                            const float gx = axis_gap_len<PER>(p.x, p.x, lo.x, hi.x, box.x);
+                            const float gy = axis_gap_len<PER>(p.y, p.y, lo.y, hi.y, box.y);
+                            const float gz = axis_gap_len<PER>(p.z, p.z, lo.z, hi.z, box.z);
+                            const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(gx, gx), __fmul_rn(gy, gy)), __fmul_rn(gz, gz));
+                            any |= p.x == p.x && d2 <= fmaxf(p.w, nrr);  // (dummies are NaN)
+                        }
+                        if (__any_sync(0xffffffffu, any)) continue;
+                        leaves &= ~(1u << b);
+                        if ((big >> b) & 1u) {  // all later nodes of the chunk lie in its subtree
+                            leaves &= (1u << b) - 1u;
+                            next = max(next, __shfl_sync(0xffffffffu, skip, b));
+                            break;
+                        }
+                    }
+                }
+                v = next;
+            }
+            if (qt == qh) break;
+            __syncwarp();
+            batch();
+        }
         __syncwarp();
+        tiles = warp_sum(tiles);
         const bool staged = cnt <= a.stage_cap;
         bool ok = staged;
         if (!staged) {
