@@ -909,6 +909,7 @@ PassArgs pass_args(const nl_list *nl)
     a.rec_off = nl->rec_off.as<uint32_t>();
     a.perm = nl->perm_pad.as<uint32_t>();
     a.aux = nl->aux.as<float2>();
+    a.aux4 = nl->aux.as<float4>();
     a.n = (uint32_t)nl->n;
     a.nsc = nl->nsc;
     a.sys = nl->tables();
@@ -1653,15 +1654,15 @@ nl_status nl_density_pass(const nl_list *cnl, const float *m, float *rho, void *
     if (half) CK(nl->hsum.ensure((size_t)nl->npad * 8));
     Status *dst = nl->status.as<Status>();
     CK(nl->mark(6, s));
-    if (half) CK(cudaMemsetAsync(&dst->m_absmax, 0, sizeof(unsigned int), s));
-    CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), m, nullptr, nullptr, 0,
-                         nl->aux.as<float2>(), s, half ? &dst->m_absmax : nullptr));
+    CK(cudaMemsetAsync(&dst->m_absmax, 0, sizeof(unsigned int), s));
+    CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), nl->pos.as<float4>(), nl->p.support,
+                         m, nullptr, nullptr, AUX_MASS, nl->aux.p, s, &dst->m_absmax));
     if (half) CK(cudaMemsetAsync(nl->hsum.p, 0, (size_t)nl->npad * 8, s));
     CK(nl->mark(7, s));
     PassArgs a = pass_args(nl);
     a.out0 = rho;
     CK(run_pass(nl, a, PASS_DENSITY, s));
-    if (half) CK(launch_half_finish(a, PASS_DENSITY, nl->npad, s));
+    if (half) CK(launch_half_finish(a, PASS_DENSITY, nl->p.cluster, nl->npad, s));
     CK(nl->mark(8, s));
     return NL_OK;
 }
@@ -1676,10 +1677,11 @@ nl_status nl_force_pass(const nl_list *cnl, int32_t kind, const float *params, c
     nl_list *nl = const_cast<nl_list *>(cnl);
     cudaStream_t s = (cudaStream_t)stream;
     const bool half = nl->p.half_list != 0;
+    const bool sph4 = pass_is_packed(PASS_SPH, nl->p.cluster, jcl(&nl->p), nl->p.support);
     if (half) CK(nl->hf.ensure((size_t)nl->npad * 24));
     if (kind == NL_FORCE_SPH_PRESSURE) {
         if (!m || !rho || !pres) return fail(NL_ERR_ARG, "SPH force needs m, rho and pres");
-        CK(nl->aux.ensure((size_t)nl->npad * 8));
+        CK(nl->aux.ensure((size_t)nl->npad * (sph4 ? 16 : 8)));
     }
     PassArgs a = pass_args(nl);  // after every buffer it points to exists
     a.out0 = ax;
@@ -1687,12 +1689,13 @@ nl_status nl_force_pass(const nl_list *cnl, int32_t kind, const float *params, c
     a.out2 = az;
     if (kind == NL_FORCE_SPH_PRESSURE) {
         CK(nl->mark(6, s));
-        CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), m, pres, rho, 1,
-                             nl->aux.as<float2>(), s));
+        CK(cudaMemsetAsync(&a.st->m_absmax, 0, sizeof(unsigned int), s));
+        CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), nl->pos.as<float4>(), nl->p.support,
+                             m, pres, rho, sph4 ? AUX_SPH4 : AUX_SPH, nl->aux.p, s, &a.st->m_absmax));
         CK(nl->mark(7, s));
         if (half) CK(cudaMemsetAsync(nl->hf.p, 0, (size_t)nl->npad * 24, s));
         CK(run_pass(nl, a, PASS_SPH, s));
-        if (half) CK(launch_half_finish(a, PASS_SPH, nl->npad, s));
+        if (half) CK(launch_half_finish(a, PASS_SPH, nl->p.cluster, nl->npad, s));
         CK(nl->mark(8, s));
     } else if (kind == NL_FORCE_LJ) {
         if (!params) return fail(NL_ERR_ARG, "LJ force needs params {eps, sigma}");
@@ -1704,7 +1707,7 @@ nl_status nl_force_pass(const nl_list *cnl, int32_t kind, const float *params, c
         CK(nl->mark(7, s));
         if (half) CK(cudaMemsetAsync(nl->hf.p, 0, (size_t)nl->npad * 24, s));
         CK(run_pass(nl, a, PASS_LJ, s));
-        if (half) CK(launch_half_finish(a, PASS_LJ, nl->npad, s));
+        if (half) CK(launch_half_finish(a, PASS_LJ, nl->p.cluster, nl->npad, s));
         CK(nl->mark(8, s));
     } else if (kind == NL_FORCE_LJ_COULOMB) {
         if (!params) return fail(NL_ERR_ARG, "LJ + Coulomb needs params {eps, sigma, rc, kc}");
@@ -1722,14 +1725,14 @@ nl_status nl_force_pass(const nl_list *cnl, int32_t kind, const float *params, c
         a.p3 = params[3];
         CK(nl->mark(6, s));
         if (m)
-            CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), m, nullptr, nullptr, 0,
-                                 nl->aux.as<float2>(), s));
+            CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), nullptr, 0.f, m, nullptr, nullptr,
+                                 AUX_CHARGE, nl->aux.p, s));
         else
             CK(cudaMemsetAsync(nl->aux.p, 0, (size_t)nl->npad * 8, s));
         CK(nl->mark(7, s));
         if (half) CK(cudaMemsetAsync(nl->hf.p, 0, (size_t)nl->npad * 24, s));
         CK(run_pass(nl, a, PASS_LJC, s));
-        if (half) CK(launch_half_finish(a, PASS_LJC, nl->npad, s));
+        if (half) CK(launch_half_finish(a, PASS_LJC, nl->p.cluster, nl->npad, s));
         CK(nl->mark(8, s));
     } else {
         return fail(NL_ERR_ARG, "unknown force kind %d", kind);
@@ -1788,7 +1791,7 @@ nl_status nl_neighbor_counts(const nl_list *cnl, uint32_t *counts, void *stream)
     PassArgs a = pass_args(nl);
     a.outc = counts;
     CK(run_pass(nl, a, PASS_COUNT, s));
-    if (half) CK(launch_half_finish(a, PASS_COUNT, nl->npad, s));
+    if (half) CK(launch_half_finish(a, PASS_COUNT, nl->p.cluster, nl->npad, s));
     return NL_OK;
 }
 
@@ -1807,7 +1810,7 @@ nl_status nl_nearest_distance(const nl_list *cnl, float *dist, void *stream)
     PassArgs a = pass_args(nl);
     a.out0 = dist;
     CK(run_pass(nl, a, PASS_MIN, s));
-    if (half) CK(launch_half_finish(a, PASS_MIN, nl->npad, s));
+    if (half) CK(launch_half_finish(a, PASS_MIN, nl->p.cluster, nl->npad, s));
     return NL_OK;
 }
 

@@ -82,7 +82,8 @@ struct Status {
     unsigned int pad2;
     // periodic super-clusters whose neighbors cannot wrap (interior) and the rest
     unsigned int n_int, n_bnd;
-    // half-list density: bits of the largest |m| (sets the fixed-point scale)
+    // density and pressure passes: bits of the largest |input| (half-list
+    // density: sets the fixed-point scale)
     unsigned int m_absmax, pad3;
 };
 
@@ -669,7 +670,10 @@ struct PassArgs {
     const uint8_t *list;
     const uint32_t *rec_off;
     const uint32_t *perm;  // caller index of every padded slot, ~0 for dummies
-    const float2 *aux;     // per padded particle: density m; SPH (m, P/rho^2); LJ + Coulomb (q, 0)
+    const float2 *aux;     // per padded particle: density (m, -1/(2h)); SPH (m, P/rho^2); LJ + Coulomb (q, 0)
+    const float4 *aux4;    // SPH, packed kernel: (3 P/(pi rho^2 h^4), m, -1/(2h), 0)
+    int packed;            // the packed kernel (pass_is_packed)
+    int split;             // packed kernel: warps that share a super-cluster (1, 2, 4, 8)
     uint32_t n, nsc;
     SysTables sys;
     float support;
@@ -703,16 +707,33 @@ __device__ __forceinline__ int half_scale_exp(unsigned int mbits)
     const int e = (int)((mbits >> 23) & 0xffu) - 126;
     return max(-126, min(127, 40 - e));
 }
-// threads 0 = 256; blocks_per_sm 0 = default
+// Tiles of at least 64 pairs run the packed kernel, which takes the cubic
+// spline's support as r = 2h; density and pressure passes on lists of another
+// support need the scalar kernel's range test.
+inline bool pass_is_packed(int kind, int M, int MJ, float support)
+{
+    return M * MJ >= 64 && ((kind != PASS_DENSITY && kind != PASS_SPH) || support == 2.f);
+}
+// The packed LJ kernel sums its terms in units of 24 eps / sigma^2 (sigma^2
+// rounded to FP32 as in the terms).
+__device__ __forceinline__ double lj_unit(int kind, const PassArgs &a)
+{
+    return kind == PASS_LJ && a.packed ? 24.0 * (double)a.p0 / (double)(a.p1 * a.p1) : 1.0;
+}
+// threads 0 = 256; blocks_per_sm 0 = default.  Sets a.packed and a.split.
 cudaError_t launch_pass(const PassArgs &a, int kind, int M, int any_periodic, int num_sms,
                         cudaStream_t s, int threads = 0, int blocks_per_sm = 0);
-// aux[k] = (a[perm[k]], ...) for real padded slots, zero for dummies;
-// amax (optional): atomic max of the bits of |aux.x| (zero it first).
-cudaError_t launch_gather_aux(uint32_t npad, const uint32_t *perm_pad, const float *a,
-                              const float *b, const float *c, int mode, float2 *aux,
+// Pass inputs in SFC order, for real padded slots (values without effect for
+// dummies): AUX_CHARGE aux = (a, 0); AUX_MASS aux = (a, -1/(2h)), -inf when
+// (support h)^2 underflows; AUX_SPH aux = (a, b / c^2); AUX_SPH4 float4
+// (3 b / (pi c^2 h^4), a, -1/(2h), 0).  amax (AUX_MASS, AUX_SPH4): atomic
+// maximum of the bits of |inputs| (zero it first).
+enum AuxMode { AUX_CHARGE = 0, AUX_SPH = 1, AUX_MASS = 2, AUX_SPH4 = 3 };
+cudaError_t launch_gather_aux(uint32_t npad, const uint32_t *perm_pad, const float4 *pos, float support,
+                              const float *a, const float *b, const float *c, int mode, void *aux,
                               cudaStream_t s, unsigned int *amax = nullptr);
 // Outputs of a half-list pass from its sums (any pass kind).
-cudaError_t launch_half_finish(const PassArgs &a, int kind, uint32_t npad, cudaStream_t s);
+cudaError_t launch_half_finish(const PassArgs &a, int kind, int M, uint32_t npad, cudaStream_t s);
 
 // pos[k].xyz = caller position perm_pad[k] (h kept); *max_disp (device, may be
 // NULL) = largest |x_new - pos_ref| over real slots, minimum image per system.

@@ -1,5 +1,7 @@
 // Dispatch of the neighborhood passes (kernels in pass_impl.cuh, one
 // translation unit per pass kind) and the gather of pass inputs.
+#include <algorithm>
+
 #include "nl_internal.cuh"
 
 namespace nlg {
@@ -18,13 +20,22 @@ cudaError_t launch_pass_ljc(const PassArgs &a, int M, int per, int grid, int thr
 cudaError_t launch_pass_min(const PassArgs &a, int M, int per, int grid, int threads,
                           cudaStream_t s);
 
-cudaError_t launch_pass(const PassArgs &a, int kind, int M, int any_periodic, int num_sms,
+cudaError_t launch_pass(const PassArgs &a0, int kind, int M, int any_periodic, int num_sms,
                         cudaStream_t s, int threads, int blocks_per_sm)
 {
-    cudaError_t e = cudaMemsetAsync(&a.st->pass_ticket, 0, 4, s);
+    cudaError_t e = cudaMemsetAsync(&a0.st->pass_ticket, 0, 4, s);
     if (e != cudaSuccess) return e;
     const int tpb = threads ? threads : 256;
-    const int grid = num_sms * (blocks_per_sm ? blocks_per_sm : kPassBlocksPerSM);
+    const int bps = blocks_per_sm ? blocks_per_sm : kPassBlocksPerSM;
+    const int grid = num_sms * bps;
+    PassArgs a = a0;
+    a.packed = pass_is_packed(kind, M, a.mj, a.support);
+    // as many warps of a block share a super-cluster as there are warp slots
+    // (two resident blocks per SM) for each
+    const uint64_t nwork = a.work ? a.nwork : a.nsc;
+    const uint64_t slots = (uint64_t)num_sms * std::min(bps, 2) * (tpb / 32);
+    a.split = 1;
+    while (a.split * 2 <= tpb / 32 && nwork * a.split * 2 <= slots) a.split *= 2;
     switch (kind) {
     case PASS_DENSITY: return launch_pass_density(a, M, any_periodic, grid, tpb, s);
     case PASS_COUNT: return launch_pass_count(a, M, any_periodic, grid, tpb, s);
@@ -36,37 +47,51 @@ cudaError_t launch_pass(const PassArgs &a, int kind, int M, int any_periodic, in
     }
 }
 
-// Gather per-particle pass inputs into SFC order.
-// mode 0: aux = (a, 0); mode 1: aux = (a, b / (c*c)) (SPH: m, P / rho^2).
+// Gather per-particle pass inputs into SFC order (AuxMode).
+template <int MODE>
 __global__ void __launch_bounds__(256) k_gather_aux(uint32_t npad, const uint32_t *__restrict__ perm_pad,
+                                                    const float4 *__restrict__ pos, float support,
                                                     const float *__restrict__ a, const float *__restrict__ b,
-                                                    const float *__restrict__ c, int mode,
-                                                    float2 *__restrict__ aux, unsigned int *amax)
+                                                    const float *__restrict__ c, void *__restrict__ aux,
+                                                    unsigned int *amax)
 {
-    __shared__ unsigned int wmax[8];
-    uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    float2 v = make_float2(0.f, 0.f);
+    constexpr bool MAXIMA = MODE == AUX_MASS || MODE == AUX_SPH4;
+    __shared__ unsigned int wm[8];
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned int mb = 0;
     if (k < npad) {
         const uint32_t o = perm_pad[k];
-        if (o != 0xffffffffu) {
-            v.x = a[o];
-            if (mode == 1) {
-                float rho = c[o];
-                v.y = b[o] / (rho * rho);
-            }
+        const bool real = o != 0xffffffffu;
+        const float x = real ? a[o] : 0.f;
+        float y = 0.f, hneg = -INFINITY, hinv = 0.f;
+        if (MAXIMA && real) {
+            const float h = pos[k].w, r = __fmul_rn(support, h);
+            hinv = 1.f / h;
+            if (__fmul_rn(r, r) > 0.f) hneg = -0.5f * hinv;
         }
-        aux[k] = v;
+        if ((MODE == AUX_SPH || MODE == AUX_SPH4) && real) {
+            const float rho = c[o];
+            y = b[o] / (rho * rho);
+        }
+        if constexpr (MODE == AUX_SPH4) {
+            y = 0.954929658551372015f * y * hinv * hinv * hinv * hinv;  // 3/pi
+            reinterpret_cast<float4 *>(aux)[k] = make_float4(y, x, hneg, 0.f);
+            mb = max(__float_as_uint(fabsf(x)), __float_as_uint(fabsf(y)));
+        } else {
+            reinterpret_cast<float2 *>(aux)[k] = make_float2(x, MODE == AUX_MASS ? hneg : y);
+            mb = __float_as_uint(fabsf(x));
+        }
     }
-    if (!amax) return;  // uniform over the grid
-    // largest |a| of the block, one atomic per block (non-negative floats
-    // order like their bit patterns)
-    unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(v.x)));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        m = threadIdx.x < (blockDim.x >> 5) ? wmax[threadIdx.x] : 0u;
-        m = __reduce_max_sync(0xffffffffu, m);
-        if (threadIdx.x == 0 && m) atomicMax(amax, m);
+    if constexpr (MAXIMA) {
+        // largest of the block, one atomic per block (non-negative floats
+        // order like their bit patterns, NaN above all)
+        mb = __reduce_max_sync(0xffffffffu, mb);
+        if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = mb;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            mb = __reduce_max_sync(0xffffffffu, threadIdx.x < (blockDim.x >> 5) ? wm[threadIdx.x] : 0u);
+            if (threadIdx.x == 0 && mb) atomicMax(amax, mb);
+        }
     }
 }
 
@@ -90,9 +115,10 @@ __global__ void __launch_bounds__(256) k_half_finish(PassArgs a, int kind, uint3
         return;
     }
     if (kind != PASS_DENSITY) {  // forces: the FP64 sums rounded once to FP32
-        a.out0[o] = (float)a.hf[3 * (size_t)k + 0];
-        a.out1[o] = (float)a.hf[3 * (size_t)k + 1];
-        a.out2[o] = (float)a.hf[3 * (size_t)k + 2];
+        const double u = lj_unit(kind, a);
+        a.out0[o] = (float)(a.hf[3 * (size_t)k + 0] * u);
+        a.out1[o] = (float)(a.hf[3 * (size_t)k + 1] * u);
+        a.out2[o] = (float)(a.hf[3 * (size_t)k + 2] * u);
         return;
     }
     const int ex = half_scale_exp(a.st->m_absmax);
@@ -102,9 +128,11 @@ __global__ void __launch_bounds__(256) k_half_finish(PassArgs a, int kind, uint3
     a.out0[o] = v * (0.318309886183790672f * hinv * hinv * hinv);
 }
 
-cudaError_t launch_half_finish(const PassArgs &a, int kind, uint32_t npad, cudaStream_t s)
+cudaError_t launch_half_finish(const PassArgs &a0, int kind, int M, uint32_t npad, cudaStream_t s)
 {
     if (kind < PASS_DENSITY || kind > PASS_MIN) return cudaErrorInvalidValue;
+    PassArgs a = a0;
+    a.packed = pass_is_packed(kind, M, a.mj, a.support);
     k_half_finish<<<(npad + 255) / 256, 256, 0, s>>>(a, kind, npad);
     return cudaGetLastError();
 }
@@ -155,11 +183,18 @@ cudaError_t launch_refresh(uint32_t npad, const uint32_t *perm_pad, const SysTab
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather_aux(uint32_t npad, const uint32_t *perm_pad, const float *a,
-                              const float *b, const float *c, int mode, float2 *aux,
+cudaError_t launch_gather_aux(uint32_t npad, const uint32_t *perm_pad, const float4 *pos, float support,
+                              const float *a, const float *b, const float *c, int mode, void *aux,
                               cudaStream_t s, unsigned int *amax)
 {
-    k_gather_aux<<<(npad + 255) / 256, 256, 0, s>>>(npad, perm_pad, a, b, c, mode, aux, amax);
+    const unsigned grid = (npad + 255) / 256;
+    switch (mode) {
+    case AUX_CHARGE: k_gather_aux<AUX_CHARGE><<<grid, 256, 0, s>>>(npad, perm_pad, pos, support, a, b, c, aux, amax); break;
+    case AUX_SPH: k_gather_aux<AUX_SPH><<<grid, 256, 0, s>>>(npad, perm_pad, pos, support, a, b, c, aux, amax); break;
+    case AUX_MASS: k_gather_aux<AUX_MASS><<<grid, 256, 0, s>>>(npad, perm_pad, pos, support, a, b, c, aux, amax); break;
+    case AUX_SPH4: k_gather_aux<AUX_SPH4><<<grid, 256, 0, s>>>(npad, perm_pad, pos, support, a, b, c, aux, amax); break;
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

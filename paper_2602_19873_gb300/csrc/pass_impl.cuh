@@ -16,25 +16,11 @@
 // is excluded on the fly by index (Sec. II-A).
 #pragma once
 #include "nl_internal.cuh"
+#include "pass_decode.cuh"
 
 namespace nlg {
 
 constexpr int PS_THREADS = 256;
-
-__device__ __forceinline__ uint32_t get_nibble(const uint8_t *body, uint32_t p)
-{
-    uint32_t b = body[p >> 1];
-    return (p & 1u) ? (b >> 4) : (b & 0xfu);
-}
-
-// sqrt.approx.f32: the hardware square root approximation (relative error
-// about 2^-22); exact 0 for 0, so coincident particles need no guard
-__device__ __forceinline__ float sqrt_approx(float x)
-{
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 
 // cubic spline shape on q < 2 (a gather pair of the density pass has
 // q < 2 up to one rounding, where the outer branch is 0 to within 1e-20)
@@ -78,41 +64,6 @@ __device__ __forceinline__ float spline_dw(float q)
     float outer = -0.75f * a * a;
     float inner = -3.f * q + 2.25f * q * q;
     return q < 1.f ? inner : (q < 2.f ? outer : 0.f);
-}
-
-// Decode the next 32 entries of a record (one per lane; Sec. II-B): the
-// block mask is read at nibble offset pos with a funnel shift, each lane
-// finds its info nibble by popcount and its data nibbles by a warp scan of
-// data lengths, and a warp scan of the differences rebuilds the j-cluster
-// indices from prevJ.  Advances pos and prevJ; uncompressed records hold
-// the u32 indices (entry t of lane).
-__device__ __forceinline__ uint32_t decode_block(const uint32_t *body, int compress, uint32_t t,
-                                                 bool valid, uint32_t &pos, uint32_t &prevJ)
-{
-    const unsigned lane = lane_id();
-    uint32_t J;
-    if (compress) {
-        const uint8_t *bodyb = reinterpret_cast<const uint8_t *>(body);
-        const uint32_t w0 = body[pos >> 3];
-        const uint32_t w1 = (pos & 7u) ? body[(pos >> 3) + 1] : 0u;
-        const uint32_t bm = __funnelshift_r(w0, w1, (pos & 7u) * 4u);
-        const bool bit = (bm >> lane) & 1u;
-        const uint32_t nbits = __popc(bm);
-        uint32_t info = bit ? get_nibble(bodyb, pos + 8 + __popc(bm & lanemask_lt())) : 0u;
-        uint32_t ndat = (bit && info < 8u) ? info + 1u : 0u;
-        uint32_t incl = warp_incl_scan(ndat);
-        uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-        uint32_t pd = pos + 8 + nbits + incl - ndat;
-        uint32_t v = 0;
-        for (uint32_t q = 0; q < ndat; ++q) v = (v << 4) | get_nibble(bodyb, pd + q);
-        uint32_t d = !bit ? 1u : (info >= 8u ? info - 6u : v);
-        J = prevJ + warp_incl_scan(d);
-        pos += 8 + nbits + tot;
-    } else {
-        J = valid ? body[t] : 0u;
-    }
-    prevJ = __shfl_sync(0xffffffffu, J, 31);
-    return J;
 }
 
 // Accumulators per i-cluster.  Floating sums are two-level: terms of one
@@ -214,49 +165,6 @@ constexpr int ps_min_blocks()
 {
     return (KIND == PASS_DENSITY || KIND == PASS_COUNT || KIND == PASS_MIN) ? 4
            : (HL || KIND == PASS_LJ) ? 2 : 3;
-}
-
-// Nearest integer of x (ties away from zero) as a 64-bit two's complement
-// word, with integer operations only; |x| < 2^62.  Subnormal x give 0.
-__device__ __forceinline__ unsigned long long fixed_of(float x)
-{
-    const uint32_t b = __float_as_uint(x);
-    const int e = (int)((b >> 23) & 0xffu) - 150;  // |x| = mant * 2^e
-    const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | 0x800000u);
-    unsigned long long q;
-    if (e >= 0)
-        q = m << e;
-    else if (e > -25)
-        q = (m + (1ull << (-e - 1))) >> (-e);
-    else
-        q = 0ull;
-    if (((b >> 23) & 0xffu) == 0u) q = 0ull;
-    return (b >> 31) ? (0ull - q) : q;
-}
-
-// The same for 0 <= x < 2^63 in two 32-bit conversions: hi = floor(x / 2^32)
-// (exact: x / 2^32 is a float), then the remainder x - hi 2^32, exact in
-// FP32 (below 2^32 it is x itself; above, a multiple of ulp(x) >= 2^9 below
-// 2^32), rounded to the nearest integer (ties to even; a remainder of x >=
-// 2^32 is already an integer)
-__device__ __forceinline__ unsigned long long fixed_of_nonneg(float x)
-{
-    const uint32_t hi = __float2uint_rz(__fmul_rn(x, 0x1p-32f));
-    const uint32_t lo = __float2uint_rn(__fmaf_rn(-__uint2float_rn(hi), 0x1p32f, x));
-    return ((unsigned long long)hi << 32) | lo;
-}
-
-// The FP64 value of x with integer operations only (exact for normal x;
-// zero and subnormals, below 1.2e-38, give 0; inf and NaN stay so).
-__device__ __forceinline__ double f64_of(float x)
-{
-    const uint32_t b = __float_as_uint(x);
-    const uint32_t e = (b >> 23) & 0xffu;
-    if (e == 0u) return 0.0;
-    const unsigned long long d = ((unsigned long long)(b >> 31) << 63) |
-                                 ((unsigned long long)(e == 255u ? 2047u : e + 896u) << 52) |
-                                 ((unsigned long long)(b & 0x7fffffu) << 29);
-    return __longlong_as_double((long long)d);
 }
 
 // HL: the list holds every cluster pair once (half list, MJ = M).  Entries
@@ -805,26 +713,27 @@ static cudaError_t launch_mk(const PassArgs &a, int per, int grid, int threads, 
     return cudaGetLastError();
 }
 
-template <int KIND>
+// ALL: every tile shape; otherwise the shapes of fewer than 64 pairs, whose
+// passes all run here.
+template <int KIND, bool ALL>
 static cudaError_t launch_k(const PassArgs &a, int M, int per, int grid, int threads, cudaStream_t s)
 {
     if (threads != 128 && threads != PS_THREADS) return cudaErrorInvalidValue;
-    if (a.half) {
-        switch (M * 100 + a.mj) {
-        case 404: return launch_mk<4, 4, KIND, true>(a, per, grid, threads, s);
-        case 808: return launch_mk<8, 8, KIND, true>(a, per, grid, threads, s);
-        case 1616: return launch_mk<16, 16, KIND, true>(a, per, grid, threads, s);
-        default: return cudaErrorInvalidValue;
-        }
+    const int shape = M * 100 + a.mj;
+    if (shape == 404)
+        return a.half ? launch_mk<4, 4, KIND, true>(a, per, grid, threads, s)
+                      : launch_mk<4, 4, KIND>(a, per, grid, threads, s);
+    if (shape == 804 && !a.half) return launch_mk<8, 4, KIND>(a, per, grid, threads, s);
+    if constexpr (ALL) {
+        if (shape == 808)
+            return a.half ? launch_mk<8, 8, KIND, true>(a, per, grid, threads, s)
+                          : launch_mk<8, 8, KIND>(a, per, grid, threads, s);
+        if (shape == 1616)
+            return a.half ? launch_mk<16, 16, KIND, true>(a, per, grid, threads, s)
+                          : launch_mk<16, 16, KIND>(a, per, grid, threads, s);
+        if (shape == 1608 && !a.half) return launch_mk<16, 8, KIND>(a, per, grid, threads, s);
     }
-    switch (M * 100 + a.mj) {
-    case 404: return launch_mk<4, 4, KIND>(a, per, grid, threads, s);
-    case 808: return launch_mk<8, 8, KIND>(a, per, grid, threads, s);
-    case 804: return launch_mk<8, 4, KIND>(a, per, grid, threads, s);
-    case 1616: return launch_mk<16, 16, KIND>(a, per, grid, threads, s);
-    case 1608: return launch_mk<16, 8, KIND>(a, per, grid, threads, s);
-    default: return cudaErrorInvalidValue;
-    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace nlg

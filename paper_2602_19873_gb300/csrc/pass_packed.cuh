@@ -1,0 +1,791 @@
+// Neighborhood passes with packed pair arithmetic: the pass kernel of every
+// tile shape with at least 64 pairs (8x8, 16x8, 16x16).
+//
+// A warp owns a super-cluster, decodes 32 list entries at a time and stages
+// the j particles of PK_SE of them in shared memory, two j particles of a
+// cluster in each word: (x, x', y, y').  Then it takes the i-clusters in turn:
+// a lane holds one i particle (lane % M), duplicated into packed registers once
+// per stage, and walks the staged entries that list the i-cluster; every step of
+// the pair arithmetic is one f32x2 instruction for the lane's two j particles.
+// With the i-clusters outside and the entries inside, the sums of one i particle
+// are all the registers a lane needs (the sums of 8 i-clusters held at once, with
+// the entries outside, took 126 registers on the force passes), there is one copy
+// of the pair code, and no instruction is spent on i-clusters that an entry does
+// not list.  On half lists the shares of the j particles wait in shared memory,
+// one word per lane and entry, and are summed and added to memory once a stage.
+//
+// The pair terms have no branches.  Kernels that vanish with the distance
+// (density, pressure force) need no range test at all: with s = 1 - q/2 clamped
+// to [0, 1] by the saturating multiply-add and p = q/2, w/2 = min(1/2 - 3 p^2 s,
+// s^3) and -w'/3 = min(p, s)(s + u), u = 2s - 1 clamped, are 0 beyond the support.
+// The others decide with the canonical FP32 predicate and select their
+// coefficient.
+//
+// A scalar form of the terms runs for single entries: those whose pairs may wrap
+// around a periodic face, those holding the self pair where it has to be left
+// out, and all entries when an input is not finite (a status word of the gather
+// kernel).
+//
+// What bounds it: the half-list density pass issues 62 warp instructions per listed
+// 8x8 tile (the scalar kernel: 96), 37 of them the pair terms, with the FMA pipe 56 %
+// and the shared-memory pipe 71 % busy; the half-list force passes are bound by
+// shared-memory bandwidth (89 %: 12 of 18 wavefronts per tile carry the j shares).
+// Pass stage, scalar kernel -> this one (CUDA events): half-list density on 2^24
+// particles 9.10 -> 7.15 ms, pressure force on the 2^21-particle Evrard sphere 2.85
+// -> 1.51, LJ at 4M particles 6.92 -> 4.28, LJ + Coulomb 4.83 -> 3.73; full lists:
+// density and nearest distance on 2M particles 1.38 -> 1.13, pressure force on 300k
+// 0.69 -> 0.30; small systems (split): density of 32k particles 0.48 -> 0.10 ms, of
+// 4096 0.32 -> 0.06 ms.
+//
+// split: W warps of a block share a super-cluster, each working on every W-th
+// stage.  Small systems have fewer super-clusters than the chip has warp slots,
+// and their passes are bound by the latency of one list.
+#pragma once
+#include "nl_internal.cuh"
+#include "pass_decode.cuh"
+
+namespace nlg {
+
+constexpr int PK_THREADS = 256;
+constexpr float PK_FAR = 1e18f;     // position of padding particles: out of every range, finite
+
+__device__ __forceinline__ f32x2 add2_rn(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ f32x2 fma2_rn(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ f32x2 dup2(float a) { return pk2(a, a); }
+
+// a * b + 1 clamped to [0, 1]; NaN gives 0
+__device__ __forceinline__ float sat_fma1(float a, float b)
+{
+    float r;
+    asm("fma.rn.sat.f32 %0, %1, %2, 0f3F800000;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ float sqrt_ftz(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ float rcp_ftz(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// w(q)/2 of the cubic spline: s = sat(1 - q/2), p = q/2.  (Beyond the support s
+// = 0; an infinite or NaN p leaves the other operand of the minimum.)  p comes
+// from the same rounded 1/h as s and the final 1/h^3: the density hardly depends
+// on h, so a rounding of 1/h that all three share cancels.
+__device__ __forceinline__ float spline_half_w(float s, float p)
+{
+    return fminf(fmaf(-3.f, p * p * s, 0.5f), s * s * s);
+}
+
+__device__ __forceinline__ f32x2 spline_half_w2(float s0, float s1, f32x2 p)
+{
+    const f32x2 s = pk2(s0, s1);
+    const f32x2 in = fma2_rn(dup2(-3.f), mul2_rn(mul2_rn(p, p), s), dup2(0.5f));
+    const f32x2 out = mul2_rn(mul2_rn(s, s), s);
+    float i0, i1, o0, o1;
+    unpk2(in, i0, i1);
+    unpk2(out, o0, o1);
+    return pk2(fminf(i0, o0), fminf(i1, o1));
+}
+
+// w'(q)/3 of the cubic spline: s = sat(1 - q/2), pn = -q/2.  -max(pn, -s) is
+// the smaller of q/2 and 1 - q/2: the factor that goes to 0 with the distance
+// keeps its relative accuracy.
+__device__ __forceinline__ float spline_third_dw(float s, float pn)
+{
+    return fmaxf(pn, -s) * (s + __saturatef(fmaf(2.f, s, -1.f)));
+}
+
+__device__ __forceinline__ f32x2 spline_third_dw2(float s0, float s1, f32x2 pn)
+{
+    float p0, p1;
+    unpk2(pn, p0, p1);
+    const f32x2 u = pk2(__saturatef(fmaf(2.f, s0, -1.f)), __saturatef(fmaf(2.f, s1, -1.f)));
+    return mul2_rn(pk2(fmaxf(p0, -s0), fmaxf(p1, -s1)), add2_rn(pk2(s0, s1), u));
+}
+
+// Shared memory of one warp.  Own particles: ia = (x, y, z, a) with a = -1/(2h)
+// (density, pressure) or the squared range (others), ib the pass inputs.  Staged
+// j particles, two (j, j + MJ/2) in a word: ja = (x, x', y, y'), jb = (z, z',
+// b, b'), jc = (c, c', d, d'):
+//   density    b = m;        jc (half lists) = -1/(2h), 1/(2h)
+//   pressure   b = -1/(2h);  jc = C, m
+//   LJ + Coulomb b = squared range; jc = q
+//   LJ, count, nearest: b = squared range
+// js: half lists: the j shares of each lane's pair, per staged entry; full
+// lists: the sums of a warp that shares its super-cluster.
+template <int M, int MJ, int KIND, bool HL>
+struct PkSmem {
+    static constexpr bool FORCE = KIND == PASS_SPH || KIND == PASS_LJ || KIND == PASS_LJC;
+    static constexpr int G = 32 / M;              // lane groups, each with its own j pairs
+    static constexpr int NT = MJ / (2 * G);       // j pairs per lane and entry
+    // list entries staged together: half lists, whose j shares take shared
+    // memory, 8 of 8 particles (more cost the force passes a resident block, and
+    // gave the density pass nothing); full lists 16 (density pass on 2M particles
+    // 1.17 -> 1.11 ms against 8), but the pressure force, whose sums cancel, 8:
+    // longer partials put it 2 % further from FP64 than the scalar kernel
+    static constexpr int SE = HL ? 8 / NT : KIND == PASS_SPH ? 8 : 16;
+    static constexpr int NI = kSC * M;
+    static constexpr int NP = SE * MJ / 2;        // staged pairs
+    static constexpr bool IB = KIND == PASS_SPH || KIND == PASS_LJC || (KIND == PASS_DENSITY && HL);
+    static constexpr bool JC = IB;
+    static constexpr int NC = FORCE ? 3 : 1;      // components of a sum
+    float4 ia[NI];
+    float4 ja[NP], jb[NP];
+    float4 jc[JC ? NP : 1];
+    f32x2 js[HL ? NC * SE * NT * 32 : NC * (kSC / G) * 16];
+    float2 ib[IB ? NI : 2];
+};
+
+// Resident blocks of 256 threads the register budget is cut for (half-list
+// density at 2^24 particles with 3 / 4 / 5: 7.38 / 7.01 / 7.58 ms; half-list LJ at
+// 4M with 2 / 3: 4.77 / 4.35 ms, with 4 its registers spill).
+template <int KIND, bool HL>
+constexpr int pk_min_blocks()
+{
+    return (KIND == PASS_SPH || KIND == PASS_LJ || KIND == PASS_LJC) ? 3 : 4;
+}
+
+// v += b with the running compensation c (Kahan)
+__device__ __forceinline__ void kahan_add(float &v, float &c, float b)
+{
+    const float y = __fsub_rn(b, c);
+    const float t = __fadd_rn(v, y);
+    c = __fsub_rn(__fsub_rn(t, v), y);
+    v = t;
+}
+
+template <int M, int MJ, bool PER, int KIND, bool HL>
+__global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pass_packed(PassArgs a)
+{
+    static_assert(M * MJ >= 64, "a tile fills the lanes with pairs of j particles");
+    static_assert(!HL || M == MJ, "half lists have j-clusters of the i-cluster size");
+    using Smem = PkSmem<M, MJ, KIND, HL>;
+    constexpr uint32_t G = Smem::G, NT = Smem::NT, SE = Smem::SE, HJ = MJ / 2;
+    constexpr uint32_t NK = kSC / G;        // i-clusters whose sums a lane keeps
+    constexpr uint32_t RJ = M / MJ;
+    constexpr bool FORCE = Smem::FORCE;
+    constexpr bool INTS = KIND == PASS_COUNT || KIND == PASS_MIN;
+    constexpr bool SELF_IN_LOOP = KIND == PASS_DENSITY || KIND == PASS_COUNT;
+    constexpr bool NO_SELF = KIND == PASS_LJ || KIND == PASS_LJC || KIND == PASS_MIN;
+    constexpr uint32_t NONE = KIND == PASS_MIN ? 0x7f800000u : 0u;  // empty sum (min: +inf)
+    extern __shared__ __align__(16) unsigned char pk_smem[];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    Smem *const all = reinterpret_cast<Smem *>(pk_smem);
+    Smem &S = all[warp];
+    const uint32_t II = lane % M, g = lane / M;
+    const uint32_t W = (uint32_t)a.split, wig = warp & (W - 1u), grp = warp / W;
+    const uint32_t ngrp = (blockDim.x >> 5) / W;
+    // inputs that are not finite: a zero kernel must not multiply them
+    const bool careful = (KIND == PASS_DENSITY || KIND == PASS_SPH) &&
+                         __any_sync(0xffffffffu, a.st->m_absmax >= 0x7f800000u);
+    // fixed-point scale of the half-list density
+    const float hscale = (HL && KIND == PASS_DENSITY)
+                             ? __int_as_float((half_scale_exp(a.st->m_absmax) + 127) << 23) : 0.f;
+    const float sig2 = a.p1 * a.p1, e24 = 24.f * a.p0;
+    // LJ terms are summed without this factor (half lists: left to the finishing
+    // kernel)
+    const double fscale = lj_unit(KIND, a);
+
+    // running sums take one partial a stage.  Density and pressure (whose sums
+    // cancel) compensated: plain adds left the pressure force of the Evrard
+    // sphere 10 % further from FP64 than the scalar kernel, 3 % less time.  Lennard-
+    // Jones sums are ruled by their nearest pairs: plain adds are as near, and 4 %
+    // faster at 4M particles.
+    auto sum_add = [](float &v, float &c, float b) {
+        if constexpr (KIND == PASS_DENSITY || KIND == PASS_SPH) kahan_add(v, c, b);
+        else v += b;
+    };
+    auto merge = [](uint32_t u, uint32_t v) { return KIND == PASS_COUNT ? u + v : min(u, v); };
+
+    const uint32_t nwork = a.work ? (a.nwork_dev ? min(a.nwork, *a.nwork_dev) : a.nwork) : a.nsc;
+    for (uint32_t it = blockIdx.x + gridDim.x * grp;; it += gridDim.x * ngrp) {
+        uint32_t s = it;
+        if (W == 1u) {
+            if (lane == 0) s = atomicAdd(&a.st->pass_ticket, 1u);
+            s = __shfl_sync(0xffffffffu, s, 0);
+        }
+        if (s >= nwork) break;
+        if (a.work) s = a.work[s];
+        const PerLen box = per_len(a.sys.box[sys_of(a.sys.pad_off, a.sys.nsys, s * kSC * M)]);
+
+        // own particles; the box around them (periodic)
+        float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+        __syncwarp();
+#pragma unroll
+        for (uint32_t t = lane; t < (uint32_t)Smem::NI; t += 32) {
+            const uint32_t i = s * kSC * M + t;
+            float4 p = a.pos[i];
+            const float r = __fmul_rn(a.support, (KIND == PASS_COUNT && a.hq) ? a.hq[i] : p.w);
+            float av = __fmul_rn(r, r);
+            if constexpr (KIND == PASS_DENSITY) {
+                const float2 x = a.aux[i];
+                av = x.y;
+                if constexpr (HL) S.ib[t] = make_float2(x.x, 0.f);
+            } else if constexpr (KIND == PASS_SPH) {
+                const float4 x = a.aux4[i];
+                av = x.z;
+                S.ib[t] = make_float2(x.x, x.y);
+            } else if constexpr (KIND == PASS_LJC) {
+                av = fminf(av, a.p2);
+                S.ib[t] = make_float2(a.p3 * a.aux[i].x, 0.f);
+            }
+            const bool real = p.x == p.x;
+            if constexpr (PER) {
+                if (real) {
+                    lo[0] = fminf(lo[0], p.x); hi[0] = fmaxf(hi[0], p.x);
+                    lo[1] = fminf(lo[1], p.y); hi[1] = fmaxf(hi[1], p.y);
+                    lo[2] = fminf(lo[2], p.z); hi[2] = fmaxf(hi[2], p.z);
+                }
+            }
+            if (!real) p.x = p.y = p.z = PK_FAR;
+            S.ia[t] = make_float4(p.x, p.y, p.z, av);
+        }
+        if constexpr (PER) {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+                for (int x = 0; x < 3; ++x) {
+                    lo[x] = fminf(lo[x], __shfl_xor_sync(0xffffffffu, lo[x], o));
+                    hi[x] = fmaxf(hi[x], __shfl_xor_sync(0xffffffffu, hi[x], o));
+                }
+        }
+        __syncwarp();
+
+        // running sums of the i-clusters g NK .. g NK + NK - 1, particle II
+        // (density: x alone; count, nearest: rc) with their compensations
+        float rx[NK], ry[NK], rz[NK], cx[NK], cy[NK], cz[NK];
+        uint32_t rc[NK];
+#pragma unroll
+        for (uint32_t q = 0; q < NK; ++q) {
+            rx[q] = ry[q] = rz[q] = cx[q] = cy[q] = cz[q] = 0.f;
+            rc[q] = NONE;
+        }
+        uint32_t selfseen = 0;  // bit r: the entry of own j-cluster r lists its own i-cluster
+
+        // a super-cluster whose list was not stored (an overflow inside a graph
+        // replay, reported by nl_graph_check) is read as an empty list
+        const uint32_t roff = a.rec_off[s];
+        const uint32_t *rec = reinterpret_cast<const uint32_t *>(a.list) + (roff == kBadRecord ? 0u : roff);
+        const uint32_t cnt = roff == kBadRecord ? 0u : rec[0];
+        const uint8_t *masks = reinterpret_cast<const uint8_t *>(rec + 1);
+        const uint32_t *body = rec + 1 + ((cnt + 3u) >> 2);
+        uint32_t pos = 0;
+        uint32_t prevJ = 0xffffffffu;
+
+        for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
+            const uint32_t t = b0 + lane;
+            const bool valid = t < cnt;
+            const uint32_t J = decode_block(body, a.compress, t, valid, pos, prevJ);
+            const uint32_t mk = valid ? masks[t] : 0u;
+            const uint32_t rel = J - s * kSC * RJ;  // own j-clusters: below kSC RJ
+            const uint32_t own = __ballot_sync(0xffffffffu, valid && rel < kSC * RJ);
+            if constexpr (SELF_IN_LOOP) {
+                const bool seen = valid && rel < kSC * RJ && ((mk >> (rel / RJ)) & 1u);
+                selfseen |= __reduce_or_sync(0xffffffffu, seen ? 1u << rel : 0u);
+            }
+            // half list: entries beyond the own clusters also feed their j particles
+            const uint32_t feeds = HL ? __ballot_sync(0xffffffffu, valid) & ~own : 0u;
+            for (uint32_t c = 0; c < min(32u, cnt - b0); c += SE) {
+                if (W != 1u && ((b0 + c) / SE & (W - 1u)) != wig) continue;
+                const uint32_t ns = min(SE, cnt - b0 - c);
+                // stage the j particles of entries c .. c + ns - 1
+                uint32_t slow = careful ? 0xffffffffu : 0u;  // bit el: entry c + el takes the scalar terms
+                if constexpr (NO_SELF) slow |= own >> c;
+                __syncwarp();
+#pragma unroll
+                for (uint32_t q0 = 0; q0 < (uint32_t)Smem::NP; q0 += 32) {
+                    const uint32_t q = q0 + lane;
+                    const uint32_t el = q / HJ;
+                    const uint32_t src = __shfl_sync(0xffffffffu, J, min(c + el, 31u)) * MJ + q % HJ;
+                    bool wr = false;
+                    if (el < ns) {
+                        float4 p[2];
+                        float bv[2] = {0.f, 0.f}, cv[2] = {0.f, 0.f}, dv[2] = {0.f, 0.f};
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const uint32_t j = src + h * HJ;
+                            p[h] = a.pos[j];
+                            if constexpr (KIND == PASS_DENSITY) {
+                                const float2 x = a.aux[j];
+                                bv[h] = x.x;
+                                cv[h] = x.y;
+                                dv[h] = -x.y;
+                            } else if constexpr (KIND == PASS_SPH) {
+                                const float4 x = a.aux4[j];
+                                bv[h] = x.z;
+                                cv[h] = x.x;
+                                dv[h] = x.y;
+                            } else {
+                                if constexpr (HL) {
+                                    const float r = __fmul_rn(a.support, p[h].w);
+                                    bv[h] = __fmul_rn(r, r);
+                                    if constexpr (KIND == PASS_LJC) bv[h] = fminf(bv[h], a.p2);
+                                }
+                                if constexpr (KIND == PASS_LJC) cv[h] = a.aux[j].x;
+                            }
+                            if constexpr (PER) {
+                                // (the canonical difference is monotone in both coordinates)
+                                const float hx = __fmul_rn(0.5f, box.x), hy = __fmul_rn(0.5f, box.y);
+                                const float hz = __fmul_rn(0.5f, box.z);
+                                wr = wr || __fsub_rn(p[h].x, lo[0]) > hx || __fsub_rn(p[h].x, hi[0]) < -hx ||
+                                     __fsub_rn(p[h].y, lo[1]) > hy || __fsub_rn(p[h].y, hi[1]) < -hy ||
+                                     __fsub_rn(p[h].z, lo[2]) > hz || __fsub_rn(p[h].z, hi[2]) < -hz;
+                            }
+                            if (!(p[h].x == p[h].x)) p[h].x = p[h].y = p[h].z = PK_FAR;
+                        }
+                        S.ja[q] = make_float4(p[0].x, p[1].x, p[0].y, p[1].y);
+                        S.jb[q] = make_float4(p[0].z, p[1].z, bv[0], bv[1]);
+                        if constexpr (Smem::JC) S.jc[q] = make_float4(cv[0], cv[1], dv[0], dv[1]);
+                    }
+                    if constexpr (PER) {
+                        const uint32_t wb = __ballot_sync(0xffffffffu, wr);
+#pragma unroll
+                        for (uint32_t e = 0; e < 32u / HJ; ++e)
+                            if ((wb >> (e * HJ)) & ((1u << HJ) - 1u)) slow |= 1u << (q0 / HJ + e);
+                    }
+                }
+                if constexpr (HL) {
+                    float4 *z = reinterpret_cast<float4 *>(S.js);
+                    const float zv = KIND == PASS_MIN ? INFINITY : 0.f;
+#pragma unroll
+                    for (uint32_t q = lane; q < sizeof(S.js) / 16; q += 32) z[q] = make_float4(zv, zv, zv, zv);
+                }
+                __syncwarp();
+
+#pragma unroll 1
+                for (uint32_t k = 0; k < kSC; ++k) {
+                    // staged entries that list i-cluster k
+                    uint32_t bits = (__ballot_sync(0xffffffffu, (mk >> k) & 1u) >> c) & ((1u << SE) - 1u);
+                    if (!bits) continue;
+                    const float4 pi = S.ia[k * M + II];
+                    float2 iv = make_float2(0.f, 0.f);
+                    if constexpr (Smem::IB) iv = S.ib[k * M + II];
+                    const f32x2 xi = dup2(pi.x), yi = dup2(pi.y), zi = dup2(pi.z);
+                    const f32x2 hpi = dup2(KIND == PASS_DENSITY ? -pi.w : pi.w);  // 1/(2h), pressure -1/(2h)
+                    const f32x2 ivx = dup2(iv.x), ivy = dup2(iv.y);
+                    f32x2 ax = 0ull, ay = 0ull, az = 0ull;  // the i particle's sums over this stage
+                    uint32_t ac = NONE;
+                    for (uint32_t todo = bits & ~slow; todo; todo &= todo - 1u) {
+                        const uint32_t el = __ffs(todo) - 1;
+#pragma unroll
+                        for (uint32_t tt = 0; tt < NT; ++tt) {
+                            const uint32_t q = el * HJ + g + tt * G;
+                            f32x2 *js = S.js + (el * NT + tt) * 32 + lane;
+                            constexpr uint32_t JS = SE * NT * 32;  // between components
+                            const float4 A = S.ja[q], B = S.jb[q];
+                            const f32x2 dx = sub2_rn(pk2(A.x, A.y), xi), dy = sub2_rn(pk2(A.z, A.w), yi);
+                            const f32x2 dz = sub2_rn(pk2(B.x, B.y), zi);
+                            if constexpr (KIND == PASS_DENSITY) {
+                                float d0, d1;
+                                unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, mul2_rn(dx, dx))), d0, d1);
+                                const float r0 = sqrt_ftz(d0), r1 = sqrt_ftz(d1);
+                                const f32x2 r = pk2(r0, r1);
+                                ax = fma2_rn(pk2(B.z, B.w),
+                                             spline_half_w2(sat_fma1(r0, pi.w), sat_fma1(r1, pi.w), mul2_rn(r, hpi)), ax);
+                                if constexpr (HL) {
+                                    const float4 C = S.jc[q];
+                                    *js = fma2_rn(ivx,
+                                                  spline_half_w2(sat_fma1(r0, C.x), sat_fma1(r1, C.y),
+                                                                 mul2_rn(r, pk2(C.z, C.w))), *js);
+                                }
+                            } else if constexpr (KIND == PASS_SPH) {
+                                // (a self pair: dx = 0; the floor keeps 1/r finite)
+                                float d0, d1;
+                                unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, mul2_rn(dx, dx))), d0, d1);
+                                d0 = fmaxf(d0, 1e-30f);
+                                d1 = fmaxf(d1, 1e-30f);
+                                const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
+                                const f32x2 r = mul2_rn(pk2(d0, d1), ir);
+                                float r0, r1;
+                                unpk2(r, r0, r1);
+                                const float4 C = S.jc[q];
+                                const f32x2 gi = spline_third_dw2(sat_fma1(r0, pi.w), sat_fma1(r1, pi.w), mul2_rn(r, hpi));
+                                const f32x2 gj = spline_third_dw2(sat_fma1(r0, B.z), sat_fma1(r1, B.w), mul2_rn(r, pk2(B.z, B.w)));
+                                const f32x2 b = mul2_rn(fma2_rn(pk2(C.x, C.y), gj, mul2_rn(ivx, gi)), ir);
+                                const f32x2 si = mul2_rn(pk2(C.z, C.w), b);
+                                ax = fma2_rn(si, dx, ax);
+                                ay = fma2_rn(si, dy, ay);
+                                az = fma2_rn(si, dz, az);
+                                if constexpr (HL) {
+                                    const f32x2 sj = mul2_rn(ivy, b);
+                                    js[0] = fma2_rn(sj, dx, js[0]);
+                                    js[JS] = fma2_rn(sj, dy, js[JS]);
+                                    js[2 * JS] = fma2_rn(sj, dz, js[2 * JS]);
+                                }
+                            } else {
+                                float d0, d1;  // the canonical squared distances
+                                sum_sq_x2(dx, dy, dz, d0, d1);
+                                const bool i0 = d0 < pi.w, i1 = d1 < pi.w;
+                                const bool j0 = d0 < B.z, j1 = d1 < B.w;
+                                if constexpr (KIND == PASS_COUNT) {
+                                    ac += (i0 ? 1u : 0u) + (i1 ? 1u : 0u);
+                                    if constexpr (HL) *js += (j0 ? 1ull : 0ull) + (j1 ? 1ull << 32 : 0ull);
+                                } else if constexpr (KIND == PASS_MIN) {
+                                    const uint32_t u0 = __float_as_uint(d0), u1 = __float_as_uint(d1);
+                                    if (i0) ac = min(ac, u0);
+                                    if (i1) ac = min(ac, u1);
+                                    if constexpr (HL) {
+                                        const f32x2 o = *js;
+                                        const uint32_t l = j0 ? min((uint32_t)o, u0) : (uint32_t)o;
+                                        const uint32_t h = j1 ? min((uint32_t)(o >> 32), u1) : (uint32_t)(o >> 32);
+                                        *js = ((f32x2)h << 32) | l;
+                                    }
+                                } else {
+                                    // f: minus the coefficient of dx in the force on j
+                                    float f0, f1;
+                                    if constexpr (KIND == PASS_LJ) {
+                                        // -1/d2 by the hardware reciprocal and one Newton step
+                                        const f32x2 r = pk2(rcp_ftz(-d0), rcp_ftz(-d1));
+                                        const f32x2 e = fma2_rn(pk2(d0, d1), r, dup2(1.f));
+                                        const f32x2 s2 = mul2_rn(dup2(sig2), fma2_rn(r, e, r));
+                                        const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);  // -(sigma/r)^6
+                                        unpk2(mul2_rn(s2, fma2_rn(add2_rn(s6, s6), s6, s6)), f0, f1);
+                                    } else {
+                                        const float4 C = S.jc[q];
+                                        const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
+                                        const f32x2 ir2 = mul2_rn(ir, ir);
+                                        const f32x2 s2 = mul2_rn(dup2(-sig2), ir2);
+                                        const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);
+                                        const f32x2 lj = mul2_rn(dup2(e24), fma2_rn(add2_rn(s6, s6), s6, s6));
+                                        const f32x2 qq = mul2_rn(ivx, pk2(C.x, C.y));
+                                        float t0, t1;
+                                        unpk2(mul2_rn(ir2, fma2_rn(qq, ir, lj)), t0, t1);
+                                        f0 = -t0;
+                                        f1 = -t1;
+                                    }
+                                    // (padding particles are far away: never in range, dx finite)
+                                    const f32x2 fi = pk2(i0 ? f0 : 0.f, i1 ? f1 : 0.f);
+                                    ax = fma2_rn(fi, dx, ax);
+                                    ay = fma2_rn(fi, dy, ay);
+                                    az = fma2_rn(fi, dz, az);
+                                    if constexpr (HL) {
+                                        const f32x2 fj = pk2(j0 ? f0 : 0.f, j1 ? f1 : 0.f);
+                                        js[0] = fma2_rn(fj, dx, js[0]);
+                                        js[JS] = fma2_rn(fj, dy, js[JS]);
+                                        js[2 * JS] = fma2_rn(fj, dz, js[2 * JS]);
+                                    }
+                                }
+                            }
+                        }
+                    }
+                    // scalar terms: canonical predicate, accurate pair vector
+#pragma unroll 1
+                    for (uint32_t todo = bits & slow; todo; todo &= todo - 1u) {
+                        const uint32_t el = __ffs(todo) - 1;
+                        const uint32_t Je = __shfl_sync(0xffffffffu, J, c + el);
+#pragma unroll 1
+                        for (uint32_t th = 0; th < 2 * NT; ++th) {
+                            const uint32_t tt = th >> 1, h = th & 1u;
+                            const uint32_t q = el * HJ + g + tt * G;
+                            float *js = reinterpret_cast<float *>(S.js + (el * NT + tt) * 32 + lane) + h;
+                            constexpr uint32_t JS = SE * NT * 64;
+                            const float *A = reinterpret_cast<const float *>(&S.ja[q]) + h;
+                            const float *B = reinterpret_cast<const float *>(&S.jb[q]) + h;
+                            const float *C = reinterpret_cast<const float *>(&S.jc[Smem::JC ? q : 0]) + h;
+                            const float4 pj = make_float4(A[0], A[2], B[0], B[2]);
+                            const float3 dv = pair_dx_acc<PER>(pi, pj, box);
+                            const float e2 = d2_of(dv);
+                            float fi = 0.f, fj = 0.f;  // coefficients of dv
+                            if constexpr (KIND == PASS_DENSITY) {
+                                const float r = sqrt_approx(e2);
+                                const float wi = spline_half_w(sat_fma1(r, pi.w), r * -pi.w);
+                                if (wi > 0.f) ax = add2_rn(ax, pk2(pj.w * wi, 0.f));
+                                if constexpr (HL) {
+                                    const float wj = spline_half_w(sat_fma1(r, C[0]), r * C[2]);
+                                    if (wj > 0.f) *js += iv.x * wj;
+                                }
+                            } else if constexpr (KIND == PASS_SPH) {
+                                const float ir = e2 > 0.f ? rsqrtf(e2) : 0.f;  // grad W(0) = 0
+                                const float r = e2 * ir;
+                                const float gi = spline_third_dw(sat_fma1(r, pi.w), r * pi.w);
+                                const float gj = spline_third_dw(sat_fma1(r, pj.w), r * pj.w);
+                                if ((gi != 0.f || gj != 0.f) && e2 > 0.f) {
+                                    const float b = ((gi != 0.f ? iv.x * gi : 0.f) + (gj != 0.f ? C[0] * gj : 0.f)) * ir;
+                                    fi = C[2] * b;
+                                    fj = iv.y * b;
+                                }
+                            } else {
+                                const float d2 = pair_d2<PER>(pi, pj, box);
+                                const bool self = NO_SELF && (s * kSC + k) * M + II == Je * MJ + g + tt * G + h * HJ;
+                                const bool ini = d2 < pi.w && !self;
+                                const bool inj = HL && d2 < pj.w && !self;
+                                if constexpr (KIND == PASS_COUNT) {
+                                    ac += ini ? 1u : 0u;
+                                    if (inj) *js = __uint_as_float(__float_as_uint(*js) + 1u);
+                                } else if constexpr (KIND == PASS_MIN) {
+                                    if (ini) ac = min(ac, __float_as_uint(e2));
+                                    if (inj) *js = fminf(*js, e2);
+                                } else if (ini || inj) {
+                                    float f;
+                                    if constexpr (KIND == PASS_LJ) {
+                                        const float s2 = sig2 * (1.f / e2);
+                                        const float s6 = s2 * s2 * s2;
+                                        f = -(s2 * (s6 * (2.f * s6 - 1.f)));
+                                    } else {
+                                        const float ir = rsqrtf(e2);
+                                        const float ir2 = ir * ir;
+                                        const float s2 = sig2 * ir2;
+                                        const float s6 = s2 * s2 * s2;
+                                        f = -(ir2 * (e24 * (s6 * (2.f * s6 - 1.f)) + iv.x * C[0] * ir));
+                                    }
+                                    if (ini) fi = f;
+                                    if (inj) fj = f;
+                                }
+                            }
+                            if constexpr (FORCE) {
+                                if (fi != 0.f) {
+                                    ax = add2_rn(ax, pk2(fi * dv.x, 0.f));
+                                    ay = add2_rn(ay, pk2(fi * dv.y, 0.f));
+                                    az = add2_rn(az, pk2(fi * dv.z, 0.f));
+                                }
+                                if constexpr (HL) {
+                                    if (fj != 0.f) {
+                                        js[0] += fj * dv.x;
+                                        js[JS] += fj * dv.y;
+                                        js[2 * JS] += fj * dv.z;
+                                    }
+                                }
+                            }
+                        }
+                    }
+                    // over the lanes of the same i particle, then to the lane
+                    // that keeps its running sum
+                    const bool mine = k / NK == g;
+                    if constexpr (INTS) {
+#pragma unroll
+                        for (int o = M; o < 32; o <<= 1) ac = merge(ac, __shfl_xor_sync(0xffffffffu, ac, o));
+#pragma unroll
+                        for (uint32_t q = 0; q < NK; ++q)
+                            if (mine && k % NK == q) rc[q] = merge(rc[q], ac);
+                    } else {
+                        float x0, x1, y0, y1, z0, z1;
+                        unpk2(ax, x0, x1);
+                        unpk2(ay, y0, y1);
+                        unpk2(az, z0, z1);
+                        float x = x0 + x1, y = y0 + y1, z = z0 + z1;
+#pragma unroll
+                        for (int o = M; o < 32; o <<= 1) {
+                            x += __shfl_xor_sync(0xffffffffu, x, o);
+                            if constexpr (FORCE) {
+                                y += __shfl_xor_sync(0xffffffffu, y, o);
+                                z += __shfl_xor_sync(0xffffffffu, z, o);
+                            }
+                        }
+#pragma unroll
+                        for (uint32_t q = 0; q < NK; ++q)
+                            if (mine && k % NK == q) {
+                                if constexpr (KIND == PASS_DENSITY) {
+                                    sum_add(rx[q], cx[q], x);
+                                } else {
+                                    sum_add(rx[q], cx[q], x);
+                                    sum_add(ry[q], cy[q], y);
+                                    sum_add(rz[q], cz[q], z);
+                                }
+                            }
+                    }
+                }
+
+                if constexpr (HL) {
+                    // the j shares over the M lanes of their i particles (in a fixed
+                    // order), then one add per j particle: one task (entry, pair) per
+                    // lane; 16-byte reads in an order that spreads over the banks
+                    __syncwarp();
+                    static_assert(SE * NT * G <= 32, "a task per lane");
+                    const uint32_t el = lane / (NT * G), tg = lane % (NT * G);
+                    const uint32_t Je = __shfl_sync(0xffffffffu, J, min(c + el, 31u));
+                    if (el < ns && ((feeds >> ((c + el) & 31u)) & 1u)) {
+                        const uint32_t tt = tg / G, gg = tg % G;
+                        const uint32_t j0 = Je * MJ + gg + tt * G;
+                        const uint4 *src = reinterpret_cast<const uint4 *>(S.js + (el * NT + tt) * 32 + gg * M);
+                        constexpr uint32_t CH = M / 2, JS = SE * NT * 16;
+#pragma unroll
+                        for (int comp = 0; comp < Smem::NC; ++comp) {
+                            f32x2 v = KIND == PASS_MIN ? pk2(INFINITY, INFINITY) : 0ull;
+#pragma unroll
+                            for (uint32_t ch = 0; ch < CH; ++ch) {
+                                const uint4 w = src[comp * JS + (ch ^ ((lane >> 1) & (CH - 1u)))];
+                                const f32x2 w0 = ((f32x2)w.y << 32) | w.x, w1 = ((f32x2)w.w << 32) | w.z;
+                                if constexpr (INTS) {
+                                    const uint32_t l = merge(merge((uint32_t)v, w.x), w.z);
+                                    const uint32_t h = merge(merge((uint32_t)(v >> 32), w.y), w.w);
+                                    v = ((f32x2)h << 32) | l;
+                                } else {
+                                    v = add2_rn(v, add2_rn(w0, w1));
+                                }
+                            }
+                            float v0, v1;
+                            unpk2(v, v0, v1);
+                            if constexpr (KIND == PASS_DENSITY) {  // units of w/2
+                                if (v0 > 0.f) atomicAdd(&a.hsum[j0], fixed_of_nonneg(__fmul_rn(v0, hscale) * 2.f));
+                                if (v1 > 0.f) atomicAdd(&a.hsum[j0 + HJ], fixed_of_nonneg(__fmul_rn(v1, hscale) * 2.f));
+                            } else if constexpr (KIND == PASS_COUNT) {
+                                if (__float_as_uint(v0)) atomicAdd(&a.hcnt[j0], __float_as_uint(v0));
+                                if (__float_as_uint(v1)) atomicAdd(&a.hcnt[j0 + HJ], __float_as_uint(v1));
+                            } else if constexpr (KIND == PASS_MIN) {
+                                // (bits of non-negative floats: an integer minimum)
+                                if (v0 < INFINITY) atomicMin(&a.hcnt[j0], __float_as_uint(v0));
+                                if (v1 < INFINITY) atomicMin(&a.hcnt[j0 + HJ], __float_as_uint(v1));
+                            } else {
+                                // FP64 adds: their order changes the sum by about
+                                // 1e-16 of it, below the FP32 rounding of the output
+                                if (v0 != 0.f) atomicAdd(&a.hf[3 * (size_t)j0 + comp], f64_of(-v0));
+                                if (v1 != 0.f) atomicAdd(&a.hf[3 * (size_t)(j0 + HJ) + comp], f64_of(-v1));
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        if constexpr (INTS) {
+#pragma unroll
+            for (uint32_t q = 0; q < NK; ++q) rx[q] = __uint_as_float(rc[q]);
+        }
+
+        // warps sharing the super-cluster: the first adds the others' sums, in
+        // a fixed order (half lists add their sums to memory anyway)
+        if (!HL && W != 1u) {
+            float *mine = reinterpret_cast<float *>(S.js);
+            __syncwarp();
+#pragma unroll
+            for (uint32_t q = 0; q < NK; ++q) {
+                mine[q * 32 + lane] = INTS ? rx[q] : __fsub_rn(rx[q], cx[q]);
+                if constexpr (FORCE) {
+                    mine[(NK + q) * 32 + lane] = __fsub_rn(ry[q], cy[q]);
+                    mine[(2 * NK + q) * 32 + lane] = __fsub_rn(rz[q], cz[q]);
+                }
+            }
+            asm volatile("bar.sync %0, %1;" ::"r"(1u + grp), "r"(W * 32u) : "memory");
+            if (wig == 0) {
+                for (uint32_t w = 1; w < W; ++w) {
+                    const float *o = reinterpret_cast<const float *>(all[warp + w].js);
+#pragma unroll
+                    for (uint32_t q = 0; q < NK; ++q) {
+                        const float v = o[q * 32 + lane];
+                        if constexpr (INTS) rx[q] = __uint_as_float(merge(__float_as_uint(rx[q]), __float_as_uint(v)));
+                        else sum_add(rx[q], cx[q], v);
+                        if constexpr (FORCE) {
+                            sum_add(ry[q], cy[q], o[(NK + q) * 32 + lane]);
+                            sum_add(rz[q], cz[q], o[(2 * NK + q) * 32 + lane]);
+                        }
+                    }
+                }
+            }
+            asm volatile("bar.sync %0, %1;" ::"r"(1u + grp), "r"(W * 32u) : "memory");
+            if (wig != 0) continue;
+        }
+
+        // write in caller order
+#pragma unroll
+        for (uint32_t q = 0; q < NK; ++q) {
+            if constexpr (KIND == PASS_DENSITY || KIND == PASS_SPH) {
+                rx[q] = __fsub_rn(rx[q], cx[q]);
+                ry[q] = __fsub_rn(ry[q], cy[q]);
+                rz[q] = __fsub_rn(rz[q], cz[q]);
+            }
+            const uint32_t k = g * NK + q;
+            const uint32_t i = (s * kSC + k) * M + II;
+            const uint32_t pc = a.perm[i];
+            if (pc == 0xffffffffu) continue;  // dummy slot
+            const uint32_t o = a.sorted_out ? i : pc;
+            // the loop took i = j iff its entry was listed and the range is
+            // nonzero (density: -1/(2h) is finite then)
+            const float av = S.ia[k * M + II].w;
+            const bool seen = (selfseen >> (k * RJ + II / MJ)) & 1u;
+            const bool took_self = seen && (KIND == PASS_DENSITY ? isfinite(av) : av > 0.f);
+            if constexpr (KIND == PASS_DENSITY) {
+                float v = 2.f * rx[q];  // sums are in units of w/2
+                if (wig == 0 && !took_self) v += a.aux[i].x;  // m_i w(0) = m_i
+                if constexpr (HL) {
+                    atomicAdd(&a.hsum[i], fixed_of(v * hscale));
+                } else {
+                    const float hk = 1.f / a.pos[i].w;
+                    a.out0[o] = v * (0.318309886183790672f * hk * hk * hk);
+                }
+            } else if constexpr (KIND == PASS_COUNT) {
+                const uint32_t v = __float_as_uint(rx[q]) - (wig == 0 && took_self ? 1u : 0u);
+                if constexpr (HL) atomicAdd(&a.hcnt[i], v);
+                else a.outc[o] = v;
+            } else if constexpr (KIND == PASS_MIN) {
+                if constexpr (HL) {
+                    if (rx[q] < INFINITY) atomicMin(&a.hcnt[i], __float_as_uint(rx[q]));
+                } else {
+                    a.out0[o] = sqrtf(rx[q]);  // +inf without a neighbor
+                }
+            } else if constexpr (HL) {
+                atomicAdd(&a.hf[3 * (size_t)i + 0], f64_of(rx[q]));
+                atomicAdd(&a.hf[3 * (size_t)i + 1], f64_of(ry[q]));
+                atomicAdd(&a.hf[3 * (size_t)i + 2], f64_of(rz[q]));
+            } else if constexpr (KIND == PASS_LJ) {
+                a.out0[o] = (float)((double)rx[q] * fscale);
+                a.out1[o] = (float)((double)ry[q] * fscale);
+                a.out2[o] = (float)((double)rz[q] * fscale);
+            } else {
+                a.out0[o] = rx[q];
+                a.out1[o] = ry[q];
+                a.out2[o] = rz[q];
+            }
+        }
+    }
+}
+
+template <int M, int MJ, int KIND, bool HL>
+static cudaError_t launch_packed_mk(const PassArgs &a, int per, int grid, int threads, cudaStream_t s)
+{
+    const size_t smem = (size_t)(threads / 32) * sizeof(PkSmem<M, MJ, KIND, HL>);
+    const void *fn = per ? (const void *)k_pass_packed<M, MJ, true, KIND, HL>
+                         : (const void *)k_pass_packed<M, MJ, false, KIND, HL>;
+    cudaError_t e = set_max_dynamic_smem(fn, (size_t)(PK_THREADS / 32) * sizeof(PkSmem<M, MJ, KIND, HL>));
+    if (e != cudaSuccess) return e;
+    if (per)
+        k_pass_packed<M, MJ, true, KIND, HL><<<grid, threads, smem, s>>>(a);
+    else
+        k_pass_packed<M, MJ, false, KIND, HL><<<grid, threads, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int KIND>
+static cudaError_t launch_packed(const PassArgs &a, int M, int per, int grid, int threads, cudaStream_t s)
+{
+    if (threads != 128 && threads != PK_THREADS) return cudaErrorInvalidValue;
+    if (a.split != 1 && a.split != 2 && a.split != 4 && (a.split != 8 || threads != 256)) return cudaErrorInvalidValue;
+    switch (M * 100 + a.mj) {
+    case 808:
+        return a.half ? launch_packed_mk<8, 8, KIND, true>(a, per, grid, threads, s)
+                      : launch_packed_mk<8, 8, KIND, false>(a, per, grid, threads, s);
+    case 1616:
+        return a.half ? launch_packed_mk<16, 16, KIND, true>(a, per, grid, threads, s)
+                      : launch_packed_mk<16, 16, KIND, false>(a, per, grid, threads, s);
+    case 1608:
+        return a.half ? cudaErrorInvalidValue : launch_packed_mk<16, 8, KIND, false>(a, per, grid, threads, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace nlg
