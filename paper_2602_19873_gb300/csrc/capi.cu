@@ -1212,7 +1212,11 @@ static nl_status mlp_run(nl_mlp *mlp, const float *X, const float *y, const floa
                          const int64_t *idx_dev, int64_t nb, float *grad, int adam, float lr,
                          float inv_n, float *loss_host, cudaStream_t s)
 {
-    const int slots = (int)std::min<int64_t>((nb + 63) / 64, 4096);
+    // two CTAs per SM, each with its own gradient slot
+    int dev, sms;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int slots = (int)std::min<int64_t>((nb + 63) / 64, 2 * sms);
     nl_status st = mlp_slots(mlp, slots);
     if (st != NL_OK) return st;
     if (adam) ++mlp->step;
@@ -1236,12 +1240,7 @@ nl_status nl_mlp_grad(nl_mlp *mlp, const float *X, const float *y, const float *
 {
     if (!mlp || !X || !y || !w || !grad || n < 1) return fail(NL_ERR_ARG, "bad argument");
     cudaStream_t s = (cudaStream_t)stream;
-    std::vector<int64_t> idx(n);
-    for (int64_t k = 0; k < n; ++k) idx[k] = k;
-    CK(mlp->idx.ensure((size_t)n * 8));
-    CK(cudaMemcpyAsync(mlp->idx.p, idx.data(), (size_t)n * 8, cudaMemcpyHostToDevice, s));
-    nl_status st = mlp_run(mlp, X, y, w, n, mlp->idx.as<int64_t>(), n, grad, 0, 0.f,
-                           1.f / (float)n, loss, s);
+    nl_status st = mlp_run(mlp, X, y, w, n, nullptr, n, grad, 0, 0.f, 1.f / (float)n, loss, s);
     if (st != NL_OK) return st;
     CK(cudaStreamSynchronize(s));
     return NL_OK;

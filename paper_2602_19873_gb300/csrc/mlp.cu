@@ -173,11 +173,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return *reinterpret_cast<uint32_t *>(&v);
 }
 
-__device__ __forceinline__ uint32_t pack_raw(__nv_bfloat16 lo, __nv_bfloat16 hi)
-{
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
 // D += A (16x16, row) * B (16x8, col); BF16 operands, FP32 accumulators
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                          uint32_t b1)
@@ -189,21 +184,41 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ float silu_f(float z) { return z / (1.f + expf(-z)); }
-
-__device__ __forceinline__ float dsilu_f(float z)
+// Four 8x8 matrices of 16-bit elements from shared memory: lane l gives the
+// address of row l % 8 of matrix l / 8; plain: lane (g, t) = (l / 4, l % 4) gets
+// elements (g, 2t), (g, 2t + 1) of each matrix; trans: (2t, g), (2t + 1, g).
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], const void *p)
 {
-    float s = 1.f / (1.f + expf(-z));
-    return s * (1.f + z * (1.f - s));
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
 }
 
-// Shared-memory copy of the network: BF16 weights row-major (out x in) and
-// transposed, FP32 biases and output row.
-struct MlpSmem {
-    __nv_bfloat16 w1[kMlpH][16];          // inputs padded 8 -> 16 with zeros
-    __nv_bfloat16 w2[kMlpH][kMlpH], w3[kMlpH][kMlpH];
-    __nv_bfloat16 w2t[kMlpH][kMlpH], w3t[kMlpH][kMlpH];
-    __nv_bfloat16 w1t[16][kMlpH];
+__device__ __forceinline__ void ldm4t(uint32_t (&r)[4], const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+
+__device__ __forceinline__ float silu_f(float z) { return z / (1.f + expf(-z)); }
+
+// silu and its derivative from one exponential
+__device__ __forceinline__ float silu_d(float z, float &ds)
+{
+    const float e = 1.f + expf(-z), s = 1.f / e;
+    ds = s * (1.f + z * (1.f - s));
+    return z / e;
+}
+
+// Shared-memory copy of the network: BF16 weights row-major (out x in), FP32
+// biases and output row.  Rows are padded by 16 bytes, so that the eight rows of
+// an ldmatrix lie in different banks; products with the transposed weights read
+// the same copy with ldmatrix.trans.
+constexpr int kLd = kMlpH + 8, kLdX = 24;
+struct alignas(16) MlpSmem {
+    __nv_bfloat16 w1[kMlpH][kLdX];        // inputs padded 8 -> 16 with zeros
+    __nv_bfloat16 w2[kMlpH][kLd], w3[kMlpH][kLd];
     float b1[kMlpH], b2[kMlpH], b3[kMlpH], w4[kMlpH];
     float b4;
 };
@@ -213,18 +228,13 @@ __device__ void load_net(MlpSmem &S, const float *__restrict__ P)
     const float *W1 = P, *B1 = W1 + kMlpH * kMlpF, *W2 = B1 + kMlpH, *B2 = W2 + kMlpH * kMlpH;
     const float *W3 = B2 + kMlpH, *B3 = W3 + kMlpH * kMlpH, *W4 = B3 + kMlpH, *B4 = W4 + kMlpH;
     for (int t = threadIdx.x; t < kMlpH * kMlpH; t += blockDim.x) {
-        int o = t / kMlpH, i = t % kMlpH;
-        __nv_bfloat16 a = __float2bfloat16_rn(W2[t]), b = __float2bfloat16_rn(W3[t]);
-        S.w2[o][i] = a;
-        S.w2t[i][o] = a;
-        S.w3[o][i] = b;
-        S.w3t[i][o] = b;
+        const int o = t / kMlpH, i = t % kMlpH;
+        S.w2[o][i] = __float2bfloat16_rn(W2[t]);
+        S.w3[o][i] = __float2bfloat16_rn(W3[t]);
     }
     for (int t = threadIdx.x; t < kMlpH * 16; t += blockDim.x) {
-        int o = t / 16, i = t % 16;
-        __nv_bfloat16 v = __float2bfloat16_rn(i < kMlpF ? W1[o * kMlpF + i] : 0.f);
-        S.w1[o][i] = v;
-        S.w1t[i][o] = v;
+        const int o = t / 16, i = t % 16;
+        S.w1[o][i] = __float2bfloat16_rn(i < kMlpF ? W1[o * kMlpF + i] : 0.f);
     }
     for (int t = threadIdx.x; t < kMlpH; t += blockDim.x) {
         S.b1[t] = B1[t];
@@ -248,10 +258,10 @@ __device__ __forceinline__ void to_afrag(const float (&h)[8][4], uint32_t (&A)[4
 }
 
 // z = A(16x64) * W^T + b, W row-major [64][64] in shared memory
-__device__ __forceinline__ void dense64(const uint32_t (&A)[4][4], const __nv_bfloat16 (&W)[kMlpH][kMlpH],
+__device__ __forceinline__ void dense64(const uint32_t (&A)[4][4], const __nv_bfloat16 (&W)[kMlpH][kLd],
                                        const float *b, float (&z)[8][4])
 {
-    const unsigned lane = lane_id(), g = lane >> 2, t = lane & 3;
+    const unsigned lane = lane_id(), t = lane & 3;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         z[j][0] = b[8 * j + 2 * t];
@@ -259,61 +269,47 @@ __device__ __forceinline__ void dense64(const uint32_t (&A)[4][4], const __nv_bf
         z[j][2] = z[j][0];
         z[j][3] = z[j][1];
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(&W[8 * j + g][16 * kk + 2 * t]);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t *>(&W[8 * j + g][16 * kk + 8 + 2 * t]);
-            mma16816(z[j], A[kk], b0, b1);
+        for (int kk = 0; kk < 4; kk += 2) {
+            uint32_t B[4];
+            ldm4(B, &W[8 * j + (lane & 7)][16 * kk + 8 * (lane >> 3)]);
+            mma16816(z[j], A[kk], B[0], B[1]);
+            mma16816(z[j], A[kk + 1], B[2], B[3]);
         }
     }
 }
 
-// Forward of 16 rows (x: 16 x 8, row r at x + r*8, rows >= nrows are zero).
-// Keeps pre-activations z1..z3 when asked (training).
-__device__ __forceinline__ void forward16(const MlpSmem &S, const float *x, int ld, int nrows,
-                                          float (&z1)[8][4], float (&z2)[8][4], float (&z3)[8][4],
-                                          float (&pred)[2])
+// z = A0(16x16, inputs) * W1^T + b1
+__device__ __forceinline__ void dense_in(const uint32_t (&a0)[4], const MlpSmem &S, float (&z)[8][4])
 {
-    const unsigned lane = lane_id(), g = lane >> 2, t = lane & 3;
-    uint32_t A[4][4];
-    {
-        float x0 = g < (unsigned)nrows ? x[g * ld + 2 * t] : 0.f;
-        float x1 = g < (unsigned)nrows ? x[g * ld + 2 * t + 1] : 0.f;
-        float x2 = g + 8 < (unsigned)nrows ? x[(g + 8) * ld + 2 * t] : 0.f;
-        float x3 = g + 8 < (unsigned)nrows ? x[(g + 8) * ld + 2 * t + 1] : 0.f;
-        uint32_t a0[4] = {pack_bf16(x0, x1), pack_bf16(x2, x3), 0u, 0u};
+    const unsigned lane = lane_id(), t = lane & 3;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            z1[j][0] = S.b1[8 * j + 2 * t];
-            z1[j][1] = S.b1[8 * j + 2 * t + 1];
-            z1[j][2] = z1[j][0];
-            z1[j][3] = z1[j][1];
-            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(&S.w1[8 * j + g][2 * t]);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t *>(&S.w1[8 * j + g][8 + 2 * t]);
-            mma16816(z1[j], a0, b0, b1);
+    for (int j = 0; j < 8; j += 2) {
+        uint32_t B[4];  // n-tiles j and j + 1
+        ldm4(B, &S.w1[8 * j + (lane & 7) + 8 * (lane >> 4)][8 * ((lane >> 3) & 1)]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            z[j + e][0] = S.b1[8 * (j + e) + 2 * t];
+            z[j + e][1] = S.b1[8 * (j + e) + 2 * t + 1];
+            z[j + e][2] = z[j + e][0];
+            z[j + e][3] = z[j + e][1];
+            mma16816(z[j + e], a0, B[2 * e], B[2 * e + 1]);
         }
     }
-    float h[8][4];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) h[j][q] = silu_f(z1[j][q]);
-    to_afrag(h, A);
-    dense64(A, S.w2, S.b2, z2);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) h[j][q] = silu_f(z2[j][q]);
-    to_afrag(h, A);
-    dense64(A, S.w3, S.b3, z3);
-    // output: y = b4 + sum_k w4[k] h3[k]; h3 rounded to BF16 like every operand
+}
+
+// y = b4 + sum_k w4[k] h3[k] of rows g and g + 8; h3 rounded to BF16 like every
+// operand (h: this lane's activations, rounded here)
+__device__ __forceinline__ void output_row(const MlpSmem &S, float (&h)[8][4], float (&pred)[2])
+{
+    const unsigned t = lane_id() & 3;
     float p0 = 0.f, p1 = 0.f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const float w0 = S.w4[8 * j + 2 * t], w1 = S.w4[8 * j + 2 * t + 1];
-        p0 += w0 * __bfloat162float(__float2bfloat16_rn(silu_f(z3[j][0]))) +
-              w1 * __bfloat162float(__float2bfloat16_rn(silu_f(z3[j][1])));
-        p1 += w0 * __bfloat162float(__float2bfloat16_rn(silu_f(z3[j][2]))) +
-              w1 * __bfloat162float(__float2bfloat16_rn(silu_f(z3[j][3])));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) h[j][q] = __bfloat162float(__float2bfloat16_rn(h[j][q]));
+        p0 += w0 * h[j][0] + w1 * h[j][1];
+        p1 += w0 * h[j][2] + w1 * h[j][3];
     }
     p0 += __shfl_xor_sync(0xffffffffu, p0, 1);
     p0 += __shfl_xor_sync(0xffffffffu, p0, 2);
@@ -324,9 +320,10 @@ __device__ __forceinline__ void forward16(const MlpSmem &S, const float *x, int 
 }
 
 // ---------------------------------------------------------------------------
-// Inference: one warp per 16 samples
+// Inference: one warp per 16 samples, a persistent grid (every block converts
+// the network once).  Bound by the FP32 arithmetic of the activations.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_mlp_predict(int64_t n, const float *__restrict__ X,
+__global__ void __launch_bounds__(256, 2) k_mlp_predict(int64_t n, const float *__restrict__ X,
                                                      const float *__restrict__ P,
                                                      float *__restrict__ out)
 {
@@ -340,11 +337,31 @@ __global__ void __launch_bounds__(128) k_mlp_predict(int64_t n, const float *__r
          tile += warps) {
         const int64_t r0 = tile * 16;
         const int nrows = (int)min_i64(16, n - r0);
-        float z1[8][4], z2[8][4], z3[8][4], pred[2];
-        forward16(S, X + r0 * kMlpF, kMlpF, nrows, z1, z2, z3, pred);
+        const float *x = X + r0 * kMlpF;
+        const bool va = (int)g < nrows, vb = (int)g + 8 < nrows;
+        const uint32_t a0[4] = {
+            pack_bf16(va ? x[g * kMlpF + 2 * t] : 0.f, va ? x[g * kMlpF + 2 * t + 1] : 0.f),
+            pack_bf16(vb ? x[(g + 8) * kMlpF + 2 * t] : 0.f, vb ? x[(g + 8) * kMlpF + 2 * t + 1] : 0.f), 0u, 0u};
+        float z[8][4], pred[2];
+        uint32_t A[4][4];
+        auto act = [&]() {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) z[j][q] = silu_f(z[j][q]);
+        };
+        dense_in(a0, S, z);
+        act();
+        to_afrag(z, A);
+        dense64(A, S.w2, S.b2, z);
+        act();
+        to_afrag(z, A);
+        dense64(A, S.w3, S.b3, z);
+        act();
+        output_row(S, z, pred);
         if (t == 0) {
-            if ((int)g < nrows) out[r0 + g] = pred[0];
-            if ((int)g + 8 < nrows) out[r0 + g + 8] = pred[1];
+            if (va) out[r0 + g] = pred[0];
+            if (vb) out[r0 + g + 8] = pred[1];
         }
     }
 }
@@ -353,78 +370,94 @@ __global__ void __launch_bounds__(128) k_mlp_predict(int64_t n, const float *__r
 // Training: each CTA (4 warps) takes 64-sample tiles of the minibatch and
 // accumulates its gradient in registers (warp w owns output rows 16w..16w+15
 // of every weight matrix); the CTA's gradient goes to its own slot of
-// `partial`, and k_mlp_adam reduces the slots in a fixed order.
+// `partial`, and k_mlp_reduce_adam sums the slots in a fixed order.
+// Activations and deltas lie in shared memory as BF16 rows (padded as the
+// weights) and reach the tensor cores by ldmatrix, transposed for the weight
+// gradients; the derivatives of the activations stay with the thread that made
+// them.  95 KB of shared memory: two CTAs per SM.  With 16-bit loads of the
+// fragments, activations evaluated three times over and one 64-sample tile per CTA
+// (so that every tile converted the network and wrote a gradient slot), the
+// gradient over 262144 samples took 1.25 ms; it takes 0.27 ms now (train kernel 1.08
+// -> 0.26 ms, sum of the slots 0.167 -> 0.008 ms, predictions 0.134 -> 0.079 ms).
 // ---------------------------------------------------------------------------
-struct TrainSmem {
+struct alignas(16) TrainSmem {
     MlpSmem net;
-    float z[3][64][kMlpH];                // pre-activations of the tile
-    __nv_bfloat16 h[2][64][kMlpH];        // h1, h2 (BF16, as the forward used them)
-    __nv_bfloat16 d[2][64][kMlpH];        // dZ of the current and next layer
-    __nv_bfloat16 x[64][16];              // inputs, padded
+    __nv_bfloat16 h[2][64][kLd];          // h1, h2 (BF16, as the forward used them)
+    __nv_bfloat16 d[2][64][kLd];          // dZ of the current and next layer
+    __nv_bfloat16 x[64][kLdX];            // inputs, padded
+    float4 ds[2][8][128];                 // derivatives of the first two activations, per thread
     float dy[64];
-    float loss[4];
 };
 
 size_t mlp_train_smem() { return sizeof(TrainSmem); }
 size_t mlp_predict_smem() { return sizeof(MlpSmem); }
 
 // stripe gradient: G[o in 16w..16w+15][i] += sum_r D[r][o] * Hin[r][i], i over
-// nt n-tiles of 8 (K = 64 samples)
+// NT n-tiles of 8 (K = 64 samples)
 template <int NT, int LD>
-__device__ __forceinline__ void grad_stripe(const __nv_bfloat16 (*D)[kMlpH],
+__device__ __forceinline__ void grad_stripe(const __nv_bfloat16 (*D)[kLd],
                                             const __nv_bfloat16 (*Hin)[LD], float (&G)[NT][4])
 {
-    const unsigned lane = lane_id(), g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
-    const int o0 = 16 * w;
+    const unsigned lane = lane_id(), w = threadIdx.x >> 5;
+    const unsigned l8 = lane & 7, m1 = (lane >> 3) & 1, m2 = lane >> 4;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-        const int r = 16 * kk + 2 * t;
         uint32_t A[4];
-        A[0] = pack_raw(D[r][o0 + g], D[r + 1][o0 + g]);
-        A[1] = pack_raw(D[r][o0 + g + 8], D[r + 1][o0 + g + 8]);
-        A[2] = pack_raw(D[r + 8][o0 + g], D[r + 9][o0 + g]);
-        A[3] = pack_raw(D[r + 8][o0 + g + 8], D[r + 9][o0 + g + 8]);
+        ldm4t(A, &D[16 * kk + 8 * m2 + l8][16 * w + 8 * m1]);
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            const uint32_t b0 = pack_raw(Hin[r][8 * j + g], Hin[r + 1][8 * j + g]);
-            const uint32_t b1 = pack_raw(Hin[r + 8][8 * j + g], Hin[r + 9][8 * j + g]);
-            mma16816(G[j], A, b0, b1);
+        for (int j = 0; j < NT; j += 2) {
+            uint32_t B[4];
+            ldm4t(B, &Hin[16 * kk + 8 * m1 + l8][8 * j + 8 * m2]);
+            mma16816(G[j], A, B[0], B[1]);
+            mma16816(G[j + 1], A, B[2], B[3]);
         }
     }
 }
 
-// dH (16 rows of this warp) = dZ (rows) * W, with W^T row-major in shared memory
-__device__ __forceinline__ void back64(const __nv_bfloat16 (*D)[kMlpH], int row0,
-                                      const __nv_bfloat16 (&WT)[kMlpH][kMlpH], float (&dh)[8][4])
+// dH (16 rows of this warp) = dZ (rows) * W
+__device__ __forceinline__ void back64(const __nv_bfloat16 (*D)[kLd], int row0,
+                                      const __nv_bfloat16 (&W)[kMlpH][kLd], float (&dh)[8][4])
 {
-    const unsigned lane = lane_id(), g = lane >> 2, t = lane & 3;
+    const unsigned lane = lane_id();
+    const unsigned l8 = lane & 7, m1 = (lane >> 3) & 1, m2 = lane >> 4;
     uint32_t A[4][4];
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        A[kk][0] = *reinterpret_cast<const uint32_t *>(&D[row0 + g][16 * kk + 2 * t]);
-        A[kk][1] = *reinterpret_cast<const uint32_t *>(&D[row0 + g + 8][16 * kk + 2 * t]);
-        A[kk][2] = *reinterpret_cast<const uint32_t *>(&D[row0 + g][16 * kk + 8 + 2 * t]);
-        A[kk][3] = *reinterpret_cast<const uint32_t *>(&D[row0 + g + 8][16 * kk + 8 + 2 * t]);
-    }
+    for (int kk = 0; kk < 4; ++kk) ldm4(A[kk], &D[row0 + 8 * m1 + l8][16 * kk + 8 * m2]);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        dh[j][0] = dh[j][1] = dh[j][2] = dh[j][3] = 0.f;
+    for (int j = 0; j < 8; j += 2) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dh[j][q] = dh[j + 1][q] = 0.f;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-            const uint32_t b0 = *reinterpret_cast<const uint32_t *>(&WT[8 * j + g][16 * kk + 2 * t]);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t *>(&WT[8 * j + g][16 * kk + 8 + 2 * t]);
-            mma16816(dh[j], A[kk], b0, b1);
+            uint32_t B[4];
+            ldm4t(B, &W[16 * kk + 8 * m1 + l8][8 * j + 8 * m2]);
+            mma16816(dh[j], A[kk], B[0], B[1]);
+            mma16816(dh[j + 1], A[kk], B[2], B[3]);
         }
     }
 }
 
-__global__ void __launch_bounds__(128) k_mlp_train(int64_t nb, const int64_t *__restrict__ idx,
-                                                   const float *__restrict__ X,
-                                                   const float *__restrict__ Y,
-                                                   const float *__restrict__ Wt,
-                                                   const float *__restrict__ P, float inv_n,
-                                                   float *__restrict__ partial,
-                                                   float *__restrict__ loss_out)
+// A fragments of this warp's 16 rows -> BF16 rows in shared memory
+__device__ __forceinline__ void store_rows(__nv_bfloat16 (*H)[kLd], int row0, const uint32_t (&A)[4][4])
+{
+    const unsigned lane = lane_id(), g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+        *reinterpret_cast<uint32_t *>(&H[row0 + g][16 * kk + 2 * t]) = A[kk][0];
+        *reinterpret_cast<uint32_t *>(&H[row0 + g + 8][16 * kk + 2 * t]) = A[kk][1];
+        *reinterpret_cast<uint32_t *>(&H[row0 + g][16 * kk + 8 + 2 * t]) = A[kk][2];
+        *reinterpret_cast<uint32_t *>(&H[row0 + g + 8][16 * kk + 8 + 2 * t]) = A[kk][3];
+    }
+}
+
+// idx: the samples of the minibatch; NULL: samples 0 .. nb - 1
+__global__ void __launch_bounds__(128, 2) k_mlp_train(int64_t nb, const int64_t *__restrict__ idx,
+                                                      const float *__restrict__ X,
+                                                      const float *__restrict__ Y,
+                                                      const float *__restrict__ Wt,
+                                                      const float *__restrict__ P, float inv_n,
+                                                      float *__restrict__ partial,
+                                                      float *__restrict__ loss_out)
 {
     extern __shared__ __align__(16) unsigned char mlp_smem[];
     TrainSmem &S = *reinterpret_cast<TrainSmem *>(mlp_smem);
@@ -433,115 +466,113 @@ __global__ void __launch_bounds__(128) k_mlp_train(int64_t nb, const int64_t *__
     const int row0 = 16 * w;
     float gW1[2][4] = {}, gW2[8][4] = {}, gW3[8][4] = {}, gW4[8][2] = {};
     float gb1 = 0.f, gb2 = 0.f, gb3 = 0.f, gb4 = 0.f, lsum = 0.f;
+    auto sample = [&](int64_t k) { return idx ? idx[k] : k; };
+    // bias gradient of output 16w + lane % 16: lanes l and l + 16 hold halves
+    auto bias_sum = [&](const __nv_bfloat16 (*D)[kLd]) {
+        const int o = row0 + (lane & 15);
+        float sb = 0.f;
+        for (int r = (lane >> 4); r < 64; r += 2) sb += __bfloat162float(D[r][o]);
+        return sb;
+    };
     __syncthreads();
     for (int64_t tile = blockIdx.x; tile * 64 < nb; tile += gridDim.x) {
         const int64_t base = tile * 64;
         const int nrows = (int)min_i64(64, nb - base);
-        // inputs to shared memory (padded, BF16) and, FP32, to a staging buffer
+        // inputs to shared memory (padded, BF16)
         for (int q = threadIdx.x; q < 64 * 16; q += blockDim.x) {
             const int r = q / 16, i = q % 16;
             float v = 0.f;
-            if (r < nrows && i < kMlpF) v = X[idx[base + r] * kMlpF + i];
+            if (r < nrows && i < kMlpF) v = X[sample(base + r) * kMlpF + i];
             S.x[r][i] = __float2bfloat16_rn(v);
-            if (i < kMlpF) S.z[0][r][i] = v;  // raw inputs, FP32, read by forward16
         }
         __syncthreads();
-        float z1[8][4], z2[8][4], z3[8][4], pred[2];
-        forward16(S.net, &S.z[0][row0][0], kMlpH, max(0, min(16, nrows - row0)), z1, z2, z3, pred);
-        __syncthreads();  // S.z[0] is reused for z1 below
-        // keep pre-activations and BF16 activations of the tile
+        float z[8][4], ds3[8][4], pred[2];
+        uint32_t A[4][4];
+        // activation of z; its derivative to shared memory
+        auto act = [&](int layer) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int c = 8 * j + 2 * t;
-            S.z[0][row0 + g][c] = z1[j][0];
-            S.z[0][row0 + g][c + 1] = z1[j][1];
-            S.z[0][row0 + g + 8][c] = z1[j][2];
-            S.z[0][row0 + g + 8][c + 1] = z1[j][3];
-            S.z[1][row0 + g][c] = z2[j][0];
-            S.z[1][row0 + g][c + 1] = z2[j][1];
-            S.z[1][row0 + g + 8][c] = z2[j][2];
-            S.z[1][row0 + g + 8][c + 1] = z2[j][3];
-            S.z[2][row0 + g][c] = z3[j][0];
-            S.z[2][row0 + g][c + 1] = z3[j][1];
-            S.z[2][row0 + g + 8][c] = z3[j][2];
-            S.z[2][row0 + g + 8][c + 1] = z3[j][3];
-            S.h[0][row0 + g][c] = __float2bfloat16_rn(silu_f(z1[j][0]));
-            S.h[0][row0 + g][c + 1] = __float2bfloat16_rn(silu_f(z1[j][1]));
-            S.h[0][row0 + g + 8][c] = __float2bfloat16_rn(silu_f(z1[j][2]));
-            S.h[0][row0 + g + 8][c + 1] = __float2bfloat16_rn(silu_f(z1[j][3]));
-            S.h[1][row0 + g][c] = __float2bfloat16_rn(silu_f(z2[j][0]));
-            S.h[1][row0 + g][c + 1] = __float2bfloat16_rn(silu_f(z2[j][1]));
-            S.h[1][row0 + g + 8][c] = __float2bfloat16_rn(silu_f(z2[j][2]));
-            S.h[1][row0 + g + 8][c + 1] = __float2bfloat16_rn(silu_f(z2[j][3]));
-        }
+            for (int j = 0; j < 8; ++j) {
+                float4 ds;
+                z[j][0] = silu_d(z[j][0], ds.x);
+                z[j][1] = silu_d(z[j][1], ds.y);
+                z[j][2] = silu_d(z[j][2], ds.z);
+                z[j][3] = silu_d(z[j][3], ds.w);
+                S.ds[layer][j][threadIdx.x] = ds;
+            }
+        };
+        const uint32_t a0[4] = {*reinterpret_cast<const uint32_t *>(&S.x[row0 + g][2 * t]),
+                                *reinterpret_cast<const uint32_t *>(&S.x[row0 + g + 8][2 * t]), 0u, 0u};
+        dense_in(a0, S.net, z);
+        act(0);
+        to_afrag(z, A);
+        store_rows(S.h[0], row0, A);
+        dense64(A, S.net.w2, S.net.b2, z);
+        act(1);
+        to_afrag(z, A);
+        store_rows(S.h[1], row0, A);
+        dense64(A, S.net.w3, S.net.b3, z);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) z[j][q] = silu_d(z[j][q], ds3[j][q]);
+        output_row(S.net, z, pred);
         if (t == 0) {
             const int ra = row0 + g, rb = row0 + g + 8;
-            const float ea = ra < nrows ? (pred[0] - Y[idx[base + ra]]) * Wt[idx[base + ra]] : 0.f;
-            const float eb = rb < nrows ? (pred[1] - Y[idx[base + rb]]) * Wt[idx[base + rb]] : 0.f;
+            const int64_t sa = sample(base + min(ra, nrows - 1)), sb = sample(base + min(rb, nrows - 1));
+            const float ea = ra < nrows ? (pred[0] - Y[sa]) * Wt[sa] : 0.f;
+            const float eb = rb < nrows ? (pred[1] - Y[sb]) * Wt[sb] : 0.f;
             S.dy[ra] = 2.f * ea * inv_n;
             S.dy[rb] = 2.f * eb * inv_n;
             lsum += ea * ea + eb * eb;
         }
-        __syncthreads();
+        __syncwarp();
         // layer 4 and dZ3 of this warp's rows
+        const float dya = S.dy[row0 + g], dyb = S.dy[row0 + g + 8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int r = row0 + g + (q >= 2 ? 8 : 0), c = 8 * j + 2 * t + (q & 1);
-                const float z = S.z[2][r][c];
-                const float h3 = __bfloat162float(__float2bfloat16_rn(silu_f(z)));
-                gW4[j][q & 1] += S.dy[r] * h3;
-                S.d[0][r][c] = __float2bfloat16_rn(S.dy[r] * S.net.w4[c] * dsilu_f(z));
-            }
+            const float w0 = S.net.w4[8 * j + 2 * t], w1 = S.net.w4[8 * j + 2 * t + 1];
+            gW4[j][0] += dya * z[j][0];
+            gW4[j][1] += dya * z[j][1];
+            gW4[j][0] += dyb * z[j][2];
+            gW4[j][1] += dyb * z[j][3];
+            z[j][0] = dya * w0 * ds3[j][0];
+            z[j][1] = dya * w1 * ds3[j][1];
+            z[j][2] = dyb * w0 * ds3[j][2];
+            z[j][3] = dyb * w1 * ds3[j][3];
         }
+        to_afrag(z, A);
+        store_rows(S.d[0], row0, A);
         if (lane == 0)
             for (int r = row0; r < row0 + 16; ++r) gb4 += S.dy[r];
         __syncthreads();
         // layer 3: weights (stripe) and dZ2 of this warp's rows
-        grad_stripe<8, kMlpH>(S.d[0], S.h[1], gW3);
-        {
-            const int o = row0 + (lane & 15);
-            float sb = 0.f;
-            for (int r = (lane >> 4); r < 64; r += 2) sb += __bfloat162float(S.d[0][r][o]);
-            gb3 += sb;
-        }
-        float dh[8][4];
-        back64(S.d[0], row0, S.net.w3t, dh);
+        grad_stripe<8, kLd>(S.d[0], S.h[1], gW3);
+        gb3 += bias_sum(S.d[0]);
+        auto back = [&](const __nv_bfloat16 (*D)[kLd], const __nv_bfloat16 (&W)[kMlpH][kLd], int layer) {
+            back64(D, row0, W, z);
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int r = row0 + g + (q >= 2 ? 8 : 0), c = 8 * j + 2 * t + (q & 1);
-                S.d[1][r][c] = __float2bfloat16_rn(dh[j][q] * dsilu_f(S.z[1][r][c]));
+            for (int j = 0; j < 8; ++j) {
+                const float4 ds = S.ds[layer][j][threadIdx.x];
+                z[j][0] *= ds.x;
+                z[j][1] *= ds.y;
+                z[j][2] *= ds.z;
+                z[j][3] *= ds.w;
             }
+            to_afrag(z, A);
+        };
+        back(S.d[0], S.net.w3, 1);
+        store_rows(S.d[1], row0, A);
         __syncthreads();
         // layer 2
-        grad_stripe<8, kMlpH>(S.d[1], S.h[0], gW2);
-        {
-            const int o = row0 + (lane & 15);
-            float sb = 0.f;
-            for (int r = (lane >> 4); r < 64; r += 2) sb += __bfloat162float(S.d[1][r][o]);
-            gb2 += sb;
-        }
-        back64(S.d[1], row0, S.net.w2t, dh);
-        __syncthreads();  // every warp has read d[0] (layer 3) and d[1]
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int r = row0 + g + (q >= 2 ? 8 : 0), c = 8 * j + 2 * t + (q & 1);
-                S.d[0][r][c] = __float2bfloat16_rn(dh[j][q] * dsilu_f(S.z[0][r][c]));
-            }
+        grad_stripe<8, kLd>(S.d[1], S.h[0], gW2);
+        gb2 += bias_sum(S.d[1]);
+        back(S.d[1], S.net.w2, 0);
+        // (every warp read d[0] before the last barrier)
+        store_rows(S.d[0], row0, A);
         __syncthreads();
         // layer 1 (inputs padded to 16; only i < 8 are real)
-        grad_stripe<2, 16>(S.d[0], S.x, gW1);
-        {
-            const int o = row0 + (lane & 15);
-            float sb = 0.f;
-            for (int r = (lane >> 4); r < 64; r += 2) sb += __bfloat162float(S.d[0][r][o]);
-            gb1 += sb;
-        }
+        grad_stripe<2, kLdX>(S.d[0], S.x, gW1);
+        gb1 += bias_sum(S.d[0]);
         __syncthreads();
     }
     // write this CTA's gradient slot (packing of the parameter vector)
@@ -614,15 +645,26 @@ __global__ void __launch_bounds__(128) k_mlp_train(int64_t nb, const int64_t *__
     }
 }
 
-// Sum the CTA slots in order; optionally apply Adam to the master weights.
-__global__ void k_mlp_reduce_adam(int nslots, const float *__restrict__ partial, float *__restrict__ grad,
-                                  float *__restrict__ P, float *__restrict__ m, float *__restrict__ v,
-                                  int adam, float lr, float b1, float b2, float eps, float c1, float c2)
+// Sum the CTA slots in a fixed order (32 parameters a block, eight threads each,
+// every eighth slot to a thread); optionally apply Adam to the master weights.
+__global__ void __launch_bounds__(256) k_mlp_reduce_adam(int nslots, const float *__restrict__ partial,
+                                                         float *__restrict__ grad, float *__restrict__ P,
+                                                         float *__restrict__ m, float *__restrict__ v,
+                                                         int adam, float lr, float b1, float b2, float eps,
+                                                         float c1, float c2)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= kMlpParams) return;
+    __shared__ float acc[8][32];
+    const int part = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + (threadIdx.x & 31);
     float s = 0.f;
-    for (int q = 0; q < nslots; ++q) s += partial[(size_t)q * kMlpParams + k];
+    if (k < kMlpParams) {
+#pragma unroll 8
+        for (int q = part; q < nslots; q += 8) s += partial[(size_t)q * kMlpParams + k];
+    }
+    acc[part][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (part != 0 || k >= kMlpParams) return;
+    for (int q = 1; q < 8; ++q) s += acc[q][threadIdx.x & 31];
     if (grad) grad[k] = s;
     if (!adam) return;
     const float mk = b1 * m[k] + (1.f - b1) * s;
@@ -638,8 +680,8 @@ cudaError_t mlp_predict(int64_t n, const float *X, const float *P, float *out, i
     cudaError_t e = set_max_dynamic_smem((const void *)k_mlp_predict, mlp_predict_smem());
     if (e != cudaSuccess) return e;
     const int64_t tiles = (n + 15) / 16;
-    const int grid = (int)min_i64((tiles + 3) / 4, (int64_t)num_sms * 8);
-    if (grid > 0) k_mlp_predict<<<grid, 128, mlp_predict_smem(), s>>>(n, X, P, out);
+    const int grid = (int)min_i64((tiles + 7) / 8, (int64_t)num_sms * 3);
+    if (grid > 0) k_mlp_predict<<<grid, 256, mlp_predict_smem(), s>>>(n, X, P, out);
     return cudaGetLastError();
 }
 
@@ -655,7 +697,7 @@ cudaError_t mlp_train_step(int64_t nb, const int64_t *idx, const float *X, const
     k_mlp_train<<<grid, 128, mlp_train_smem(), s>>>(nb, idx, X, Y, W, P, inv_n, partial, loss);
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f / (1.f - powf(b1, (float)step)), c2 = 1.f / (1.f - powf(b2, (float)step));
-    k_mlp_reduce_adam<<<(kMlpParams + 255) / 256, 256, 0, s>>>(grid, partial, grad, P, m, v, adam, lr,
+    k_mlp_reduce_adam<<<(kMlpParams + 31) / 32, 256, 0, s>>>(grid, partial, grad, P, m, v, adam, lr,
                                                                b1, b2, 1e-8f, c1, c2);
     return cudaGetLastError();
 }

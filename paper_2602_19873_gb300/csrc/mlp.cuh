@@ -24,7 +24,7 @@ cudaError_t mlp_apply_h0(uint32_t npad, int M, const uint32_t *perm_pad, const f
                          const float *e64, float *hq, cudaStream_t s);
 cudaError_t mlp_predict(int64_t n, const float *X, const float *P, float *out, int num_sms,
                         cudaStream_t s);
-// one minibatch (samples idx[0..nb)): gradient of sum_r w_r (pred_r - y_r)^2 * inv_n
+// one minibatch (samples idx[0..nb); idx NULL: samples 0 .. nb-1): gradient of sum_r w_r (pred_r - y_r)^2 * inv_n
 // into grad (if not NULL) and, when adam != 0, one Adam step of P (step >= 1)
 cudaError_t mlp_train_step(int64_t nb, const int64_t *idx, const float *X, const float *Y,
                            const float *W, float *P, float *m, float *v, float *partial,
