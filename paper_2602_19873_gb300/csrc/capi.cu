@@ -135,6 +135,10 @@ struct nl_list {
     uint32_t n_open = 0, n_per = 0;
     // periodic super-clusters split by the last search: interior / boundary
     DevBuf sc_int, sc_bnd;
+    // heavy super-clusters of the half search (two lists, and the parts of one),
+    // lists of more than kLongList entries: their number at the last build
+    DevBuf heavy, hpart, long_list, seek, seek_of;
+    uint32_t n_long = 0;
     DevBuf perm_pad, sys_off, sys_pad, sys_box, sys_root, sys_hcap;
     int32_t nsys = 1;
     // positions replaced since the search (nl_refresh_positions); pos_ref
@@ -205,7 +209,7 @@ struct nl_list {
                          &it_words, &it_tmp, &ml_X, &ml_e64, &ml_pred, &ml_slo, &ml_shi,
                          &uJ, &uM, &up_off, &up_cnt, &lower_cnt, &seg_off, &tkey, &tkey_alt,
                          &tval, &tval_alt, &thist, &sc_open, &sc_per, &sc_int, &sc_bnd,
-                         &pos_ref, &hsum, &hcnt, &hf};
+                         &pos_ref, &hsum, &hcnt, &hf, &heavy, &hpart, &long_list, &seek, &seek_of};
         for (DevBuf *b : all) b->release();
         for (int i = 0; i <= kStages; ++i)
             if (ev[i]) cudaEventDestroy(ev[i]);
@@ -367,6 +371,11 @@ nl_status do_prep(nl_list *nl, const float *x, const float *y, const float *z, c
     CK(nl->rec_off.ensure((size_t)nsc * 4));
     CK(nl->redo.ensure((size_t)nsc * 4));
     CK(nl->work.ensure((size_t)nsc * 4));
+    CK(nl->long_list.ensure((size_t)nsc * 8));
+    // seek points of the long records (those that find no room are decoded from
+    // their start)
+    CK(nl->seek.ensure(((size_t)N / 8 + nsc) * 8));
+    CK(nl->seek_of.ensure(((size_t)N / 8 + nsc) * 4));
     CK(nl->status.ensure(sizeof(Status)));
     CK(nl->sys_off.ensure((size_t)(nsys + 1) * 4));
     CK(nl->sys_pad.ensure((size_t)(nsys + 1) * 4));
@@ -512,7 +521,7 @@ cudaError_t search_all(nl_list *nl, const SearchArgs &sa, int M, int grid, int t
 
 // A pass over all super-clusters (a.work == NULL) or over a.work; split by
 // system kind and interior / boundary as the last search was.
-cudaError_t run_pass(const nl_list *nl, const PassArgs &a, int kind, cudaStream_t s)
+cudaError_t run_pass_split(const nl_list *nl, const PassArgs &a, int kind, cudaStream_t s)
 {
     const int M = nl->p.cluster;
     const int tpb = nl->p.threads_per_block, bps = nl->p.blocks_per_sm;
@@ -539,6 +548,29 @@ cudaError_t run_pass(const nl_list *nl, const PassArgs &a, int kind, cudaStream_
     return launch_pass(q, kind, M, 1, nl->num_sms, s, tpb, bps);
 }
 
+cudaError_t run_pass(const nl_list *nl, const PassArgs &a0, int kind, cudaStream_t s)
+{
+    const int M = nl->p.cluster;
+    const int tpb = nl->p.threads_per_block, bps = nl->p.blocks_per_sm;
+    PassArgs a = a0;
+    if (nl->n_long && !nl->graph_mode && pass_is_packed(kind, M, a.mj, a.support)) {
+        // the long lists, by many warps each, after the others (the device holds
+        // their list and number; those the caller did not ask for give the values
+        // they had)
+        a.skip_longer = kLongList;
+        cudaError_t e = run_pass_split(nl, a, kind, s);
+        if (e != cudaSuccess) return e;
+        a.work = nullptr;
+        a.nwork = nl->nsc;
+        a.nwork_dev = &a.st->n_long;
+        a.skip_longer = 0;
+        a.longs = nl->long_list.as<uint2>();
+        a.seek = nl->seek.as<uint2>();
+        return launch_pass(a, kind, M, nl->any_per, nl->num_sms, s, tpb, bps);
+    }
+    return run_pass_split(nl, a, kind, s);
+}
+
 // Half search (j-clusters = i-clusters): every super-cluster searches only
 // the j-clusters from its own first one on and sends the transposed tiles to
 // the later super-clusters; the tuples are sorted by (target, j-cluster) and
@@ -557,6 +589,7 @@ nl_status do_search_half(nl_list *nl, cudaStream_t s)
     const size_t search_words = sizeof(Status) - offsetof(Status, ticket);
     CK(cudaMemsetAsync(&dst->ticket, 0, search_words, s));
     size_t upc = 0, tuc = 0;
+    const uint32_t hcap = std::min<uint32_t>(nsc, 65536u);
     const int tpb = p->threads_per_block ? p->threads_per_block : 256;
     const int wpb = tpb / 32;
     const int grid0 = nl->num_sms * (p->blocks_per_sm ? p->blocks_per_sm : kSearchBlocksPerSM);
@@ -574,6 +607,7 @@ nl_status do_search_half(nl_list *nl, cudaStream_t s)
         CK(nl->uM.ensure(upc));
         CK(nl->tkey.ensure(tuc * 8));
         CK(nl->tval.ensure(tuc * 4));
+        CK(nl->heavy.ensure((size_t)2 * hcap * 4));
         if (const char *e = std::getenv("NLGB_STAGE_CAP0"))
             if (!nl->stage_grown) nl->stage_cap = (uint32_t)std::strtoul(e, nullptr, 10);
         CK(nl->stageJ.ensure(slots * nl->stage_cap * 4));
@@ -606,6 +640,10 @@ nl_status do_search_half(nl_list *nl, cudaStream_t s)
     sa.up_cnt = nl->up_cnt.as<uint32_t>();
     sa.lower_cnt = nl->lower_cnt.as<uint32_t>();
     sa.seg_off = nl->seg_off.as<uint32_t>();
+    sa.long_list = nl->long_list.as<uint2>();
+    sa.seek = nl->seek.as<uint2>();
+    sa.seek_of = nl->seek_of.as<uint32_t>();
+    sa.seek_cap = (uint32_t)std::min(nl->seek.cap / 8, nl->seek_of.cap / 4);
 
     int bits = 1;
     while (bits < 64 && ((unsigned long long)nsc * ncl >> bits) != 0) ++bits;
@@ -654,12 +692,29 @@ nl_status do_search_half(nl_list *nl, cudaStream_t s)
         sa.tkey = nl->tkey.as<uint64_t>();
         sa.tval = nl->tval.as<uint32_t>();
         sa.tu_cap = tuc;
+        // (a graph replay cannot come back for super-clusters set aside, nor do
+        // the redo rounds)
+        sa.heavy[0] = work ? nullptr : nl->heavy.as<uint32_t>();
+        sa.heavy[1] = work ? nullptr : nl->heavy.as<uint32_t>() + hcap;
+        sa.hcap = hcap;
         if (work)
             CK(launch_search_ctl(sa, work, count, nl->redo.as<uint32_t>(), M, nl->any_per, grid, tpb, s));
         else
             CK(search_all(nl, sa, M, grid, tpb, s));
         st = read_status(nl, s);
         if (st != NL_OK) return st;
+        const uint32_t heavy[2] = {std::min(nl->hst->n_heavy[0], hcap), std::min(nl->hst->n_heavy[1], hcap)};
+        if (!work && (heavy[0] || heavy[1]) && !nl->hst->half_overflow) {
+            uint32_t np[2];
+            for (int per = 0; per < 2; ++per)
+                np[per] = std::min(kSearchPartsMax, std::max(kSearchPartsMin, kSearchItems / std::max(heavy[per], 1u)));
+            CK(nl->hpart.ensure(std::max((size_t)heavy[0] * np[0], (size_t)heavy[1] * np[1]) * 4));
+            sa.hpart = nl->hpart.as<uint32_t>();
+            for (int per = 0; per < 2; ++per)
+                if (heavy[per]) CK(launch_search_heavy(sa, heavy[per], np[per], M, per, grid, tpb, s));
+            st = read_status(nl, s);
+            if (st != NL_OK) return st;
+        }
         nv += nl->hst->node_visits;
         lv += nl->hst->leaf_visits;
         jx += nl->hst->j_examined;
@@ -732,11 +787,18 @@ nl_status do_search_half(nl_list *nl, cudaStream_t s)
         CK(cudaMemsetAsync(&dst->n_tiles, 0, sizeof(dst->n_tiles), s));
         CK(cudaMemsetAsync(&dst->list_overflow, 0, sizeof(dst->list_overflow), s));
         CK(cudaMemsetAsync(&dst->asm_ticket, 0, sizeof(dst->asm_ticket), s));
+        CK(cudaMemsetAsync(&dst->n_long, 0, 2 * sizeof(dst->n_long), s));  // and n_seek
         sa.list = nl->list.as<uint8_t>();
         sa.list_cap = nl->list.cap - 8;  // 8 bytes of slack behind the last record
+        sa.defer_long = 1;
         CK(launch_assemble(sa, grid0, s));
         st = read_status(nl, s);
         if (st != NL_OK) return st;
+        if (nl->hst->n_seek && !nl->hst->list_overflow) {
+            CK(launch_assemble_long(sa, nl->hst->n_long, std::min(nl->hst->n_seek, sa.seek_cap), s));
+            st = read_status(nl, s);
+            if (st != NL_OK) return st;
+        }
         if (!nl->hst->list_overflow) break;
         const size_t need = (size_t)nl->hst->list_used + nl->hst->list_used / 8 + 65536;
         nl->list.release();
@@ -745,6 +807,7 @@ nl_status do_search_half(nl_list *nl, cudaStream_t s)
     CK(nl->mark(6, s));
     nl->collect(0, 6);
     nl->n = nl->n_prepared;
+    nl->n_long = nl->hst->n_long;
     nl->list_bytes = nl->hst->list_used;
     nl->n_entries = nl->hst->n_entries;
     nl->n_tiles = nl->hst->n_tiles;
@@ -809,6 +872,10 @@ nl_status do_search(nl_list *nl, cudaStream_t s)
     sa.compress = p->compress;
     sa.st = dst;
     sa.rec_off = nl->rec_off.as<uint32_t>();
+    sa.long_list = nl->long_list.as<uint2>();
+    sa.seek = nl->seek.as<uint2>();
+    sa.seek_of = nl->seek_of.as<uint32_t>();
+    sa.seek_cap = (uint32_t)std::min(nl->seek.cap / 8, nl->seek_of.cap / 4);
     sa.half = p->half_list ? 2 : 0;  // the half list: the half search's own entries as records
 
     unsigned long long entries = 0, tiles = 0, used = 0, nv = 0, lv = 0, jx = 0, tt = 0;
@@ -864,7 +931,10 @@ nl_status do_search(nl_list *nl, cudaStream_t s)
             bigger.p = nullptr;
         }
         const unsigned int keep_int = nl->hst->n_int, keep_bnd = nl->hst->n_bnd;
+        const unsigned int keep_long = nl->hst->n_long, keep_seek = nl->hst->n_seek;
         std::memset(&nl->hst->ticket, 0, search_words);
+        nl->hst->n_long = keep_long;
+        nl->hst->n_seek = keep_seek;
         nl->hst->list_used = keep;
         nl->hst->fail_off = ~0ull;
         nl->hst->n_int = keep_int;  // the passes use the first round's split
@@ -875,6 +945,7 @@ nl_status do_search(nl_list *nl, cudaStream_t s)
     CK(nl->mark(6, s));  // the full search has no assembly stage
     nl->collect(0, 6);
     nl->n = nl->n_prepared;
+    nl->n_long = nl->hst->n_long;
     nl->list_bytes = used;
     nl->n_entries = entries;
     nl->n_tiles = tiles;

@@ -12,6 +12,17 @@ constexpr int kKeyBits = 21;         // bits per axis of the 63-bit SFC key
 constexpr int kMaxLevel = 21;        // deepest octree level
 constexpr int kSC = 8;               // clusters per super-cluster (8-bit masks, Sec. II-A)
 constexpr uint32_t kBadRecord = 0xffffffffu;
+constexpr uint32_t kNoSeek = 0xffffffffu;
+// One warp works a list entry off in about 0.4 us (search) and 0.3 - 0.6 us (pass),
+// so lists of more entries than these are shared by many warps: a sparse
+// particle whose radius reaches a dense core can list all clusters of its system.
+constexpr uint32_t kLongSearch = 1024, kLongList = 1024;
+// j ranges a heavy super-cluster's search is split into: enough items for 32 per
+// warp of the grid (one range can be all neighbors: with 64 ranges of a 2^20-particle
+// system, 2048 j-clusters, a part ran for 1 ms)
+constexpr uint32_t kSearchPartsMin = 64, kSearchPartsMax = 1024, kSearchItems = 155648;
+constexpr uint32_t kPassParts = 16;         // blocks that share a long list at most
+constexpr uint32_t kSeek = 256;             // entries between the places a long record can be entered (multiple of 32)
 
 // Box with the derived FP32 quantities every kernel uses.  len = hi - lo,
 // half = 0.5f * len, qs = 2^21 / len, all rounded to nearest in FP32.
@@ -84,7 +95,10 @@ struct Status {
     unsigned int n_int, n_bnd;
     // density and pressure passes: bits of the largest |input| (half-list
     // density: sets the fixed-point scale)
-    unsigned int m_absmax, pad3;
+    unsigned int m_absmax;
+    // super-clusters whose lists grew past kLongSearch while searched (open and
+    // periodic kernel), and lists longer than kLongList
+    unsigned int n_heavy[2], n_long, n_seek;
 };
 
 // ---------------------------------------------------------------------------
@@ -640,10 +654,28 @@ struct SearchArgs {
     unsigned long long tu_cap;
     uint32_t *lower_cnt;           // per super-cluster: tuples addressed to it
     const uint32_t *seg_off;       // exclusive scan of lower_cnt (record assembly)
+    // records of more than kLongList entries (st->n_long of them): super-cluster
+    // and first seek point, one (stream position, previous index) per kSeek
+    // entries (kNoSeek: no room was left for them)
+    uint2 *long_list;
+    uint2 *seek;
+    uint32_t *seek_of;             // seek point -> index in long_list
+    uint32_t seek_cap;
+    int defer_long;                // record assembly: leave long records to launch_assemble_long
+    // heavy super-clusters of the half search, one list for the open and one for
+    // the periodic kernel (hcap entries each; NULL: none are set aside)
+    uint32_t *heavy[2];
+    uint32_t hcap;
+    uint32_t *hpart;               // per heavy super-cluster and part: entries, then their place in uJ
 };
 cudaError_t launch_search_ctl(const SearchArgs &a, const uint32_t *work, uint32_t count,
                               uint32_t *redo, int M, int any_periodic, int grid_blocks,
                               int threads, cudaStream_t s, const uint32_t *count_dev = nullptr);
+// Searches the count super-clusters a.heavy[per] in nparts j ranges each:
+// counts their upper entries, reserves them (super-cluster by super-cluster) and
+// writes them with their tuples.  Half search only.
+cudaError_t launch_search_heavy(const SearchArgs &a, uint32_t count, uint32_t nparts, int M, int per,
+                                int grid_blocks, int threads, cudaStream_t s);
 // Splits the super-clusters list[0..n) (NULL: 0..n-1) of periodic systems:
 // interior ones (their box widened by the system's largest radius, plus a
 // rounding margin, stays inside the box on every periodic axis, so no
@@ -657,6 +689,9 @@ cudaError_t launch_classify(const uint32_t *list, uint32_t n, int M, const SysTa
 // sorted tuples (lower j-clusters) followed by its upper entries, encoded as
 // by the search.  tkey/tval sorted by key; seg_off from seg_offsets().
 cudaError_t launch_assemble(const SearchArgs &a, int grid_blocks, cudaStream_t s);
+// Encodes the long records that the assembly left (a.defer_long), their n_seek
+// stretches of kSeek entries in parallel.
+cudaError_t launch_assemble_long(const SearchArgs &a, uint32_t n_long, uint32_t n_seek, cudaStream_t s);
 // keys[k] = fill for min(*used, cap) <= k < cap (unused tuple slots of a graph replay)
 cudaError_t launch_fill_keys(uint64_t *keys, uint32_t cap, const unsigned long long *used,
                              uint64_t fill, cudaStream_t s);
@@ -674,6 +709,9 @@ struct PassArgs {
     const float4 *aux4;    // SPH, packed kernel: (3 P/(pi rho^2 h^4), m, -1/(2h), 0)
     int packed;            // the packed kernel (pass_is_packed)
     int split;             // packed kernel: warps that share a super-cluster (1, 2, 4, 8)
+    uint32_t skip_longer;  // packed kernel: leave lists of more entries to a pass over the long ones (0: none)
+    const uint2 *longs;    // packed kernel: the long lists (nwork of them), worked off in parts
+    const uint2 *seek;
     uint32_t n, nsc;
     SysTables sys;
     float support;

@@ -35,7 +35,7 @@ cudaError_t launch_pass(const PassArgs &a0, int kind, int M, int any_periodic, i
     const uint64_t nwork = a.work ? a.nwork : a.nsc;
     const uint64_t slots = (uint64_t)num_sms * std::min(bps, 2) * (tpb / 32);
     a.split = 1;
-    while (a.split * 2 <= tpb / 32 && nwork * a.split * 2 <= slots) a.split *= 2;
+    while (a.split * 2 <= tpb / 32 && (a.longs || nwork * a.split * 2 <= slots)) a.split *= 2;
     switch (kind) {
     case PASS_DENSITY: return launch_pass_density(a, M, any_periodic, grid, tpb, s);
     case PASS_COUNT: return launch_pass_count(a, M, any_periodic, grid, tpb, s);

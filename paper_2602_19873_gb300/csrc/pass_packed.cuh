@@ -39,7 +39,9 @@
 //
 // split: W warps of a block share a super-cluster, each working on every W-th
 // stage.  Small systems have fewer super-clusters than the chip has warp slots,
-// and their passes are bound by the latency of one list.
+// and their passes are bound by the latency of one list.  Lists of more than
+// kLongList entries (skip_longer, longs) get a launch of their own in which whole
+// blocks, several of them where sums can meet in memory, share one list.
 #pragma once
 #include "nl_internal.cuh"
 #include "pass_decode.cuh"
@@ -161,6 +163,7 @@ struct PkSmem {
     float4 jc[JC ? NP : 1];
     f32x2 js[HL ? NC * SE * NT * 32 : NC * (kSC / G) * 16];
     float2 ib[IB ? NI : 2];
+    uint32_t seen, pad[3];
 };
 
 // Resident blocks of 256 threads the register budget is cut for (half-list
@@ -181,7 +184,8 @@ __device__ __forceinline__ void kahan_add(float &v, float &c, float b)
     v = t;
 }
 
-template <int M, int MJ, bool PER, int KIND, bool HL>
+// LONG: the pass over the long lists (a.longs).
+template <int M, int MJ, bool PER, int KIND, bool HL, bool LONG>
 __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pass_packed(PassArgs a)
 {
     static_assert(M * MJ >= 64, "a tile fills the lanes with pairs of j particles");
@@ -224,15 +228,49 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
     };
     auto merge = [](uint32_t u, uint32_t v) { return KIND == PASS_COUNT ? u + v : min(u, v); };
 
-    const uint32_t nwork = a.work ? (a.nwork_dev ? min(a.nwork, *a.nwork_dev) : a.nwork) : a.nsc;
+    const uint32_t nwork = a.work || LONG ? (a.nwork_dev ? min(a.nwork, *a.nwork_dev) : a.nwork) : a.nsc;
     for (uint32_t it = blockIdx.x + gridDim.x * grp;; it += gridDim.x * ngrp) {
-        uint32_t s = it;
-        if (W == 1u) {
-            if (lane == 0) s = atomicAdd(&a.st->pass_ticket, 1u);
-            s = __shfl_sync(0xffffffffu, s, 0);
+        uint32_t s = it, part = 0, seek = kNoSeek;
+        if constexpr (LONG) {  // (long list, block of it); first the first blocks of all
+            if (it >= nwork * kPassParts) break;
+            part = it / nwork;
+            const uint2 l = a.longs[it % nwork];
+            s = l.x;
+            seek = l.y;
+        } else {
+            if (W == 1u) {
+                if (lane == 0) s = atomicAdd(&a.st->pass_ticket, 1u);
+                s = __shfl_sync(0xffffffffu, s, 0);
+            }
+            if (s >= nwork) break;
+            if (a.work) s = a.work[s];
         }
-        if (s >= nwork) break;
-        if (a.work) s = a.work[s];
+        // a super-cluster whose list was not stored (an overflow inside a graph
+        // replay, reported by nl_graph_check) is read as an empty list
+        const uint32_t roff = a.rec_off[s];
+        const uint32_t *rec = reinterpret_cast<const uint32_t *>(a.list) + (roff == kBadRecord ? 0u : roff);
+        const uint32_t cnt = roff == kBadRecord ? 0u : rec[0];
+        // blocks that share the list: only where their sums meet in memory
+        constexpr bool SHARED = HL || INTS;
+        const uint32_t chunks = (cnt + kSeek - 1u) / kSeek;
+        uint32_t np = 1;
+        if constexpr (LONG) {
+            if (SHARED) np = min(kPassParts, (chunks + W - 1u) / W);
+            if (part >= np) continue;
+        }
+        if (!LONG && a.skip_longer && cnt > a.skip_longer) {
+            if constexpr (!HL && INTS) {  // empty results for the blocks to add to
+                for (uint32_t t = lane; t < (uint32_t)Smem::NI; t += 32) {
+                    const uint32_t i = s * kSC * M + t, pc = a.perm[i];
+                    if (pc == 0xffffffffu || wig != 0) continue;
+                    const uint32_t o = a.sorted_out ? i : pc;
+                    if constexpr (KIND == PASS_COUNT) a.outc[o] = 0u;
+                    else a.out0[o] = INFINITY;
+                }
+            }
+            continue;
+        }
+        const uint32_t VW = W * np, vw = part * W + wig;  // warps that share the list
         const PerLen box = per_len(a.sys.box[sys_of(a.sys.pad_off, a.sys.nsys, s * kSC * M)]);
 
         // own particles; the box around them (periodic)
@@ -289,20 +327,20 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
         }
         uint32_t selfseen = 0;  // bit r: the entry of own j-cluster r lists its own i-cluster
 
-        // a super-cluster whose list was not stored (an overflow inside a graph
-        // replay, reported by nl_graph_check) is read as an empty list
-        const uint32_t roff = a.rec_off[s];
-        const uint32_t *rec = reinterpret_cast<const uint32_t *>(a.list) + (roff == kBadRecord ? 0u : roff);
-        const uint32_t cnt = roff == kBadRecord ? 0u : rec[0];
         const uint8_t *masks = reinterpret_cast<const uint8_t *>(rec + 1);
         const uint32_t *body = rec + 1 + ((cnt + 3u) >> 2);
-        uint32_t pos = 0;
-        uint32_t prevJ = 0xffffffffu;
-
-        for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
+        // a long list: every VW-th chunk of kSeek entries, entered at its seek
+        // point; else the whole list, of which the warps take stages in turn
+        for (uint32_t ch = LONG ? vw : 0u; ch < (LONG ? chunks : 1u); ch += VW) {
+        const uint32_t cbeg = LONG ? ch * kSeek : 0u, cend = LONG ? min(cnt, cbeg + kSeek) : cnt;
+        const uint2 at = LONG && seek != kNoSeek ? a.seek[seek + ch] : make_uint2(0u, 0xffffffffu);
+        uint32_t pos = at.x;
+        uint32_t prevJ = at.y;
+        for (uint32_t b0 = LONG && seek != kNoSeek ? cbeg : 0u; b0 < cend; b0 += 32) {
             const uint32_t t = b0 + lane;
             const bool valid = t < cnt;
             const uint32_t J = decode_block(body, a.compress, t, valid, pos, prevJ);
+            if (LONG && b0 < cbeg) continue;  // (no seek points: decode up to the chunk)
             const uint32_t mk = valid ? masks[t] : 0u;
             const uint32_t rel = J - s * kSC * RJ;  // own j-clusters: below kSC RJ
             const uint32_t own = __ballot_sync(0xffffffffu, valid && rel < kSC * RJ);
@@ -313,7 +351,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             // half list: entries beyond the own clusters also feed their j particles
             const uint32_t feeds = HL ? __ballot_sync(0xffffffffu, valid) & ~own : 0u;
             for (uint32_t c = 0; c < min(32u, cnt - b0); c += SE) {
-                if (W != 1u && ((b0 + c) / SE & (W - 1u)) != wig) continue;
+                if (!LONG && W != 1u && (b0 + c) / SE % W != wig) continue;
                 const uint32_t ns = min(SE, cnt - b0 - c);
                 // stage the j particles of entries c .. c + ns - 1
                 uint32_t slow = careful ? 0xffffffffu : 0u;  // bit el: entry c + el takes the scalar terms
@@ -663,6 +701,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                 }
             }
         }
+        }
         if constexpr (INTS) {
 #pragma unroll
             for (uint32_t q = 0; q < NK; ++q) rx[q] = __uint_as_float(rc[q]);
@@ -672,6 +711,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
         // a fixed order (half lists add their sums to memory anyway)
         if (!HL && W != 1u) {
             float *mine = reinterpret_cast<float *>(S.js);
+            if (lane == 0) S.seen = selfseen;
             __syncwarp();
 #pragma unroll
             for (uint32_t q = 0; q < NK; ++q) {
@@ -685,6 +725,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             if (wig == 0) {
                 for (uint32_t w = 1; w < W; ++w) {
                     const float *o = reinterpret_cast<const float *>(all[warp + w].js);
+                    selfseen |= all[warp + w].seen;
 #pragma unroll
                     for (uint32_t q = 0; q < NK; ++q) {
                         const float v = o[q * 32 + lane];
@@ -721,7 +762,8 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             const bool took_self = seen && (KIND == PASS_DENSITY ? isfinite(av) : av > 0.f);
             if constexpr (KIND == PASS_DENSITY) {
                 float v = 2.f * rx[q];  // sums are in units of w/2
-                if (wig == 0 && !took_self) v += a.aux[i].x;  // m_i w(0) = m_i
+                // m_i w(0) = m_i  (half lists: the own entries come first, at warp 0)
+                if (vw == 0 && !took_self) v += a.aux[i].x;
                 if constexpr (HL) {
                     atomicAdd(&a.hsum[i], fixed_of(v * hscale));
                 } else {
@@ -729,12 +771,16 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                     a.out0[o] = v * (0.318309886183790672f * hk * hk * hk);
                 }
             } else if constexpr (KIND == PASS_COUNT) {
-                const uint32_t v = __float_as_uint(rx[q]) - (wig == 0 && took_self ? 1u : 0u);
+                // (of a long list only the warps or block at the own entries saw them)
+                const uint32_t v = __float_as_uint(rx[q]) - ((vw == 0 || LONG) && took_self ? 1u : 0u);
                 if constexpr (HL) atomicAdd(&a.hcnt[i], v);
+                else if (np > 1u) atomicAdd(&a.outc[o], v);
                 else a.outc[o] = v;
             } else if constexpr (KIND == PASS_MIN) {
                 if constexpr (HL) {
                     if (rx[q] < INFINITY) atomicMin(&a.hcnt[i], __float_as_uint(rx[q]));
+                } else if (np > 1u) {
+                    atomicMin(reinterpret_cast<unsigned int *>(&a.out0[o]), __float_as_uint(sqrtf(rx[q])));
                 } else {
                     a.out0[o] = sqrtf(rx[q]);  // +inf without a neighbor
                 }
@@ -758,15 +804,13 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
 template <int M, int MJ, int KIND, bool HL>
 static cudaError_t launch_packed_mk(const PassArgs &a, int per, int grid, int threads, cudaStream_t s)
 {
-    const size_t smem = (size_t)(threads / 32) * sizeof(PkSmem<M, MJ, KIND, HL>);
-    const void *fn = per ? (const void *)k_pass_packed<M, MJ, true, KIND, HL>
-                         : (const void *)k_pass_packed<M, MJ, false, KIND, HL>;
-    cudaError_t e = set_max_dynamic_smem(fn, (size_t)(PK_THREADS / 32) * sizeof(PkSmem<M, MJ, KIND, HL>));
+    // (the periodic arithmetic gives open axes, of infinite length, the open results)
+    auto *fn = a.longs ? k_pass_packed<M, MJ, true, KIND, HL, true>
+               : per   ? k_pass_packed<M, MJ, true, KIND, HL, false>
+                       : k_pass_packed<M, MJ, false, KIND, HL, false>;
+    cudaError_t e = set_max_dynamic_smem((const void *)fn, (size_t)(PK_THREADS / 32) * sizeof(PkSmem<M, MJ, KIND, HL>));
     if (e != cudaSuccess) return e;
-    if (per)
-        k_pass_packed<M, MJ, true, KIND, HL><<<grid, threads, smem, s>>>(a);
-    else
-        k_pass_packed<M, MJ, false, KIND, HL><<<grid, threads, smem, s>>>(a);
+    fn<<<grid, threads, (size_t)(threads / 32) * sizeof(PkSmem<M, MJ, KIND, HL>), s>>>(a);
     return cudaGetLastError();
 }
 

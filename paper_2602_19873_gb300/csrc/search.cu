@@ -55,6 +55,12 @@ struct SearchCtl {
     uint32_t count;
     uint32_t *redo;         // ids that could not be stored this time
     const uint32_t *count_dev;  // optional device count (at most count)
+    uint32_t *heavy;            // half search: super-clusters set aside as heavy (NULL: none are)
+    unsigned int *n_heavy;
+    // the heavy super-clusters in work, nparts j ranges each: phase 1 counts their
+    // entries, phase 2 writes them
+    int phase;
+    uint32_t nparts;
 };
 
 __device__ __forceinline__ uint32_t hex_digits(uint32_t v) { return (32u - __clz(v) + 3u) >> 2; }
@@ -65,67 +71,79 @@ __device__ __forceinline__ void win_put(uint32_t *win, uint32_t W0, uint32_t p, 
     atomicOr(&win[l >> 3], v << ((l & 7u) * 4u));
 }
 
-// Encode the list of one super-cluster: entry t is (getJ(t), getM(t)),
-// ascending in J.  Returns false when the list buffer is full (nothing
-// written for this super-cluster).
-template <class GJ, class GM>
-__device__ bool encode_record(uint32_t cnt, GJ getJ, GM getM, uint32_t *win, const SearchArgs &a,
-                              uint32_t s)
+// Place of a long record in the list of long records and its seek points
+// (kNoSeek: no room), one warp.
+__device__ uint32_t long_record(uint32_t cnt, const SearchArgs &a, uint32_t s)
 {
     const unsigned lane = lane_id();
-    const unsigned lt = lanemask_lt();
-    uint32_t nib = 0;
-    if (a.compress) {
-        uint32_t carry = 0xffffffffu;  // J_{-1} = -1
-        for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
-            uint32_t t = b0 + lane;
-            uint32_t J = t < cnt ? getJ(t) : 0u;
-            uint32_t prev = __shfl_up_sync(0xffffffffu, J, 1);
-            if (lane == 0) prev = carry;
-            uint32_t d = t < cnt ? J - prev : 1u;
-            uint32_t nb = d == 1u ? 0u : (d <= 9u ? 1u : 1u + hex_digits(d));
-            nib += 8u + warp_sum(nb);
-            carry = __shfl_sync(0xffffffffu, J, 31);
-        }
-    }
-    const uint32_t mask_words = (cnt + 3u) >> 2;
-    const uint32_t body_words = a.compress ? (nib + 7u) >> 3 : cnt;
-    const uint32_t words = 1u + mask_words + body_words;
-    unsigned long long off = 0;
-    if (lane == 0) off = atomicAdd(&a.st->list_used, (unsigned long long)words * 4ull);
-    off = __shfl_sync(0xffffffffu, off, 0);
-    if (off + (unsigned long long)words * 4ull > a.list_cap) {
-        // reservations only grow, so every record below the lowest failed
-        // offset was stored; the host resumes allocation there
-        if (lane == 0) atomicMin(&a.st->fail_off, off);
-        return false;
-    }
-    uint32_t *rec = reinterpret_cast<uint32_t *>(a.list + off);
+    const uint32_t ns = (cnt + kSeek - 1u) / kSeek;
+    uint32_t li = 0, seek = 0;
     if (lane == 0) {
-        rec[0] = cnt;
-        a.rec_off[s] = (uint32_t)(off >> 2);
+        li = atomicAdd(&a.st->n_long, 1u);
+        seek = atomicAdd(&a.st->n_seek, ns);
     }
-    for (uint32_t w = lane; w < mask_words; w += 32) {
+    li = __shfl_sync(0xffffffffu, li, 0);
+    seek = __shfl_sync(0xffffffffu, seek, 0);
+    const bool room = seek <= a.seek_cap && ns <= a.seek_cap - seek;
+    // (the points below the capacity that found no room belong to no record)
+    for (uint32_t k = lane; k < ns && seek + k < a.seek_cap; k += 32) a.seek_of[seek + k] = room ? li : kNoSeek;
+    if (!room) seek = kNoSeek;
+    if (lane == 0) a.long_list[li] = make_uint2(s, seek);
+    return seek;
+}
+
+// Nibbles of the stream of entries beg .. end (carry: the index before them).
+template <class GJ>
+__device__ uint32_t stream_nibbles(uint32_t beg, uint32_t end, uint32_t carry, GJ getJ)
+{
+    const unsigned lane = lane_id();
+    uint32_t nib = 0;
+    for (uint32_t b0 = beg; b0 < end; b0 += 32) {
+        uint32_t t = b0 + lane;
+        uint32_t J = t < end ? getJ(t) : 0u;
+        uint32_t prev = __shfl_up_sync(0xffffffffu, J, 1);
+        if (lane == 0) prev = carry;
+        uint32_t d = t < end ? J - prev : 1u;
+        uint32_t nb = d == 1u ? 0u : (d <= 9u ? 1u : 1u + hex_digits(d));
+        nib += 8u + warp_sum(nb);
+        carry = __shfl_sync(0xffffffffu, J, 31);
+    }
+    return nib;
+}
+
+// Mask words of entries beg .. end (beg a multiple of 4).
+template <class GM>
+__device__ void put_masks(uint32_t *words, uint32_t beg, uint32_t end, GM getM)
+{
+    for (uint32_t w = beg / 4 + lane_id(); w < (end + 3u) / 4; w += 32) {
         uint32_t v = 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             uint32_t t = 4 * w + q;
-            if (t < cnt) v |= (getM(t) & 0xffu) << (8 * q);
+            if (t < end) v |= (getM(t) & 0xffu) << (8 * q);
         }
-        rec[1 + w] = v;
+        words[w] = v;
     }
-    uint32_t *body = rec + 1 + mask_words;
-    if (!a.compress) {
-        for (uint32_t t = lane; t < cnt; t += 32) body[t] = getJ(t);
-        return true;
-    }
+}
+
+// Stream of entries beg .. end from nibble pos on (carry: the index before
+// them).  PART: words shared with other stretches (zeroed before) are or-ed in.
+// seek: where to note the seek points, or NULL.
+template <bool PART, class GJ>
+__device__ void put_stream(uint32_t *body, uint32_t *win, uint32_t beg, uint32_t end, uint32_t pos, uint32_t carry,
+                           GJ getJ, uint2 *seek)
+{
+    const unsigned lane = lane_id();
+    const unsigned lt = lanemask_lt();
+    uint32_t W0 = pos & ~7u;
+    bool shared = PART && (pos & 7u);  // the first word of the window
     win[lane] = 0u;
     win[lane + 32] = 0u;
     __syncwarp();
-    uint32_t W0 = 0, pos = 0, carry = 0xffffffffu;
-    for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
+    for (uint32_t b0 = beg; b0 < end; b0 += 32) {
+        if (seek && b0 % kSeek == 0 && lane == 0) seek[b0 / kSeek] = make_uint2(pos, carry);
         uint32_t t = b0 + lane;
-        bool valid = t < cnt;
+        bool valid = t < end;
         uint32_t J = valid ? getJ(t) : 0u;
         uint32_t prev = __shfl_up_sync(0xffffffffu, J, 1);
         if (lane == 0) prev = carry;
@@ -144,7 +162,11 @@ __device__ bool encode_record(uint32_t cnt, GJ getJ, GM getM, uint32_t *win, con
         __syncwarp();
         uint32_t pend = pos + 8 + nbits + tot;
         uint32_t full = (pend - W0) >> 3;
-        for (uint32_t w = lane; w < full; w += 32) body[(W0 >> 3) + w] = win[w];
+        for (uint32_t w = lane; w < full; w += 32) {
+            if (PART && shared && w == 0) atomicOr(&body[W0 >> 3], win[0]);
+            else body[(W0 >> 3) + w] = win[w];
+        }
+        if (full) shared = false;
         __syncwarp();
         uint32_t keep = win[full];
         __syncwarp();
@@ -157,8 +179,55 @@ __device__ bool encode_record(uint32_t cnt, GJ getJ, GM getM, uint32_t *win, con
         pos = pend;
         carry = __shfl_sync(0xffffffffu, J, 31);
     }
-    if (pos > W0 && lane == 0) body[W0 >> 3] = win[0];
+    if (pos > W0 && lane == 0) {
+        if (PART) atomicOr(&body[W0 >> 3], win[0]);
+        else body[W0 >> 3] = win[0];
+    }
     __syncwarp();
+}
+
+// Room for a record of `words` words: its words, or NULL when the list buffer
+// is full.  Writes the count and the super-cluster's offset.
+__device__ uint32_t *take_record(uint32_t words, uint32_t cnt, const SearchArgs &a, uint32_t s)
+{
+    const unsigned lane = lane_id();
+    unsigned long long off = 0;
+    if (lane == 0) off = atomicAdd(&a.st->list_used, (unsigned long long)words * 4ull);
+    off = __shfl_sync(0xffffffffu, off, 0);
+    if (off + (unsigned long long)words * 4ull > a.list_cap) {
+        // reservations only grow, so every record below the lowest failed
+        // offset was stored; the host resumes allocation there
+        if (lane == 0) atomicMin(&a.st->fail_off, off);
+        return nullptr;
+    }
+    uint32_t *rec = reinterpret_cast<uint32_t *>(a.list + off);
+    if (lane == 0) {
+        rec[0] = cnt;
+        a.rec_off[s] = (uint32_t)(off >> 2);
+    }
+    return rec;
+}
+
+// Encode the list of one super-cluster: entry t is (getJ(t), getM(t)),
+// ascending in J.  Returns false when the list buffer is full (nothing
+// written for this super-cluster).
+// noted: a long record that has its place in the list of long records already.
+template <class GJ, class GM>
+__device__ bool encode_record(uint32_t cnt, GJ getJ, GM getM, uint32_t *win, const SearchArgs &a,
+                              uint32_t s, bool noted = false)
+{
+    const uint32_t nib = a.compress ? stream_nibbles(0, cnt, 0xffffffffu, getJ) : 0u;  // J_{-1} = -1
+    const uint32_t mask_words = (cnt + 3u) >> 2;
+    uint32_t *rec = take_record(1u + mask_words + (a.compress ? (nib + 7u) >> 3 : cnt), cnt, a, s);
+    if (!rec) return false;
+    const uint32_t seek = cnt > kLongList && !noted ? long_record(cnt, a, s) : kNoSeek;
+    put_masks(rec + 1, 0, cnt, getM);
+    uint32_t *body = rec + 1 + mask_words;
+    if (!a.compress) {
+        for (uint32_t t = lane_id(); t < cnt; t += 32) body[t] = getJ(t);
+        return true;
+    }
+    put_stream<false>(body, win, 0, cnt, 0, 0xffffffffu, getJ, seek != kNoSeek ? a.seek + seek : nullptr);
     return true;
 }
 
@@ -170,11 +239,13 @@ __device__ bool encode_record(uint32_t cnt, GJ getJ, GM getM, uint32_t *win, con
 // them, so a group spans at most two 32-entry chunks and is carried over).
 // Returns false when a buffer was too small (the reservations still count,
 // so the host learns the sizes it needs).
+__device__ bool half_tuples(uint32_t cnt, const uint32_t *stJ, const uint8_t *stM, const SearchArgs &a,
+                            uint32_t s);
+
 __device__ bool half_output(uint32_t cnt, const uint32_t *stJ, const uint8_t *stM,
                             const SearchArgs &a, uint32_t s)
 {
     const unsigned lane = lane_id();
-    constexpr uint32_t NONE = 0xffffffffu;
     unsigned long long off = 0;
     if (lane == 0) off = atomicAdd(&a.st->up_used, (unsigned long long)cnt);
     off = __shfl_sync(0xffffffffu, off, 0);
@@ -190,6 +261,16 @@ __device__ bool half_output(uint32_t cnt, const uint32_t *stJ, const uint8_t *st
         a.up_off[s] = (uint32_t)off;
         a.up_cnt[s] = cnt;
     }
+    return half_tuples(cnt, stJ, stM, a, s);
+}
+
+// The transposed tuples of entries of super-cluster s (all of one target
+// super-cluster together).
+__device__ bool half_tuples(uint32_t cnt, const uint32_t *stJ, const uint8_t *stM, const SearchArgs &a,
+                            uint32_t s)
+{
+    const unsigned lane = lane_id();
+    constexpr uint32_t NONE = 0xffffffffu;
     const uint32_t own_end = (s + 1) * kSC;  // first cluster after the own ones
     const uint32_t i0 = s * kSC;
     bool ok = true;
@@ -316,7 +397,8 @@ __device__ __forceinline__ void box_pair_near(const float4 *ib, const float4 &bl
 
 // MODE 0: full list.  MODE 1: half search, upper entries and transposed
 // tuples for the record assembly.  MODE 2: half list (each pair stored once,
-// Sec. II-D): the half search's upper entries encoded as the record.
+// Sec. II-D): the half search's upper entries encoded as the record.  MODE 3:
+// mode 1 for the parts of heavy super-clusters (ctl.phase).
 template <int M, int MJ, bool PER, int MODE>
 __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCtl ctl)
 {
@@ -345,10 +427,31 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
         if (lane == 0) tk = atomicAdd(&a.st->ticket, 1u);
         tk = __shfl_sync(0xffffffffu, tk, 0);
         if (tk >= count) break;
-        const uint32_t s = ctl.work ? ctl.work[tk] : tk;
+        const uint32_t wi = MODE == 3 ? tk / ctl.nparts : tk;
+        const uint32_t s = ctl.work ? ctl.work[wi] : wi;
         const uint32_t base = s * kSC * M;
         // the super-cluster's system: its box and its own octree subtree
         const uint32_t sy = sys_of(a.sys.pad_off, a.sys.nsys, base);
+        // particles searched: from the own first one on (half search), or one of
+        // nparts ranges of whole super-clusters of them
+        uint32_t pbeg = HALF ? base : 0u, pend = 0xffffffffu;
+        uint32_t cap = a.stage_cap;
+        if constexpr (MODE == 3) {
+            const uint32_t n8 = (a.sys.pad_off[sy + 1] - base) / (kSC * M), part = tk % ctl.nparts;
+            pbeg = base + (uint32_t)((uint64_t)n8 * part / ctl.nparts) * (kSC * M);
+            pend = base + (uint32_t)((uint64_t)n8 * (part + 1) / ctl.nparts) * (kSC * M);
+            cap = 0;
+            if (ctl.phase == 2) {
+                if (a.st->half_overflow) continue;  // (the host starts over)
+                stJ = a.uJ + a.hpart[tk];
+                stM = a.uM + a.hpart[tk];
+                cap = 0xffffffffu;
+            }
+            if (pbeg == pend) {
+                if (ctl.phase == 1 && lane == 0) a.hpart[tk] = 0u;
+                continue;
+            }
+        }
         const PerLen box = per_len(a.sys.box[sy]);
         // (clamped to the node arrays: after a node overflow in a graph replay
         // the tables may be stale, and the replay is reported as failed)
@@ -390,8 +493,9 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
 
         uint32_t cnt = 0, tiles = 0, nvis = 0, lvis = 0, jex = 0, ttests = 0;
         uint32_t qh = 0, qt = 0;  // queue of j-clusters, ring positions
+        bool aside = MODE == 1 && ctl.heavy != nullptr;  // may be set aside
         // the half search takes only j-clusters from its own first one on
-        int lastJ = HALF ? (int)(base / MJ) - 1 : -1;
+        int lastJ = (int)(pbeg / MJ) - 1;
 
         // Test a batch of up to NB queued j-clusters.
         auto batch = [&]() {
@@ -486,7 +590,7 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 mask = S.found[lane];
                 const uint32_t has = __ballot_sync(0xffffffffu, mask != 0u);
                 const uint32_t o = cnt + __popc(has & lanemask_lt());
-                if (mask && o < a.stage_cap) {
+                if (mask && o < cap) {
                     stJ[o] = J;
                     stM[o] = (uint8_t)mask;
                 }
@@ -506,14 +610,14 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
         // j-clusters of the leaves that pass are queued until a batch is full.
         uint32_t v = vroot, leaves = 0;  // leaves: of the current chunk, not queued yet
         if constexpr (HALF) {
-            // start at the leaf that holds the first own particle: the last
-            // node in pre-order whose range begins at or before it (the range
-            // starts ascend in pre-order); 32 probes a round
+            // start at the leaf that holds the first particle: the last node in
+            // pre-order whose range begins at or before it (the range starts
+            // ascend in pre-order); 32 probes a round
             uint32_t hi = vend;  // nodes [v, hi) may be it; v itself begins early enough
             while (hi - v > 1) {
                 const uint32_t step = (hi - v + 31u) >> 5;
                 const uint32_t u = v + lane * step;
-                const uint32_t m = __ballot_sync(0xffffffffu, u < hi && (uint32_t)a.nrng[min(u, vend - 1)].x <= base);
+                const uint32_t m = __ballot_sync(0xffffffffu, u < hi && (uint32_t)a.nrng[min(u, vend - 1)].x <= pbeg);
                 const uint32_t last = 31u - __clz(m | 1u);
                 v += last * step;
                 hi = min(hi, v + step);
@@ -535,6 +639,7 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                     leaves &= leaves - 1u;
                     Jlo = max(__shfl_sync(0xffffffffu, rg.x, b) / MJ, lastJ + 1);
                     Jhi = (__shfl_sync(0xffffffffu, rg.y, b) - 1) / MJ;
+                    if (MODE == 3) Jhi = (int)min((uint32_t)Jhi, pend / MJ - 1u);
                     lastJ = max(lastJ, Jhi);
                     ++lvis;
                     jex += (uint32_t)max(Jhi - Jlo + 1, 0);
@@ -550,10 +655,12 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                     nhi = a.nhi[u];
                     rg = a.nrng[u];
                     skip = (uint32_t)__float_as_int(nhi.w);
-                    // (wholly before the own particles: not for a half search)
-                    near = (!HALF || (uint32_t)rg.y > base) && boxes_near<PER>(slo, shi, nlo, nhi, box);
+                    // (wholly before the first particle: not for a half search)
+                    near = (!HALF || (uint32_t)rg.y > pbeg) && (MODE != 3 || (uint32_t)rg.x < pend) &&
+                           boxes_near<PER>(slo, shi, nlo, nhi, box);
                 }
                 uint32_t next = max(v + 32u, __reduce_max_sync(0xffffffffu, near ? 0u : skip));
+                if (MODE == 3 && __any_sync(0xffffffffu, u < vend && (uint32_t)rg.x >= pend)) next = vend;
                 leaves = __ballot_sync(0xffffffffu, near && skip == u + 1u);
                 nvis += min(32u, vend - v);
                 // (also when few of the j-clusters reached by boxes hold a pair)
@@ -593,8 +700,34 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
             if (qt == qh) break;
             __syncwarp();
             batch();
+            if (MODE == 1 && aside && cnt > kLongSearch) {
+                // too long for one warp: set aside for the search in parts
+                uint32_t h = 0;
+                if (lane == 0) {
+                    h = atomicAdd(ctl.n_heavy, 1u);
+                    if (h < a.hcap) ctl.heavy[h] = s;
+                }
+                h = __shfl_sync(0xffffffffu, h, 0);
+                if (h < a.hcap) break;
+                aside = false;
+            }
         }
         __syncwarp();
+        if (MODE == 1 && aside && cnt > kLongSearch) continue;
+        if constexpr (MODE == 3) {
+            if (ctl.phase == 1) {
+                if (lane == 0) a.hpart[tk] = cnt;
+            } else if (!half_tuples(cnt, stJ, stM, a, s) && lane == 0) {
+                atomicExch(&a.st->half_overflow, 1u);
+            }
+            if (lane == 0 && ctl.phase == 2) {
+                atomicAdd(&a.st->node_visits, (unsigned long long)nvis);
+                atomicAdd(&a.st->leaf_visits, (unsigned long long)lvis);
+                atomicAdd(&a.st->j_examined, (unsigned long long)jex);
+                atomicAdd(&a.st->tile_tests, (unsigned long long)ttests);
+            }
+            continue;
+        }
         tiles = warp_sum(tiles);
         const bool staged = cnt <= a.stage_cap;
         bool ok = staged;
@@ -649,7 +782,8 @@ cudaError_t launch_search_ctl(const SearchArgs &a, const uint32_t *work, uint32_
                               uint32_t *redo, int M, int any_periodic, int grid, int threads,
                               cudaStream_t s, const uint32_t *count_dev)
 {
-    SearchCtl c{work, count, redo, count_dev};
+    SearchCtl c{work, count, redo, count_dev, a.half == 1 ? a.heavy[any_periodic ? 1 : 0] : nullptr,
+                &a.st->n_heavy[any_periodic ? 1 : 0], 0, 0};
     if (threads != 128 && threads != SR_THREADS) return cudaErrorInvalidValue;
     if (a.half && a.mj != M) return cudaErrorInvalidValue;  // needs j-clusters = i-clusters
     if (a.half < 0 || a.half > 2) return cudaErrorInvalidValue;
@@ -672,10 +806,77 @@ cudaError_t launch_search_ctl(const SearchArgs &a, const uint32_t *work, uint32_
     }
 }
 
+// Upper entries of a heavy super-cluster from the counts of its parts: one
+// reservation, then the place of every part (one warp per super-cluster).
+__global__ void __launch_bounds__(128) k_heavy_place(SearchArgs a, const uint32_t *heavy, uint32_t count, uint32_t nparts)
+{
+    const uint32_t h = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (h >= count) return;
+    const unsigned lane = lane_id();
+    uint32_t *part = a.hpart + (size_t)h * nparts, cnt = 0;
+    for (uint32_t p = lane; p < nparts; p += 32) cnt += part[p];
+    cnt = warp_sum(cnt);
+    unsigned long long off = 0;
+    if (lane == 0) off = atomicAdd(&a.st->up_used, (unsigned long long)cnt);
+    off = __shfl_sync(0xffffffffu, off, 0);
+    if (off + cnt > a.up_cap) {
+        if (lane == 0) atomicExch(&a.st->half_overflow, 1u);
+        return;
+    }
+    if (lane == 0) {
+        a.up_off[heavy[h]] = (uint32_t)off;
+        a.up_cnt[heavy[h]] = cnt;
+    }
+    uint32_t at = (uint32_t)off;
+    for (uint32_t p0 = 0; p0 < nparts; p0 += 32) {
+        const uint32_t c = p0 + lane < nparts ? part[p0 + lane] : 0u;
+        const uint32_t incl = warp_incl_scan(c);
+        if (p0 + lane < nparts) part[p0 + lane] = at + incl - c;
+        at += __shfl_sync(0xffffffffu, incl, 31);
+    }
+}
+
+cudaError_t launch_search_heavy(const SearchArgs &a, uint32_t count, uint32_t nparts, int M, int per, int grid,
+                                int threads, cudaStream_t s)
+{
+    if (a.half != 1 || !count || !nparts) return cudaErrorInvalidValue;
+    const uint32_t *heavy = a.heavy[per ? 1 : 0];
+    for (int phase = 1; phase <= 2; ++phase) {
+        SearchCtl c{heavy, count * nparts, nullptr, nullptr, nullptr, nullptr, phase, nparts};
+        cudaError_t e = cudaMemsetAsync(&a.st->ticket, 0, sizeof(a.st->ticket), s);
+        if (e != cudaSuccess) return e;
+        switch (M) {
+        case 4: e = launch_m<4, 4, 3>(a, c, per, grid, threads, s); break;
+        case 8: e = launch_m<8, 8, 3>(a, c, per, grid, threads, s); break;
+        case 16: e = launch_m<16, 16, 3>(a, c, per, grid, threads, s); break;
+        default: e = cudaErrorInvalidValue;
+        }
+        if (e != cudaSuccess) return e;
+        if (phase == 1) k_heavy_place<<<(count + 3) / 4, 128, 0, s>>>(a, heavy, count, nparts);
+    }
+    return cudaGetLastError();
+}
+
 // Record assembly of the half search: one warp per super-cluster t.  Its
 // record is the sorted tuples addressed to it (j-clusters below its own
 // clusters; keys t * ncl + J, values the mask bits) followed by its upper
 // entries, encoded exactly like a record of the full search.
+struct AssembleSrc {
+    const uint64_t *tkey;
+    const uint32_t *tval, *uJ;
+    const uint8_t *uM;
+    uint64_t kb;
+    uint32_t lc, so, uc, uo;
+    __device__ AssembleSrc(const SearchArgs &a, uint32_t t)
+        : tkey(a.tkey), tval(a.tval), uJ(a.uJ), uM(a.uM), kb((uint64_t)t * a.ncl), lc(a.lower_cnt[t]),
+          so(a.seg_off[t]), uc(a.up_cnt[t]), uo(a.up_off[t])
+    {
+    }
+    __device__ uint32_t count() const { return lc + uc; }
+    __device__ uint32_t J(uint32_t i) const { return i < lc ? (uint32_t)(tkey[so + i] - kb) : uJ[uo + (i - lc)]; }
+    __device__ uint32_t M(uint32_t i) const { return i < lc ? tval[so + i] : (uint32_t)uM[uo + (i - lc)]; }
+};
+
 __global__ void __launch_bounds__(SR_THREADS) k_assemble(SearchArgs a)
 {
     __shared__ uint32_t wins[SR_WARPS][WIN_WORDS];
@@ -692,19 +893,14 @@ __global__ void __launch_bounds__(SR_THREADS) k_assemble(SearchArgs a)
             if (lane == 0) a.rec_off[t] = kBadRecord;
             continue;
         }
-        const uint32_t lc = a.lower_cnt[t], so = a.seg_off[t];
-        const uint32_t uc = a.up_cnt[t], uo = a.up_off[t];
-        const uint32_t cnt = lc + uc;
-        const uint64_t kb = (uint64_t)t * a.ncl;
-        auto getJ = [&](uint32_t i) -> uint32_t {
-            return i < lc ? (uint32_t)(a.tkey[so + i] - kb) : a.uJ[uo + (i - lc)];
-        };
-        auto getM = [&](uint32_t i) -> uint32_t {
-            return i < lc ? a.tval[so + i] : (uint32_t)a.uM[uo + (i - lc)];
-        };
-        const bool ok = encode_record(cnt, getJ, getM, win, a, t);
+        const AssembleSrc src(a, t);
+        const uint32_t cnt = src.count();
+        const bool noted = a.defer_long && cnt > kLongList;
+        if (noted && long_record(cnt, a, t) != kNoSeek) continue;
+        const bool ok = encode_record(
+            cnt, [&](uint32_t i) { return src.J(i); }, [&](uint32_t i) { return src.M(i); }, win, a, t, noted);
         uint32_t tiles = 0;
-        for (uint32_t i = lane; i < cnt; i += 32) tiles += __popc(getM(i));
+        for (uint32_t i = lane; i < cnt; i += 32) tiles += __popc(src.M(i));
         tiles = warp_sum(tiles);
         if (lane == 0) {
             if (!ok) {
@@ -716,6 +912,94 @@ __global__ void __launch_bounds__(SR_THREADS) k_assemble(SearchArgs a)
             }
         }
     }
+}
+
+// Long records, one warp per stretch of kSeek entries: the nibbles of its stream
+// (the seek point holds them and the index before the stretch for now).
+__global__ void __launch_bounds__(SR_THREADS) k_long_count(SearchArgs a, uint32_t n_seek)
+{
+    const uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (q >= n_seek || a.seek_of[q] == kNoSeek) return;
+    const uint2 l = a.long_list[a.seek_of[q]];
+    const AssembleSrc src(a, l.x);
+    const uint32_t beg = (q - l.y) * kSeek, end = min(src.count(), beg + kSeek);
+    const uint32_t prev = beg ? src.J(beg - 1u) : 0xffffffffu;
+    const uint32_t nib = a.compress ? stream_nibbles(beg, end, prev, [&](uint32_t i) { return src.J(i); }) : 0u;
+    if (lane_id() == 0) a.seek[q] = make_uint2(nib, prev);
+}
+
+// ... the record's place, the stretches' places in its stream, and zeros in the
+// words that stretches share (one warp per record).
+__global__ void __launch_bounds__(SR_THREADS) k_long_place(SearchArgs a, uint32_t n_long)
+{
+    const uint32_t li = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (li >= n_long) return;
+    const unsigned lane = lane_id();
+    const uint2 l = a.long_list[li];
+    if (l.y == kNoSeek) return;  // (encoded by the assembly)
+    const uint32_t cnt = AssembleSrc(a, l.x).count(), ns = (cnt + kSeek - 1u) / kSeek;
+    uint32_t nib = 0;
+    for (uint32_t k0 = 0; k0 < ns; k0 += 32) {
+        const uint32_t c = k0 + lane < ns ? a.seek[l.y + k0 + lane].x : 0u;
+        const uint32_t incl = warp_incl_scan(c);
+        if (k0 + lane < ns) a.seek[l.y + k0 + lane].x = nib + incl - c;
+        nib += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    const uint32_t mask_words = (cnt + 3u) >> 2, body_words = a.compress ? (nib + 7u) >> 3 : cnt;
+    uint32_t *rec = take_record(1u + mask_words + body_words, cnt, a, l.x);
+    if (!rec) {
+        if (lane == 0) {
+            atomicExch(&a.st->list_overflow, 1u);
+            a.rec_off[l.x] = kBadRecord;
+        }
+        return;
+    }
+    if (a.compress) {
+        uint32_t *body = rec + 1 + mask_words;
+        __syncwarp();
+        for (uint32_t k = lane; k < ns; k += 32) body[a.seek[l.y + k].x >> 3] = 0u;
+        if (lane == 0) body[body_words - 1u] = 0u;
+    }
+}
+
+// ... masks and stream of every stretch.
+__global__ void __launch_bounds__(SR_THREADS) k_long_put(SearchArgs a, uint32_t n_seek)
+{
+    __shared__ uint32_t wins[SR_WARPS][WIN_WORDS];
+    const uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (q >= n_seek || a.seek_of[q] == kNoSeek) return;
+    const unsigned lane = lane_id();
+    const uint2 l = a.long_list[a.seek_of[q]];
+    const uint32_t roff = a.rec_off[l.x];
+    if (roff == kBadRecord) return;  // (no room: the host grows the list and starts over)
+    const AssembleSrc src(a, l.x);
+    const uint32_t cnt = src.count(), beg = (q - l.y) * kSeek, end = min(cnt, beg + kSeek);
+    uint32_t *rec = reinterpret_cast<uint32_t *>(a.list) + roff;
+    auto getJ = [&](uint32_t i) { return src.J(i); };
+    put_masks(rec + 1, beg, end, [&](uint32_t i) { return src.M(i); });
+    uint32_t *body = rec + 1 + ((cnt + 3u) >> 2);
+    if (a.compress) {
+        const uint2 at = a.seek[q];
+        put_stream<true>(body, wins[threadIdx.x >> 5], beg, end, at.x, at.y, getJ, nullptr);
+    } else {
+        for (uint32_t t = beg + lane; t < end; t += 32) body[t] = getJ(t);
+    }
+    uint32_t tiles = 0;
+    for (uint32_t i = beg + lane; i < end; i += 32) tiles += __popc(src.M(i));
+    tiles = warp_sum(tiles);
+    if (lane == 0) {
+        atomicAdd(&a.st->n_entries, (unsigned long long)(end - beg));
+        atomicAdd(&a.st->n_tiles, (unsigned long long)tiles);
+    }
+}
+
+cudaError_t launch_assemble_long(const SearchArgs &a, uint32_t n_long, uint32_t n_seek, cudaStream_t s)
+{
+    if (!n_seek) return cudaSuccess;
+    k_long_count<<<(n_seek + SR_WARPS - 1) / SR_WARPS, SR_THREADS, 0, s>>>(a, n_seek);
+    k_long_place<<<(n_long + SR_WARPS - 1) / SR_WARPS, SR_THREADS, 0, s>>>(a, n_long);
+    k_long_put<<<(n_seek + SR_WARPS - 1) / SR_WARPS, SR_THREADS, 0, s>>>(a, n_seek);
+    return cudaGetLastError();
 }
 
 __global__ void k_classify(const uint32_t *__restrict__ list, uint32_t n, int M, SysTables t,
