@@ -28,6 +28,7 @@
 // instructions per super-cluster on the Evrard sphere at 2^21; search stage (half
 // lists, CUDA events) 1.18 -> 0.75 ms there, 15.9 -> 9.2 ms on 2^24 particles in
 // 64 Plummer spheres, 3.36 -> 2.20 ms on the 4M-particle fluid.
+#include <algorithm>
 #include <type_traits>
 
 #include "nl_internal.cuh"
@@ -239,11 +240,11 @@ __device__ bool encode_record(uint32_t cnt, GJ getJ, GM getM, uint32_t *win, con
 // them, so a group spans at most two 32-entry chunks and is carried over).
 // Returns false when a buffer was too small (the reservations still count,
 // so the host learns the sizes it needs).
-__device__ bool half_tuples(uint32_t cnt, const uint32_t *stJ, const uint8_t *stM, const SearchArgs &a,
-                            uint32_t s);
+template <class GJ, class GM>
+__device__ bool half_tuples(uint32_t cnt, GJ getJ, GM getM, const SearchArgs &a, uint32_t s);
 
-__device__ bool half_output(uint32_t cnt, const uint32_t *stJ, const uint8_t *stM,
-                            const SearchArgs &a, uint32_t s)
+template <class GJ, class GM>
+__device__ bool half_output(uint32_t cnt, GJ getJ, GM getM, const SearchArgs &a, uint32_t s)
 {
     const unsigned lane = lane_id();
     unsigned long long off = 0;
@@ -254,20 +255,20 @@ __device__ bool half_output(uint32_t cnt, const uint32_t *stJ, const uint8_t *st
         return false;
     }
     for (uint32_t t = lane; t < cnt; t += 32) {
-        a.uJ[off + t] = stJ[t];
-        a.uM[off + t] = stM[t];
+        a.uJ[off + t] = getJ(t);
+        a.uM[off + t] = (uint8_t)getM(t);
     }
     if (lane == 0) {
         a.up_off[s] = (uint32_t)off;
         a.up_cnt[s] = cnt;
     }
-    return half_tuples(cnt, stJ, stM, a, s);
+    return half_tuples(cnt, getJ, getM, a, s);
 }
 
 // The transposed tuples of entries of super-cluster s (all of one target
 // super-cluster together).
-__device__ bool half_tuples(uint32_t cnt, const uint32_t *stJ, const uint8_t *stM, const SearchArgs &a,
-                            uint32_t s)
+template <class GJ, class GM>
+__device__ bool half_tuples(uint32_t cnt, GJ getJ, GM getM, const SearchArgs &a, uint32_t s)
 {
     const unsigned lane = lane_id();
     constexpr uint32_t NONE = 0xffffffffu;
@@ -306,9 +307,9 @@ __device__ bool half_tuples(uint32_t cnt, const uint32_t *stJ, const uint8_t *st
     };
     for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
         const uint32_t e = b0 + lane;
-        const uint32_t J = e < cnt ? stJ[e] : 0u;
+        const uint32_t J = e < cnt ? getJ(e) : 0u;
         const bool valid = e < cnt && J >= own_end;
-        const uint32_t m = valid ? (uint32_t)stM[e] : 0u;
+        const uint32_t m = valid ? getM(e) : 0u;
         const uint32_t t = valid ? J / kSC : NONE;
         // a carried group that does not continue here is complete
         if (carry_t != NONE && __shfl_sync(0xffffffffu, t, 0) != carry_t) {
@@ -359,6 +360,16 @@ struct SearchSmem {
     uint32_t win[WIN_WORDS];
 };
 
+// Super-clusters shared by the warps of a block (SPLIT): per batch of
+// j-clusters, its first entry in the list and in the staging of the warp that
+// tested it.
+constexpr uint32_t kSplitBatches = 1024;
+struct SplitSmem {
+    uint16_t first[kSplitBatches + 1], src[kSplitBatches];
+    uint32_t ticket, cnt[SR_WARPS], tiles;
+    unsigned long long ttests;
+};
+
 // Could some particle of i-cluster box c (pair layout, half e) be a symmetric
 // neighbor of one in box B (b squared radius brr)?  The monotone gaps of
 // boxes_near.
@@ -399,9 +410,13 @@ __device__ __forceinline__ void box_pair_near(const float4 *ib, const float4 &bl
 // tuples for the record assembly.  MODE 2: half list (each pair stored once,
 // Sec. II-D): the half search's upper entries encoded as the record.  MODE 3:
 // mode 1 for the parts of heavy super-clusters (ctl.phase).
-template <int M, int MJ, bool PER, int MODE>
+// SPLIT: the warps of a block share a super-cluster, for systems with fewer of
+// them than the chip holds blocks: every warp walks the octree, the batches of
+// j-clusters go to the warps in turn, and the first warp encodes the list.
+template <int M, int MJ, bool PER, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCtl ctl)
 {
+    static_assert(!SPLIT || MODE != 3, "the parts of heavy super-clusters have a warp each");
     constexpr bool HALF = MODE != 0;  // only j-clusters from the own first one on
     constexpr uint32_t NB = sr_batch<MJ>();
     constexpr uint32_t G = 32 / M;        // tiles tested together, M lanes each
@@ -411,8 +426,11 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t slot = blockIdx.x * (blockDim.x >> 5) + warp;
     // a warp without staging room stays idle; the work counter hands its
-    // super-clusters to the others (warps never wait on each other here)
-    if (slot >= a.stage_slots) return;
+    // super-clusters to the others (warps wait on each other only in a block
+    // that shares super-clusters)
+    const uint32_t W = blockDim.x >> 5;
+    SplitSmem &B = *reinterpret_cast<SplitSmem *>(search_smem + W * sizeof(SearchSmem<M, MJ>));
+    if ((SPLIT ? (blockIdx.x + 1u) * W - 1u : slot) >= a.stage_slots) return;
     uint32_t *stJ = a.stageJ + (size_t)slot * a.stage_cap;
     uint8_t *stM = a.stageM + (size_t)slot * a.stage_cap;
     const uint32_t II = lane % M, grp = lane / M;
@@ -424,8 +442,19 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
 
     for (;;) {
         uint32_t tk = 0;
-        if (lane == 0) tk = atomicAdd(&a.st->ticket, 1u);
-        tk = __shfl_sync(0xffffffffu, tk, 0);
+        if constexpr (SPLIT) {
+            __syncthreads();  // (the last super-cluster is encoded)
+            if (threadIdx.x == 0) {
+                B.ticket = atomicAdd(&a.st->ticket, 1u);
+                B.tiles = 0u;
+                B.ttests = 0ull;
+            }
+            __syncthreads();
+            tk = B.ticket;
+        } else {
+            if (lane == 0) tk = atomicAdd(&a.st->ticket, 1u);
+            tk = __shfl_sync(0xffffffffu, tk, 0);
+        }
         if (tk >= count) break;
         const uint32_t wi = MODE == 3 ? tk / ctl.nparts : tk;
         const uint32_t s = ctl.work ? ctl.work[wi] : wi;
@@ -493,13 +522,23 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
 
         uint32_t cnt = 0, tiles = 0, nvis = 0, lvis = 0, jex = 0, ttests = 0;
         uint32_t qh = 0, qt = 0;  // queue of j-clusters, ring positions
-        bool aside = MODE == 1 && ctl.heavy != nullptr;  // may be set aside
+        bool aside = MODE == 1 && !SPLIT && ctl.heavy != nullptr;  // may be set aside
+        uint32_t nbatch = 0;                              // SPLIT: batches so far
         // the half search takes only j-clusters from its own first one on
         int lastJ = (int)(pbeg / MJ) - 1;
 
         // Test a batch of up to NB queued j-clusters.
         auto batch = [&]() {
             const uint32_t nq = min(NB, qt - qh);
+            if constexpr (SPLIT) {
+                const uint32_t b = nbatch++;
+                if (b % W != warp) {  // another warp's
+                    qh += nq;
+                    return;
+                }
+                if (lane == 0) B.src[b] = (uint16_t)cnt;
+            }
+            const uint32_t cnt0 = cnt;
             // 1. box tests, one j-cluster per lane against the 8 i-clusters
             const uint32_t J = lane < nq ? S.jq[(qh + lane) & 63u] : 0u;
             uint32_t cm = 0;
@@ -599,6 +638,7 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 ttests += T;
                 __syncwarp();
             }
+            if (SPLIT && lane == 0) B.first[nbatch] = (uint16_t)(cnt - cnt0);
             qh += nq;
         };
 
@@ -664,7 +704,8 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 leaves = __ballot_sync(0xffffffffu, near && skip == u + 1u);
                 nvis += min(32u, vend - v);
                 // (also when few of the j-clusters reached by boxes hold a pair)
-                loose = loose || jex > kLooseMin + kLooseRate * cnt;
+                // (not where warps share it: all must form the same batches)
+                loose = loose || (!SPLIT && jex > kLooseMin + kLooseRate * cnt);
                 if (loose) {
                     // particles against the leaves and the nodes reaching beyond the chunk
                     const uint32_t big = __ballot_sync(0xffffffffu, near && skip > v + 32u);
@@ -714,10 +755,52 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
         }
         __syncwarp();
         if (MODE == 1 && aside && cnt > kLongSearch) continue;
+        bool staged = cnt <= a.stage_cap;
+        if constexpr (SPLIT) {
+            // the batches' places in the list; the first warp goes on with it
+            tiles = warp_sum(tiles);
+            if (lane == 0) {
+                B.cnt[warp] = cnt;
+                atomicAdd(&B.tiles, tiles);
+                atomicAdd(&B.ttests, (unsigned long long)ttests);
+            }
+            __syncthreads();
+            if (warp != 0) continue;
+            cnt = 0;
+            for (uint32_t w = 0; w < W; ++w) {
+                cnt += B.cnt[w];
+                staged = staged && B.cnt[w] <= a.stage_cap;
+            }
+            staged = staged && cnt <= a.stage_cap;
+            uint32_t at = 0;
+            for (uint32_t b0 = 0; b0 < nbatch; b0 += 32) {
+                const uint32_t c = b0 + lane < nbatch ? B.first[b0 + lane + 1] : 0u;
+                const uint32_t incl = warp_incl_scan(c);
+                if (b0 + lane < nbatch) B.first[b0 + lane + 1] = (uint16_t)(at + incl);
+                at += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) B.first[0] = 0;
+            __syncwarp();
+            tiles = lane == 0 ? B.tiles : 0u;
+            ttests = (uint32_t)B.ttests;
+        }
+        // entry t: in the staging of the warp of its batch
+        auto place = [&](uint32_t t) -> size_t {
+            if constexpr (!SPLIT) return t;
+            uint32_t lo = 0, hi = nbatch;  // first[lo] <= t < first[hi]
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (B.first[mid] <= t) lo = mid;
+                else hi = mid;
+            }
+            return (size_t)(lo % W) * a.stage_cap + B.src[lo] + (t - B.first[lo]);
+        };
+        auto getJ = [&](uint32_t t) { return stJ[place(t)]; };
+        auto getM = [&](uint32_t t) { return (uint32_t)stM[place(t)]; };
         if constexpr (MODE == 3) {
             if (ctl.phase == 1) {
                 if (lane == 0) a.hpart[tk] = cnt;
-            } else if (!half_tuples(cnt, stJ, stM, a, s) && lane == 0) {
+            } else if (!half_tuples(cnt, getJ, getM, a, s) && lane == 0) {
                 atomicExch(&a.st->half_overflow, 1u);
             }
             if (lane == 0 && ctl.phase == 2) {
@@ -729,17 +812,14 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
             continue;
         }
         tiles = warp_sum(tiles);
-        const bool staged = cnt <= a.stage_cap;
         bool ok = staged;
         if (!staged) {
             if (lane == 0) atomicMax(&a.st->max_count, cnt);
         } else if constexpr (MODE == 1) {
             // a buffer overflow here makes the host re-run every super-cluster
-            ok = half_output(cnt, stJ, stM, a, s);
+            ok = half_output(cnt, getJ, getM, a, s);
         } else {
-            ok = encode_record(
-                cnt, [&](uint32_t t) { return stJ[t]; },
-                [&](uint32_t t) { return (uint32_t)stM[t]; }, S.win, a, s);
+            ok = encode_record(cnt, getJ, getM, S.win, a, s);
             if (!ok && lane == 0) atomicExch(&a.st->list_overflow, 1u);
         }
         if (lane == 0) {
@@ -761,21 +841,33 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
     }
 }
 
-template <int M, int MJ, int MODE>
+template <int M, int MJ, int MODE, bool SPLIT = false>
 static cudaError_t launch_m(const SearchArgs &a, const SearchCtl &c, int per, int grid, int threads,
                             cudaStream_t s)
 {
-    const size_t smem = (size_t)(threads / 32) * sizeof(SearchSmem<M, MJ>);
-    const size_t smax = (size_t)SR_WARPS * sizeof(SearchSmem<M, MJ>);
-    const void *fn = per ? (const void *)k_search<M, MJ, true, MODE>
-                         : (const void *)k_search<M, MJ, false, MODE>;
-    cudaError_t e = set_max_dynamic_smem(fn, smax);
+    const size_t extra = SPLIT ? sizeof(SplitSmem) : 0;
+    auto *fn = per ? k_search<M, MJ, true, MODE, SPLIT> : k_search<M, MJ, false, MODE, SPLIT>;
+    cudaError_t e = set_max_dynamic_smem((const void *)fn, (size_t)SR_WARPS * sizeof(SearchSmem<M, MJ>) + extra);
     if (e != cudaSuccess) return e;
-    if (per)
-        k_search<M, MJ, true, MODE><<<grid, threads, smem, s>>>(a, c);
-    else
-        k_search<M, MJ, false, MODE><<<grid, threads, smem, s>>>(a, c);
+    fn<<<grid, threads, (size_t)(threads / 32) * sizeof(SearchSmem<M, MJ>) + extra, s>>>(a, c);
     return cudaGetLastError();
+}
+
+// The warps of a block share a super-cluster when there are at most three of
+// them per resident block, unless their lists may hold more batches or entries
+// than the block's tables.  Search of an Evrard sphere (half / full lists, ms, a
+// warp each -> shared): 512 super-clusters 0.118 / 0.138 -> 0.066 / 0.078, 1216
+// 0.134 / 0.145 -> 0.091 / 0.117, 1875 0.141 / 0.153 -> 0.118 / 0.155, 2422 0.149 /
+// 0.160 -> 0.148 / 0.197; periodic cubes of 4096 and 32768 particles 0.34 -> 0.14,
+// 0.43 -> 0.18.
+template <int M, int MJ, int MODE>
+static cudaError_t launch_split(const SearchArgs &a, const SearchCtl &c, int per, int grid, int threads,
+                                cudaStream_t s)
+{
+    const uint64_t batches = ((uint64_t)a.nsc * kSC * (M / MJ)) / sr_batch<MJ>() + 2;
+        if (a.nsc <= 3u * (uint32_t)grid && batches <= kSplitBatches && a.stage_cap < 65536u / SR_WARPS)
+        return launch_m<M, MJ, MODE, true>(a, c, per, (int)std::min<uint32_t>(c.count, (uint32_t)grid), threads, s);
+    return launch_m<M, MJ, MODE>(a, c, per, grid, threads, s);
 }
 
 cudaError_t launch_search_ctl(const SearchArgs &a, const uint32_t *work, uint32_t count,
@@ -787,23 +879,27 @@ cudaError_t launch_search_ctl(const SearchArgs &a, const uint32_t *work, uint32_
     if (threads != 128 && threads != SR_THREADS) return cudaErrorInvalidValue;
     if (a.half && a.mj != M) return cudaErrorInvalidValue;  // needs j-clusters = i-clusters
     if (a.half < 0 || a.half > 2) return cudaErrorInvalidValue;
+    if (count == 0) return cudaSuccess;
+#define NL_SEARCH(M_, MJ_, MODE_) \
+    return launch_split<M_, MJ_, MODE_>(a, c, any_periodic, grid, threads, s)
     switch (M * 100 + a.mj) {
     case 404:
-        if (a.half == 1) return launch_m<4, 4, 1>(a, c, any_periodic, grid, threads, s);
-        if (a.half == 2) return launch_m<4, 4, 2>(a, c, any_periodic, grid, threads, s);
-        return launch_m<4, 4, 0>(a, c, any_periodic, grid, threads, s);
+        if (a.half == 1) NL_SEARCH(4, 4, 1);
+        if (a.half == 2) NL_SEARCH(4, 4, 2);
+        NL_SEARCH(4, 4, 0);
     case 808:
-        if (a.half == 1) return launch_m<8, 8, 1>(a, c, any_periodic, grid, threads, s);
-        if (a.half == 2) return launch_m<8, 8, 2>(a, c, any_periodic, grid, threads, s);
-        return launch_m<8, 8, 0>(a, c, any_periodic, grid, threads, s);
-    case 804: return launch_m<8, 4, 0>(a, c, any_periodic, grid, threads, s);
+        if (a.half == 1) NL_SEARCH(8, 8, 1);
+        if (a.half == 2) NL_SEARCH(8, 8, 2);
+        NL_SEARCH(8, 8, 0);
+    case 804: NL_SEARCH(8, 4, 0);
     case 1616:
-        if (a.half == 1) return launch_m<16, 16, 1>(a, c, any_periodic, grid, threads, s);
-        if (a.half == 2) return launch_m<16, 16, 2>(a, c, any_periodic, grid, threads, s);
-        return launch_m<16, 16, 0>(a, c, any_periodic, grid, threads, s);
-    case 1608: return launch_m<16, 8, 0>(a, c, any_periodic, grid, threads, s);
+        if (a.half == 1) NL_SEARCH(16, 16, 1);
+        if (a.half == 2) NL_SEARCH(16, 16, 2);
+        NL_SEARCH(16, 16, 0);
+    case 1608: NL_SEARCH(16, 8, 0);
     default: return cudaErrorInvalidValue;
     }
+#undef NL_SEARCH
 }
 
 // Upper entries of a heavy super-cluster from the counts of its parts: one
