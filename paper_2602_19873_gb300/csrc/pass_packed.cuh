@@ -3,16 +3,23 @@
 //
 // A warp owns a super-cluster, decodes 32 list entries at a time and stages
 // the j particles of PK_SE of them in shared memory, two j particles of a
-// cluster in each word: (x, x', y, y').  Then it takes the i-clusters in turn:
-// a lane holds one i particle (lane % M), duplicated into packed registers once
-// per stage, and walks the staged entries that list the i-cluster; every step of
-// the pair arithmetic is one f32x2 instruction for the lane's two j particles.
-// With the i-clusters outside and the entries inside, the sums of one i particle
-// are all the registers a lane needs (the sums of 8 i-clusters held at once, with
-// the entries outside, took 126 registers on the force passes), there is one copy
-// of the pair code, and no instruction is spent on i-clusters that an entry does
-// not list.  On half lists the shares of the j particles wait in shared memory,
-// one word per lane and entry, and are summed and added to memory once a stage.
+// cluster in each word: (x, x', y, y').  Then it takes the i-clusters two at a
+// time: a lane holds one i particle (lane % M) of each, duplicated into packed
+// registers once per stage, and walks the staged entries that list them; every
+// step of the pair arithmetic is one f32x2 instruction for the lane's two j
+// particles.  With the i-clusters outside and the entries inside, the sums of two
+// i particles are all the registers a lane needs (the sums of 8 i-clusters held at
+// once, with the entries outside, took 126 registers on the force passes), and no
+// instruction is spent on i-clusters that an entry does not list.  On half lists
+// the shares of the j particles wait in shared memory, one word per lane and
+// entry, and are summed and added to memory once a stage.  Neighboring i-clusters
+// share two thirds of their entries: such an entry's j words and j shares are read
+// and written once for two tiles, and the two tiles' chains overlap.  (One
+// i-cluster at a time left the half-list force passes bound by shared memory, 12 of
+// 18 wavefronts per tile carrying the j shares: LJ at 4M particles 4.28 -> 3.8 ms,
+// LJ + Coulomb 3.73 -> 3.19, density and pressure of the 2^21-particle Evrard
+// sphere 1.51 -> 1.26 each; evaluating every entry for both would have cost 18 %
+// in pairs that are not listed.)
 //
 // The pair terms have no branches.  Kernels that vanish with the distance
 // (density, pressure force) need no range test at all: with s = 1 - q/2 clamped
@@ -21,21 +28,23 @@
 // The others decide with the canonical FP32 predicate and select their
 // coefficient.
 //
-// A scalar form of the terms runs for single entries: those whose pairs may wrap
-// around a periodic face, those holding the self pair where it has to be left
-// out, and all entries when an input is not finite (a status word of the gather
-// kernel).
+// Entries with pairs across a periodic face (an eighth of the tiles of LJ at 4M
+// particles) take the packed terms with the pair vector wrapped, one i-cluster at
+// a time.  A scalar form of the terms is left for tiles that hold self pairs which
+// have to be left out, and for all of them when an input is not finite (a status
+// word of the gather kernel).  (All entries of the own j-clusters and all wrapped
+// ones in the scalar form: LJ at 4M 3.8 ms instead of 3.39.)
 //
-// What bounds it: the half-list density pass issues 62 warp instructions per listed
-// 8x8 tile (the scalar kernel: 96), 37 of them the pair terms, with the FMA pipe 56 %
-// and the shared-memory pipe 71 % busy; the half-list force passes are bound by
-// shared-memory bandwidth (89 %: 12 of 18 wavefronts per tile carry the j shares).
+// What bounds it: instruction issue.  The half-list density pass issues 0.69, the
+// force passes 0.62 to 0.65 instructions per scheduler and cycle, with the FMA pipe
+// 60 % (LJ 31 %) and the shared-memory pipe 46 to 64 % (LJ 29 %) busy; what is left is
+// the wait for fixed latencies at 24 to 32 warps per SM, as many as the registers allow.
 // Pass stage, scalar kernel -> this one (CUDA events): half-list density on 2^24
-// particles 9.10 -> 7.15 ms, pressure force on the 2^21-particle Evrard sphere 2.85
-// -> 1.51, LJ at 4M particles 6.92 -> 4.28, LJ + Coulomb 4.83 -> 3.73; full lists:
-// density and nearest distance on 2M particles 1.38 -> 1.13, pressure force on 300k
-// 0.69 -> 0.30; small systems (split): density of 32k particles 0.48 -> 0.10 ms, of
-// 4096 0.32 -> 0.06 ms.
+// particles 9.10 -> 6.77 ms, pressure force on the 2^21-particle Evrard sphere 2.85
+// -> 1.26, LJ at 4M particles 6.92 -> 3.39, LJ + Coulomb 4.83 -> 2.79; full lists:
+// density and nearest distance on 2M particles 1.38 -> 1.03, pressure force on 300k
+// 0.69 -> 0.29; small systems (split): density of 32k particles 0.48 -> 0.09 ms, of
+// 4096 0.32 -> 0.05 ms.
 //
 // split: W warps of a block share a super-cluster, each working on every W-th
 // stage.  Small systems have fewer super-clusters than the chip has warp slots,
@@ -43,6 +52,8 @@
 // kLongList entries (skip_longer, longs) get a launch of their own in which whole
 // blocks, several of them where sums can meet in memory, share one list.
 #pragma once
+#include <type_traits>
+
 #include "nl_internal.cuh"
 #include "pass_decode.cuh"
 
@@ -167,13 +178,26 @@ struct PkSmem {
 };
 
 // Resident blocks of 256 threads the register budget is cut for (half-list
-// density at 2^24 particles with 3 / 4 / 5: 7.38 / 7.01 / 7.58 ms; half-list LJ at
-// 4M with 2 / 3: 4.77 / 4.35 ms, with 4 its registers spill).
+// density at 2^24 particles with 3 / 4: 6.99 / 6.77 ms; half-list LJ at 4M with
+// 2 / 3: 3.56 / 3.39 ms, LJ + Coulomb 2.93 / 2.79, pressure force the same).
 template <int KIND, bool HL>
 constexpr int pk_min_blocks()
 {
     return (KIND == PASS_SPH || KIND == PASS_LJ || KIND == PASS_LJC) ? 3 : 4;
 }
+
+// One i particle, duplicated into packed registers: position, a as in PkSmem::ia,
+// hp = +-a, and its pass inputs u, v.
+template <int KIND>
+struct IPart {
+    f32x2 x, y, z, hp, u, v;
+    float a;
+};
+// Sums of one i particle over a stage: (x, y, z), count or minimum.
+struct ISum {
+    f32x2 x, y, z;
+    uint32_t c;
+};
 
 // v += b with the running compensation c (Kahan)
 __device__ __forceinline__ void kahan_add(float &v, float &c, float b)
@@ -220,13 +244,222 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
     // running sums take one partial a stage.  Density and pressure (whose sums
     // cancel) compensated: plain adds left the pressure force of the Evrard
     // sphere 10 % further from FP64 than the scalar kernel, 3 % less time.  Lennard-
-    // Jones sums are ruled by their nearest pairs: plain adds are as near, and 4 %
-    // faster at 4M particles.
+    // Jones alone too (median error at 4M particles 3.60e-7 plain, 3.55e-7
+    // compensated, scalar kernel 3.57e-7; 4 % of the time); with Coulomb terms plain
+    // sums are as near as the scalar kernel's (4.73e-7).
     auto sum_add = [](float &v, float &c, float b) {
-        if constexpr (KIND == PASS_DENSITY || KIND == PASS_SPH) kahan_add(v, c, b);
+        if constexpr (KIND == PASS_DENSITY || KIND == PASS_SPH || KIND == PASS_LJ) kahan_add(v, c, b);
         else v += b;
     };
     auto merge = [](uint32_t u, uint32_t v) { return KIND == PASS_COUNT ? u + v : min(u, v); };
+
+    constexpr uint32_t JS = SE * NT * 32;  // j shares: between components
+
+    // own particle II of i-cluster k
+    auto own_part = [&](uint32_t k) {
+        const float4 p = S.ia[k * M + II];
+        IPart<KIND> I;
+        I.x = dup2(p.x);
+        I.y = dup2(p.y);
+        I.z = dup2(p.z);
+        I.a = p.w;
+        if constexpr (KIND == PASS_DENSITY) I.hp = dup2(-p.w);  // 1/(2h)
+        if constexpr (KIND == PASS_SPH) I.hp = dup2(p.w);
+        if constexpr (Smem::IB) {
+            const float2 v = S.ib[k * M + II];
+            I.u = dup2(v.x);
+            I.v = dup2(v.y);
+        }
+        return I;
+    };
+    // the lane's pair tt of staged entry el, with its shares
+    struct JPart {
+        float4 A, B, C;
+        f32x2 x, y, z;
+    };
+    auto load_j = [&](uint32_t el, uint32_t tt) {
+        const uint32_t q = el * HJ + g + tt * G;
+        JPart j;
+        j.A = S.ja[q];
+        j.B = S.jb[q];
+        if constexpr (Smem::JC) j.C = S.jc[q];
+        if constexpr (HL) {
+            const f32x2 *js = S.js + (el * NT + tt) * 32 + lane;
+            j.x = js[0];
+            if constexpr (FORCE) {
+                j.y = js[JS];
+                j.z = js[2 * JS];
+            }
+        }
+        return j;
+    };
+    auto store_j = [&](uint32_t el, uint32_t tt, const JPart &j) {
+        if constexpr (HL) {
+            f32x2 *js = S.js + (el * NT + tt) * 32 + lane;
+            js[0] = j.x;
+            if constexpr (FORCE) {
+                js[JS] = j.y;
+                js[2 * JS] = j.z;
+            }
+        }
+    };
+    // the terms of one i particle and the lane's two j particles; wrap: pairs
+    // may lie across a periodic face
+    auto terms = [&](const IPart<KIND> &I, JPart &j, ISum &T, auto wrap, const PerLen &box) {
+        constexpr bool WR = decltype(wrap)::value;
+        const float4 &A = j.A, &B = j.B, &C = j.C;
+        f32x2 dx = sub2_rn(pk2(A.x, A.y), I.x), dy = sub2_rn(pk2(A.z, A.w), I.y);
+        f32x2 dz = sub2_rn(pk2(B.x, B.y), I.z);
+        float w0, w1;  // the canonical squared distances of such pairs
+        if constexpr (WR) {
+            float ix, iy, iz, u;
+            unpk2(I.x, ix, u);
+            unpk2(I.y, iy, u);
+            unpk2(I.z, iz, u);
+            if constexpr (KIND != PASS_DENSITY && KIND != PASS_SPH)
+                pair_d2_x2<true>(pk2(A.x, A.y), pk2(A.z, A.w), pk2(B.x, B.y), I.x, I.y, I.z, box, w0, w1);
+            const float4 pi = make_float4(ix, iy, iz, 0.f);
+            const float3 v0 = pair_dx_acc<true>(pi, make_float4(A.x, A.z, B.x, 0.f), box);
+            const float3 v1 = pair_dx_acc<true>(pi, make_float4(A.y, A.w, B.y, 0.f), box);
+            dx = pk2(v0.x, v1.x);
+            dy = pk2(v0.y, v1.y);
+            dz = pk2(v0.z, v1.z);
+        }
+        float d0, d1;
+        if constexpr (KIND == PASS_DENSITY) {
+            unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, mul2_rn(dx, dx))), d0, d1);
+            const float r0 = sqrt_ftz(d0), r1 = sqrt_ftz(d1);
+            const f32x2 r = pk2(r0, r1);
+            T.x = fma2_rn(pk2(B.z, B.w), spline_half_w2(sat_fma1(r0, I.a), sat_fma1(r1, I.a), mul2_rn(r, I.hp)), T.x);
+            if constexpr (HL)
+                j.x = fma2_rn(I.u, spline_half_w2(sat_fma1(r0, C.x), sat_fma1(r1, C.y), mul2_rn(r, pk2(C.z, C.w))), j.x);
+        } else if constexpr (KIND == PASS_SPH) {
+            // (a self pair: dx = 0; the floor keeps 1/r finite)
+            unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, mul2_rn(dx, dx))), d0, d1);
+            d0 = fmaxf(d0, 1e-30f);
+            d1 = fmaxf(d1, 1e-30f);
+            const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
+            const f32x2 r = mul2_rn(pk2(d0, d1), ir);
+            float r0, r1;
+            unpk2(r, r0, r1);
+            const f32x2 gi = spline_third_dw2(sat_fma1(r0, I.a), sat_fma1(r1, I.a), mul2_rn(r, I.hp));
+            const f32x2 gj = spline_third_dw2(sat_fma1(r0, B.z), sat_fma1(r1, B.w), mul2_rn(r, pk2(B.z, B.w)));
+            const f32x2 b = mul2_rn(fma2_rn(pk2(C.x, C.y), gj, mul2_rn(I.u, gi)), ir);
+            const f32x2 si = mul2_rn(pk2(C.z, C.w), b);
+            T.x = fma2_rn(si, dx, T.x);
+            T.y = fma2_rn(si, dy, T.y);
+            T.z = fma2_rn(si, dz, T.z);
+            if constexpr (HL) {
+                const f32x2 sj = mul2_rn(I.v, b);
+                j.x = fma2_rn(sj, dx, j.x);
+                j.y = fma2_rn(sj, dy, j.y);
+                j.z = fma2_rn(sj, dz, j.z);
+            }
+        } else {
+            sum_sq_x2(dx, dy, dz, d0, d1);
+            if constexpr (!WR) {  // these are the canonical ones
+                w0 = d0;
+                w1 = d1;
+            }
+            const bool i0 = w0 < I.a, i1 = w1 < I.a;
+            [[maybe_unused]] const bool j0 = HL && w0 < B.z, j1 = HL && w1 < B.w;
+            if constexpr (KIND == PASS_COUNT) {
+                T.c += (i0 ? 1u : 0u) + (i1 ? 1u : 0u);
+                if constexpr (HL) j.x += (j0 ? 1ull : 0ull) + (j1 ? 1ull << 32 : 0ull);
+            } else if constexpr (KIND == PASS_MIN) {
+                const uint32_t u0 = __float_as_uint(d0), u1 = __float_as_uint(d1);
+                if (i0) T.c = min(T.c, u0);
+                if (i1) T.c = min(T.c, u1);
+                if constexpr (HL) {
+                    const uint32_t l = j0 ? min((uint32_t)j.x, u0) : (uint32_t)j.x;
+                    const uint32_t h = j1 ? min((uint32_t)(j.x >> 32), u1) : (uint32_t)(j.x >> 32);
+                    j.x = ((f32x2)h << 32) | l;
+                }
+            } else {
+                // f: minus the coefficient of dx in the force on j
+                float f0, f1;
+                if constexpr (KIND == PASS_LJ) {
+                    // -1/d2 by the hardware reciprocal and one Newton step
+                    const f32x2 r = pk2(rcp_ftz(-d0), rcp_ftz(-d1));
+                    const f32x2 e = fma2_rn(pk2(d0, d1), r, dup2(1.f));
+                    const f32x2 s2 = mul2_rn(dup2(sig2), fma2_rn(r, e, r));
+                    const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);  // -(sigma/r)^6
+                    unpk2(mul2_rn(s2, fma2_rn(add2_rn(s6, s6), s6, s6)), f0, f1);
+                } else {
+                    const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
+                    const f32x2 ir2 = mul2_rn(ir, ir);
+                    const f32x2 s2 = mul2_rn(dup2(-sig2), ir2);
+                    const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);
+                    const f32x2 lj = mul2_rn(dup2(e24), fma2_rn(add2_rn(s6, s6), s6, s6));
+                    const f32x2 qq = mul2_rn(I.u, pk2(C.x, C.y));
+                    float t0, t1;
+                    unpk2(mul2_rn(ir2, fma2_rn(qq, ir, lj)), t0, t1);
+                    f0 = -t0;
+                    f1 = -t1;
+                }
+                // (padding particles are far away: never in range, dx finite)
+                const f32x2 fi = pk2(i0 ? f0 : 0.f, i1 ? f1 : 0.f);
+                T.x = fma2_rn(fi, dx, T.x);
+                T.y = fma2_rn(fi, dy, T.y);
+                T.z = fma2_rn(fi, dz, T.z);
+                if constexpr (HL) {
+                    const f32x2 fj = pk2(j0 ? f0 : 0.f, j1 ? f1 : 0.f);
+                    j.x = fma2_rn(fj, dx, j.x);
+                    j.y = fma2_rn(fj, dy, j.y);
+                    j.z = fma2_rn(fj, dz, j.z);
+                }
+            }
+        }
+    };
+
+    // running sums of particle II of the i-clusters cluster_of(q)
+    float rx[NK], ry[NK], rz[NK];  // (density: x alone; count, nearest: rc)
+    float cx[NK], cy[NK], cz[NK];  // their compensations
+    uint32_t rc[NK];
+    // lane group g keeps, of the pairs of i-clusters (2p, 2p + 1) with p = g mod
+    // G/2, the first (g < G/2) or the second
+    auto cluster_of = [&](uint32_t q) { return 2u * (q * (G / 2) + g % (G / 2)) + g / (G / 2); };
+    // a stage's sums of i-clusters k, k + 1 over the lanes of the same particle,
+    // then to the lanes that keep them
+    auto keep = [&](uint32_t k, const ISum &A0, const ISum &A1) {
+        const bool up = lane & 16u;  // g >= G/2
+        const uint32_t p = k >> 1, mq = p / (G / 2);
+        const bool mine = p % (G / 2) == g % (G / 2);
+        if constexpr (INTS) {
+            uint32_t v = merge(up ? A1.c : A0.c, __shfl_xor_sync(0xffffffffu, up ? A0.c : A1.c, 16));
+#pragma unroll
+            for (int o = M; o < 16; o <<= 1) v = merge(v, __shfl_xor_sync(0xffffffffu, v, o));
+#pragma unroll
+            for (uint32_t q = 0; q < NK; ++q)
+                if (mine && mq == q) rc[q] = merge(rc[q], v);
+        } else {
+            auto fold = [&](f32x2 a0, f32x2 a1) {
+                float l0, h0, l1, h1;
+                unpk2(a0, l0, h0);
+                unpk2(a1, l1, h1);
+                const float s0 = l0 + h0, s1 = l1 + h1;
+                float v = (up ? s1 : s0) + __shfl_xor_sync(0xffffffffu, up ? s0 : s1, 16);
+#pragma unroll
+                for (int o = M; o < 16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                return v;
+            };
+            const float x = fold(A0.x, A1.x);
+            float y = 0.f, z = 0.f;
+            if constexpr (FORCE) {
+                y = fold(A0.y, A1.y);
+                z = fold(A0.z, A1.z);
+            }
+#pragma unroll
+            for (uint32_t q = 0; q < NK; ++q)
+                if (mine && mq == q) {
+                    sum_add(rx[q], cx[q], x);
+                    if constexpr (FORCE) {
+                        sum_add(ry[q], cy[q], y);
+                        sum_add(rz[q], cz[q], z);
+                    }
+                }
+        }
+    };
 
     const uint32_t nwork = a.work || LONG ? (a.nwork_dev ? min(a.nwork, *a.nwork_dev) : a.nwork) : a.nsc;
     for (uint32_t it = blockIdx.x + gridDim.x * grp;; it += gridDim.x * ngrp) {
@@ -316,10 +549,6 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
         }
         __syncwarp();
 
-        // running sums of the i-clusters g NK .. g NK + NK - 1, particle II
-        // (density: x alone; count, nearest: rc) with their compensations
-        float rx[NK], ry[NK], rz[NK], cx[NK], cy[NK], cz[NK];
-        uint32_t rc[NK];
 #pragma unroll
         for (uint32_t q = 0; q < NK; ++q) {
             rx[q] = ry[q] = rz[q] = cx[q] = cy[q] = cz[q] = 0.f;
@@ -355,7 +584,6 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                 const uint32_t ns = min(SE, cnt - b0 - c);
                 // stage the j particles of entries c .. c + ns - 1
                 uint32_t slow = careful ? 0xffffffffu : 0u;  // bit el: entry c + el takes the scalar terms
-                if constexpr (NO_SELF) slow |= own >> c;
                 __syncwarp();
 #pragma unroll
                 for (uint32_t q0 = 0; q0 < (uint32_t)Smem::NP; q0 += 32) {
@@ -417,236 +645,162 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                 }
                 __syncwarp();
 
+                // i-clusters k and k + 1 together: entries that list both (about
+                // two thirds of those that list one) read their j words, and keep
+                // their j shares in registers, once for two tiles
+                const uint32_t staged = (1u << SE) - 1u;
+                // entries that list i-cluster k and hold its own particles: their
+                // self pairs take the scalar terms
+                const uint32_t owns = NO_SELF ? (own >> c) & staged : 0u;
+                auto diag = [&](uint32_t k) {
+                    return owns ? __ballot_sync(0xffffffffu, valid && rel / RJ == k) >> c : 0u;
+                };
 #pragma unroll 1
-                for (uint32_t k = 0; k < kSC; ++k) {
-                    // staged entries that list i-cluster k
-                    uint32_t bits = (__ballot_sync(0xffffffffu, (mk >> k) & 1u) >> c) & ((1u << SE) - 1u);
-                    if (!bits) continue;
-                    const float4 pi = S.ia[k * M + II];
-                    float2 iv = make_float2(0.f, 0.f);
-                    if constexpr (Smem::IB) iv = S.ib[k * M + II];
-                    const f32x2 xi = dup2(pi.x), yi = dup2(pi.y), zi = dup2(pi.z);
-                    const f32x2 hpi = dup2(KIND == PASS_DENSITY ? -pi.w : pi.w);  // 1/(2h), pressure -1/(2h)
-                    const f32x2 ivx = dup2(iv.x), ivy = dup2(iv.y);
-                    f32x2 ax = 0ull, ay = 0ull, az = 0ull;  // the i particle's sums over this stage
-                    uint32_t ac = NONE;
-                    for (uint32_t todo = bits & ~slow; todo; todo &= todo - 1u) {
+                for (uint32_t k = 0; k < kSC; k += 2) {
+                    const uint32_t b0w = (__ballot_sync(0xffffffffu, (mk >> k) & 1u) >> c) & staged & ~(slow | diag(k));
+                    const uint32_t b1w = (__ballot_sync(0xffffffffu, (mk >> k) & 2u) >> c) & staged & ~(slow | diag(k + 1u));
+                    if (!(b0w | b1w)) continue;
+                    const IPart<KIND> I0 = own_part(k), I1 = own_part(k + 1);
+                    ISum A0{0ull, 0ull, 0ull, NONE}, A1 = A0;
+                    for (uint32_t todo = b0w & b1w; todo; todo &= todo - 1u) {
                         const uint32_t el = __ffs(todo) - 1;
 #pragma unroll
                         for (uint32_t tt = 0; tt < NT; ++tt) {
-                            const uint32_t q = el * HJ + g + tt * G;
-                            f32x2 *js = S.js + (el * NT + tt) * 32 + lane;
-                            constexpr uint32_t JS = SE * NT * 32;  // between components
-                            const float4 A = S.ja[q], B = S.jb[q];
-                            const f32x2 dx = sub2_rn(pk2(A.x, A.y), xi), dy = sub2_rn(pk2(A.z, A.w), yi);
-                            const f32x2 dz = sub2_rn(pk2(B.x, B.y), zi);
-                            if constexpr (KIND == PASS_DENSITY) {
-                                float d0, d1;
-                                unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, mul2_rn(dx, dx))), d0, d1);
-                                const float r0 = sqrt_ftz(d0), r1 = sqrt_ftz(d1);
-                                const f32x2 r = pk2(r0, r1);
-                                ax = fma2_rn(pk2(B.z, B.w),
-                                             spline_half_w2(sat_fma1(r0, pi.w), sat_fma1(r1, pi.w), mul2_rn(r, hpi)), ax);
-                                if constexpr (HL) {
-                                    const float4 C = S.jc[q];
-                                    *js = fma2_rn(ivx,
-                                                  spline_half_w2(sat_fma1(r0, C.x), sat_fma1(r1, C.y),
-                                                                 mul2_rn(r, pk2(C.z, C.w))), *js);
-                                }
-                            } else if constexpr (KIND == PASS_SPH) {
-                                // (a self pair: dx = 0; the floor keeps 1/r finite)
-                                float d0, d1;
-                                unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, mul2_rn(dx, dx))), d0, d1);
-                                d0 = fmaxf(d0, 1e-30f);
-                                d1 = fmaxf(d1, 1e-30f);
-                                const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
-                                const f32x2 r = mul2_rn(pk2(d0, d1), ir);
-                                float r0, r1;
-                                unpk2(r, r0, r1);
-                                const float4 C = S.jc[q];
-                                const f32x2 gi = spline_third_dw2(sat_fma1(r0, pi.w), sat_fma1(r1, pi.w), mul2_rn(r, hpi));
-                                const f32x2 gj = spline_third_dw2(sat_fma1(r0, B.z), sat_fma1(r1, B.w), mul2_rn(r, pk2(B.z, B.w)));
-                                const f32x2 b = mul2_rn(fma2_rn(pk2(C.x, C.y), gj, mul2_rn(ivx, gi)), ir);
-                                const f32x2 si = mul2_rn(pk2(C.z, C.w), b);
-                                ax = fma2_rn(si, dx, ax);
-                                ay = fma2_rn(si, dy, ay);
-                                az = fma2_rn(si, dz, az);
-                                if constexpr (HL) {
-                                    const f32x2 sj = mul2_rn(ivy, b);
-                                    js[0] = fma2_rn(sj, dx, js[0]);
-                                    js[JS] = fma2_rn(sj, dy, js[JS]);
-                                    js[2 * JS] = fma2_rn(sj, dz, js[2 * JS]);
-                                }
-                            } else {
-                                float d0, d1;  // the canonical squared distances
-                                sum_sq_x2(dx, dy, dz, d0, d1);
-                                const bool i0 = d0 < pi.w, i1 = d1 < pi.w;
-                                const bool j0 = d0 < B.z, j1 = d1 < B.w;
-                                if constexpr (KIND == PASS_COUNT) {
-                                    ac += (i0 ? 1u : 0u) + (i1 ? 1u : 0u);
-                                    if constexpr (HL) *js += (j0 ? 1ull : 0ull) + (j1 ? 1ull << 32 : 0ull);
-                                } else if constexpr (KIND == PASS_MIN) {
-                                    const uint32_t u0 = __float_as_uint(d0), u1 = __float_as_uint(d1);
-                                    if (i0) ac = min(ac, u0);
-                                    if (i1) ac = min(ac, u1);
-                                    if constexpr (HL) {
-                                        const f32x2 o = *js;
-                                        const uint32_t l = j0 ? min((uint32_t)o, u0) : (uint32_t)o;
-                                        const uint32_t h = j1 ? min((uint32_t)(o >> 32), u1) : (uint32_t)(o >> 32);
-                                        *js = ((f32x2)h << 32) | l;
-                                    }
-                                } else {
-                                    // f: minus the coefficient of dx in the force on j
-                                    float f0, f1;
-                                    if constexpr (KIND == PASS_LJ) {
-                                        // -1/d2 by the hardware reciprocal and one Newton step
-                                        const f32x2 r = pk2(rcp_ftz(-d0), rcp_ftz(-d1));
-                                        const f32x2 e = fma2_rn(pk2(d0, d1), r, dup2(1.f));
-                                        const f32x2 s2 = mul2_rn(dup2(sig2), fma2_rn(r, e, r));
-                                        const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);  // -(sigma/r)^6
-                                        unpk2(mul2_rn(s2, fma2_rn(add2_rn(s6, s6), s6, s6)), f0, f1);
-                                    } else {
-                                        const float4 C = S.jc[q];
-                                        const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
-                                        const f32x2 ir2 = mul2_rn(ir, ir);
-                                        const f32x2 s2 = mul2_rn(dup2(-sig2), ir2);
-                                        const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);
-                                        const f32x2 lj = mul2_rn(dup2(e24), fma2_rn(add2_rn(s6, s6), s6, s6));
-                                        const f32x2 qq = mul2_rn(ivx, pk2(C.x, C.y));
-                                        float t0, t1;
-                                        unpk2(mul2_rn(ir2, fma2_rn(qq, ir, lj)), t0, t1);
-                                        f0 = -t0;
-                                        f1 = -t1;
-                                    }
-                                    // (padding particles are far away: never in range, dx finite)
-                                    const f32x2 fi = pk2(i0 ? f0 : 0.f, i1 ? f1 : 0.f);
-                                    ax = fma2_rn(fi, dx, ax);
-                                    ay = fma2_rn(fi, dy, ay);
-                                    az = fma2_rn(fi, dz, az);
-                                    if constexpr (HL) {
-                                        const f32x2 fj = pk2(j0 ? f0 : 0.f, j1 ? f1 : 0.f);
-                                        js[0] = fma2_rn(fj, dx, js[0]);
-                                        js[JS] = fma2_rn(fj, dy, js[JS]);
-                                        js[2 * JS] = fma2_rn(fj, dz, js[2 * JS]);
-                                    }
-                                }
-                            }
+                            JPart j = load_j(el, tt);
+                            terms(I0, j, A0, std::false_type(), box);
+                            terms(I1, j, A1, std::false_type(), box);
+                            store_j(el, tt, j);
                         }
                     }
-                    // scalar terms: canonical predicate, accurate pair vector
-#pragma unroll 1
-                    for (uint32_t todo = bits & slow; todo; todo &= todo - 1u) {
+                    for (uint32_t todo = b0w & ~b1w; todo; todo &= todo - 1u) {
                         const uint32_t el = __ffs(todo) - 1;
-                        const uint32_t Je = __shfl_sync(0xffffffffu, J, c + el);
-#pragma unroll 1
-                        for (uint32_t th = 0; th < 2 * NT; ++th) {
-                            const uint32_t tt = th >> 1, h = th & 1u;
-                            const uint32_t q = el * HJ + g + tt * G;
-                            float *js = reinterpret_cast<float *>(S.js + (el * NT + tt) * 32 + lane) + h;
-                            constexpr uint32_t JS = SE * NT * 64;
-                            const float *A = reinterpret_cast<const float *>(&S.ja[q]) + h;
-                            const float *B = reinterpret_cast<const float *>(&S.jb[q]) + h;
-                            const float *C = reinterpret_cast<const float *>(&S.jc[Smem::JC ? q : 0]) + h;
-                            const float4 pj = make_float4(A[0], A[2], B[0], B[2]);
-                            const float3 dv = pair_dx_acc<PER>(pi, pj, box);
-                            const float e2 = d2_of(dv);
-                            float fi = 0.f, fj = 0.f;  // coefficients of dv
-                            if constexpr (KIND == PASS_DENSITY) {
-                                const float r = sqrt_approx(e2);
-                                const float wi = spline_half_w(sat_fma1(r, pi.w), r * -pi.w);
-                                if (wi > 0.f) ax = add2_rn(ax, pk2(pj.w * wi, 0.f));
-                                if constexpr (HL) {
-                                    const float wj = spline_half_w(sat_fma1(r, C[0]), r * C[2]);
-                                    if (wj > 0.f) *js += iv.x * wj;
-                                }
-                            } else if constexpr (KIND == PASS_SPH) {
-                                const float ir = e2 > 0.f ? rsqrtf(e2) : 0.f;  // grad W(0) = 0
-                                const float r = e2 * ir;
-                                const float gi = spline_third_dw(sat_fma1(r, pi.w), r * pi.w);
-                                const float gj = spline_third_dw(sat_fma1(r, pj.w), r * pj.w);
-                                if ((gi != 0.f || gj != 0.f) && e2 > 0.f) {
-                                    const float b = ((gi != 0.f ? iv.x * gi : 0.f) + (gj != 0.f ? C[0] * gj : 0.f)) * ir;
-                                    fi = C[2] * b;
-                                    fj = iv.y * b;
-                                }
-                            } else {
-                                const float d2 = pair_d2<PER>(pi, pj, box);
-                                const bool self = NO_SELF && (s * kSC + k) * M + II == Je * MJ + g + tt * G + h * HJ;
-                                const bool ini = d2 < pi.w && !self;
-                                const bool inj = HL && d2 < pj.w && !self;
-                                if constexpr (KIND == PASS_COUNT) {
-                                    ac += ini ? 1u : 0u;
-                                    if (inj) *js = __uint_as_float(__float_as_uint(*js) + 1u);
-                                } else if constexpr (KIND == PASS_MIN) {
-                                    if (ini) ac = min(ac, __float_as_uint(e2));
-                                    if (inj) *js = fminf(*js, e2);
-                                } else if (ini || inj) {
-                                    float f;
-                                    if constexpr (KIND == PASS_LJ) {
-                                        const float s2 = sig2 * (1.f / e2);
-                                        const float s6 = s2 * s2 * s2;
-                                        f = -(s2 * (s6 * (2.f * s6 - 1.f)));
-                                    } else {
-                                        const float ir = rsqrtf(e2);
-                                        const float ir2 = ir * ir;
-                                        const float s2 = sig2 * ir2;
-                                        const float s6 = s2 * s2 * s2;
-                                        f = -(ir2 * (e24 * (s6 * (2.f * s6 - 1.f)) + iv.x * C[0] * ir));
-                                    }
-                                    if (ini) fi = f;
-                                    if (inj) fj = f;
-                                }
-                            }
-                            if constexpr (FORCE) {
-                                if (fi != 0.f) {
-                                    ax = add2_rn(ax, pk2(fi * dv.x, 0.f));
-                                    ay = add2_rn(ay, pk2(fi * dv.y, 0.f));
-                                    az = add2_rn(az, pk2(fi * dv.z, 0.f));
-                                }
-                                if constexpr (HL) {
-                                    if (fj != 0.f) {
-                                        js[0] += fj * dv.x;
-                                        js[JS] += fj * dv.y;
-                                        js[2 * JS] += fj * dv.z;
-                                    }
-                                }
-                            }
+#pragma unroll
+                        for (uint32_t tt = 0; tt < NT; ++tt) {
+                            JPart j = load_j(el, tt);
+                            terms(I0, j, A0, std::false_type(), box);
+                            store_j(el, tt, j);
                         }
                     }
-                    // over the lanes of the same i particle, then to the lane
-                    // that keeps its running sum
-                    const bool mine = k / NK == g;
-                    if constexpr (INTS) {
+                    for (uint32_t todo = b1w & ~b0w; todo; todo &= todo - 1u) {
+                        const uint32_t el = __ffs(todo) - 1;
 #pragma unroll
-                        for (int o = M; o < 32; o <<= 1) ac = merge(ac, __shfl_xor_sync(0xffffffffu, ac, o));
-#pragma unroll
-                        for (uint32_t q = 0; q < NK; ++q)
-                            if (mine && k % NK == q) rc[q] = merge(rc[q], ac);
-                    } else {
-                        float x0, x1, y0, y1, z0, z1;
-                        unpk2(ax, x0, x1);
-                        unpk2(ay, y0, y1);
-                        unpk2(az, z0, z1);
-                        float x = x0 + x1, y = y0 + y1, z = z0 + z1;
-#pragma unroll
-                        for (int o = M; o < 32; o <<= 1) {
-                            x += __shfl_xor_sync(0xffffffffu, x, o);
-                            if constexpr (FORCE) {
-                                y += __shfl_xor_sync(0xffffffffu, y, o);
-                                z += __shfl_xor_sync(0xffffffffu, z, o);
-                            }
+                        for (uint32_t tt = 0; tt < NT; ++tt) {
+                            JPart j = load_j(el, tt);
+                            terms(I1, j, A1, std::false_type(), box);
+                            store_j(el, tt, j);
                         }
+                    }
+                    keep(k, A0, A1);
+                }
+                if ((slow | owns) & staged) {
+                    // pairs across a periodic face, packed; self pairs and inputs
+                    // that are not finite, scalar: canonical predicate, accurate
+                    // pair vector
+#pragma unroll 1
+                    for (uint32_t k = 0; k < kSC; ++k) {
+                        const uint32_t lists = (__ballot_sync(0xffffffffu, (mk >> k) & 1u) >> c) & staged;
+                        const uint32_t dg = diag(k), bits = careful ? lists : lists & dg;
+                        const uint32_t wrapped = PER && !careful ? lists & slow & ~dg : 0u;
+                        if (!(bits | wrapped)) continue;
+                        ISum T{0ull, 0ull, 0ull, NONE};
+                        if constexpr (PER) {
+                            if (wrapped) {
+                                const IPart<KIND> I = own_part(k);
+#pragma unroll 1
+                                for (uint32_t todo = wrapped; todo; todo &= todo - 1u) {
+                                    const uint32_t el = __ffs(todo) - 1;
 #pragma unroll
-                        for (uint32_t q = 0; q < NK; ++q)
-                            if (mine && k % NK == q) {
-                                if constexpr (KIND == PASS_DENSITY) {
-                                    sum_add(rx[q], cx[q], x);
-                                } else {
-                                    sum_add(rx[q], cx[q], x);
-                                    sum_add(ry[q], cy[q], y);
-                                    sum_add(rz[q], cz[q], z);
+                                    for (uint32_t tt = 0; tt < NT; ++tt) {
+                                        JPart j = load_j(el, tt);
+                                        terms(I, j, T, std::true_type(), box);
+                                        store_j(el, tt, j);
+                                    }
                                 }
                             }
+                        }
+                        const float4 pi = S.ia[k * M + II];
+                        const float2 iv = Smem::IB ? S.ib[Smem::IB ? k * M + II : 0] : make_float2(0.f, 0.f);
+#pragma unroll 1
+                        for (uint32_t todo = bits; todo; todo &= todo - 1u) {
+                            const uint32_t el = __ffs(todo) - 1;
+                            const uint32_t Je = __shfl_sync(0xffffffffu, J, c + el);
+#pragma unroll 1
+                            for (uint32_t th = 0; th < 2 * NT; ++th) {
+                                const uint32_t tt = th >> 1, h = th & 1u;
+                                const uint32_t q = el * HJ + g + tt * G;
+                                float *js = reinterpret_cast<float *>(S.js + (el * NT + tt) * 32 + lane) + h;
+                                const float *A = reinterpret_cast<const float *>(&S.ja[q]) + h;
+                                const float *B = reinterpret_cast<const float *>(&S.jb[q]) + h;
+                                const float *C = reinterpret_cast<const float *>(&S.jc[Smem::JC ? q : 0]) + h;
+                                const float4 pj = make_float4(A[0], A[2], B[0], B[2]);
+                                const float3 dv = pair_dx_acc<PER>(pi, pj, box);
+                                const float e2 = d2_of(dv);
+                                float fi = 0.f, fj = 0.f;  // coefficients of dv
+                                if constexpr (KIND == PASS_DENSITY) {
+                                    const float r = sqrt_approx(e2);
+                                    const float wi = spline_half_w(sat_fma1(r, pi.w), r * -pi.w);
+                                    if (wi > 0.f) T.x = add2_rn(T.x, pk2(pj.w * wi, 0.f));
+                                    if constexpr (HL) {
+                                        const float wj = spline_half_w(sat_fma1(r, C[0]), r * C[2]);
+                                        if (wj > 0.f) *js += iv.x * wj;
+                                    }
+                                } else if constexpr (KIND == PASS_SPH) {
+                                    const float ir = e2 > 0.f ? rsqrtf(e2) : 0.f;  // grad W(0) = 0
+                                    const float r = e2 * ir;
+                                    const float gi = spline_third_dw(sat_fma1(r, pi.w), r * pi.w);
+                                    const float gj = spline_third_dw(sat_fma1(r, pj.w), r * pj.w);
+                                    if ((gi != 0.f || gj != 0.f) && e2 > 0.f) {
+                                        const float b = ((gi != 0.f ? iv.x * gi : 0.f) + (gj != 0.f ? C[0] * gj : 0.f)) * ir;
+                                        fi = C[2] * b;
+                                        fj = iv.y * b;
+                                    }
+                                } else {
+                                    const float d2 = pair_d2<PER>(pi, pj, box);
+                                    const bool self = NO_SELF && (s * kSC + k) * M + II == Je * MJ + g + tt * G + h * HJ;
+                                    const bool ini = d2 < pi.w && !self;
+                                    const bool inj = HL && d2 < pj.w && !self;
+                                    if constexpr (KIND == PASS_COUNT) {
+                                        T.c += ini ? 1u : 0u;
+                                        if (inj) *js = __uint_as_float(__float_as_uint(*js) + 1u);
+                                    } else if constexpr (KIND == PASS_MIN) {
+                                        if (ini) T.c = min(T.c, __float_as_uint(e2));
+                                        if (inj) *js = fminf(*js, e2);
+                                    } else if (ini || inj) {
+                                        float f;
+                                        if constexpr (KIND == PASS_LJ) {
+                                            const float s2 = sig2 * (1.f / e2);
+                                            const float s6 = s2 * s2 * s2;
+                                            f = -(s2 * (s6 * (2.f * s6 - 1.f)));
+                                        } else {
+                                            const float ir = rsqrtf(e2);
+                                            const float ir2 = ir * ir;
+                                            const float s2 = sig2 * ir2;
+                                            const float s6 = s2 * s2 * s2;
+                                            f = -(ir2 * (e24 * (s6 * (2.f * s6 - 1.f)) + iv.x * C[0] * ir));
+                                        }
+                                        if (ini) fi = f;
+                                        if (inj) fj = f;
+                                    }
+                                }
+                                if constexpr (FORCE) {
+                                    if (fi != 0.f) {
+                                        T.x = add2_rn(T.x, pk2(fi * dv.x, 0.f));
+                                        T.y = add2_rn(T.y, pk2(fi * dv.y, 0.f));
+                                        T.z = add2_rn(T.z, pk2(fi * dv.z, 0.f));
+                                    }
+                                    if constexpr (HL) {
+                                        if (fj != 0.f) {
+                                            js[0] += fj * dv.x;
+                                            js[2 * JS] += fj * dv.y;
+                                            js[4 * JS] += fj * dv.z;
+                                        }
+                                    }
+                                }
+                            }
+                        }
+                        const ISum Z{0ull, 0ull, 0ull, NONE};
+                        if (k & 1u) keep(k - 1u, Z, T);
+                        else keep(k, T, Z);
                     }
                 }
 
@@ -750,7 +904,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                 ry[q] = __fsub_rn(ry[q], cy[q]);
                 rz[q] = __fsub_rn(rz[q], cz[q]);
             }
-            const uint32_t k = g * NK + q;
+            const uint32_t k = cluster_of(q);
             const uint32_t i = (s * kSC + k) * M + II;
             const uint32_t pc = a.perm[i];
             if (pc == 0xffffffffu) continue;  // dummy slot
