@@ -286,6 +286,13 @@ __device__ __forceinline__ f32x2 mul2_rn(f32x2 a, f32x2 b)
     return r;
 }
 
+__device__ __forceinline__ f32x2 fma2_rn(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 template <bool PER>
 __device__ __forceinline__ float pair_d2(const float4 &pi, const float4 &pj, const PerLen &L)
 {

@@ -69,13 +69,6 @@ __device__ __forceinline__ f32x2 add2_rn(f32x2 a, f32x2 b)
     return r;
 }
 
-__device__ __forceinline__ f32x2 fma2_rn(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 __device__ __forceinline__ f32x2 dup2(float a) { return pk2(a, a); }
 
 // a * b + 1 clamped to [0, 1]; NaN gives 0

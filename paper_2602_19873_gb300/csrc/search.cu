@@ -12,7 +12,13 @@
 //      the M x MJ tiles of Sec. II-A / III-A), 32 at a time against the boxes of
 //      the 8 i-clusters;
 //   3. a few single pairs of each candidate tile by the exact FP32 predicate;
-//   4. all M x MJ pairs of the tiles still undecided, 32 / M tiles at a time.
+//   4. all M x MJ pairs of the tiles still undecided, 32 / M tiles at a time, in
+//      fused packed arithmetic whose sign decides them unless it is within its
+//      own rounding of zero: then by the exact predicate.
+// Periodic systems wrap differences only in batches that can hold a wrapped pair
+// (the boxes of their j-clusters against the super-cluster's); that code is kept
+// rolled, as both copies unrolled waited 2.2 cycles per instruction for the
+// instruction cache.
 // All box tests use monotone round-to-nearest gaps, so that no pair accepted by
 // the FP32 predicate can be pruned.  Depth-first order yields ascending
 // j-clusters (Sec. II-A), so the (J, mask) list is produced sorted; it is staged
@@ -22,12 +28,14 @@
 // buffer.  Super-clusters whose list exceeds the staging capacity or the
 // list buffer are queued in a redo list and re-run by the host after growth.
 //
-// What bounds it: instruction issue (75 % of cycles) and shared-memory wavefronts
-// (60 %), not DRAM.  The lane-per-item steps replaced a walk that tested one node,
-// four j-clusters and one tile at a time with the whole warp: 78.7k -> 20k warp
-// instructions per super-cluster on the Evrard sphere at 2^21; search stage (half
-// lists, CUDA events) 1.18 -> 0.75 ms there, 15.9 -> 9.2 ms on 2^24 particles in
-// 64 Plummer spheres, 3.36 -> 2.20 ms on the 4M-particle fluid.
+// What bounds it: instruction issue (0.65 to 0.76 per scheduler and cycle), not
+// DRAM; about half of the time goes to step 4, a quarter to the walk.  The
+// lane-per-item steps replaced a walk that tested one node, four j-clusters and one
+// tile at a time with the whole warp: 78.7k -> 20k warp instructions per
+// super-cluster on the Evrard sphere at 2^21; search stage (half lists, CUDA events)
+// 1.18 -> 0.75 ms there, 15.9 -> 9.2 ms on 2^24 particles in 64 Plummer spheres, 3.36
+// -> 2.22 ms on the 4M-particle fluid.  Fused tile tests, and wraps only where they
+// can happen: 0.74, 9.1 and 1.90 ms.
 #include <algorithm>
 #include <type_traits>
 
@@ -352,10 +360,13 @@ constexpr uint32_t sr_batch() { return MJ > 8 ? 256 / MJ : 32; }
 template <int M, int MJ>
 struct SearchSmem {
     float4 ip[kSC * M];                 // i particles
-    float4 jp[sr_batch<MJ>() * MJ];     // j particles of the batch
+    // j particles of the batch, in pairs (q, q + MJ/2) of a cluster:
+    // (x, x', y, y'), (z, z', -r^2, -r'^2)
+    float4 ja[sr_batch<MJ>() * MJ / 2], jb[sr_batch<MJ>() * MJ / 2];
     float4 ibox[kSC / 2][4];            // boxes of the i-clusters, in pairs
     uint32_t jq[64];                    // j-clusters to test, ascending (ring)
     uint32_t found[32];                 // per batch slot: tiles holding a pair
+    float jrr[32];                      // per batch slot: largest r^2
     uint8_t tl[32 * kSC];               // candidate tiles: slot * 8 + i-cluster
     uint32_t win[WIN_WORDS];
 };
@@ -406,6 +417,14 @@ __device__ __forceinline__ void box_pair_near(const float4 *ib, const float4 &bl
     n1 = db <= fmaxf(B.w, brr);
 }
 
+// Does the canonical difference of some pair of the intervals [a0, a1], [b0, b1]
+// wrap around a periodic axis?
+__device__ __forceinline__ bool wraps(float a0, float a1, float b0, float b1, float len)
+{
+    const float half = __fmul_rn(0.5f, len);
+    return __fsub_rn(b1, a0) > half || __fsub_rn(b0, a1) < -half;
+}
+
 // MODE 0: full list.  MODE 1: half search, upper entries and transposed
 // tuples for the record assembly.  MODE 2: half list (each pair stored once,
 // Sec. II-D): the half search's upper entries encoded as the record.  MODE 3:
@@ -420,6 +439,7 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
     constexpr bool HALF = MODE != 0;  // only j-clusters from the own first one on
     constexpr uint32_t NB = sr_batch<MJ>();
     constexpr uint32_t G = 32 / M;        // tiles tested together, M lanes each
+    constexpr uint32_t HJ = MJ / 2;       // pairs of j particles of a cluster
     constexpr int NPI = (kSC * M) / 32;   // i particles per lane
     extern __shared__ __align__(16) unsigned char search_smem[];
     SearchSmem<M, MJ> &S = reinterpret_cast<SearchSmem<M, MJ> *>(search_smem)[threadIdx.x >> 5];
@@ -436,7 +456,7 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
     const uint32_t II = lane % M, grp = lane / M;
     // order in which a group of lanes reads the j particles of its tile: the
     // groups read different 16-byte columns of the staged clusters (banks)
-    const uint32_t swz = (MJ >= 8 ? 2u * grp : grp) & (uint32_t)(MJ - 1);
+    const uint32_t swz = grp & (HJ - 1u);
     const uint32_t gbits = (M == 32 ? 0xffffffffu : ((1u << M) - 1u)) << (grp * M);
     const uint32_t count = ctl.count_dev ? min(ctl.count, *ctl.count_dev) : ctl.count;
 
@@ -539,39 +559,56 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 if (lane == 0) B.src[b] = (uint16_t)cnt;
             }
             const uint32_t cnt0 = cnt;
-            // 1. box tests, one j-cluster per lane against the 8 i-clusters
             const uint32_t J = lane < nq ? S.jq[(qh + lane) & 63u] : 0u;
-            uint32_t cm = 0;
+            float4 blo, bhi;
             if (lane < nq) {
-                const float4 blo = a.jlo[J], bhi = a.jhi[J];
-                const float brr = __fmul_rn(blo.w, blo.w);
-#pragma unroll
-                for (int k = 0; k < kSC; k += 2) {
-                    bool n0, n1;
-                    box_pair_near<PER>(S.ibox[k >> 1], blo, bhi, brr, box, n0, n1);
-                    cm |= (n0 ? 1u << k : 0u) | (n1 ? 2u << k : 0u);
-                }
+                blo = a.jlo[J];
+                bhi = a.jhi[J];
             }
-            if (__any_sync(0xffffffffu, cm != 0u)) {
+            uint32_t mask = 0;
+            // wr: pairs of the batch may lie across a periodic face
+            auto test = [&](auto wr) {
+                constexpr bool WR = decltype(wr)::value;
+                // 1. box tests, one j-cluster per lane against the 8 i-clusters
+                uint32_t cm = 0;
+                if (lane < nq) {
+                    const float brr = __fmul_rn(blo.w, blo.w);
+                    S.jrr[lane] = brr;
+#pragma unroll (WR ? 1 : kSC / 2)
+                    for (int k = 0; k < kSC; k += 2) {
+                        bool n0, n1;
+                        box_pair_near<WR>(S.ibox[k >> 1], blo, bhi, brr, box, n0, n1);
+                        cm |= (n0 ? 1u << k : 0u) | (n1 ? 2u << k : 0u);
+                    }
+                }
+                if (!__any_sync(0xffffffffu, cm != 0u)) return false;
                 // 2. stage the j particles
-                for (uint32_t q = lane; q < nq * MJ; q += 32) {
-                    const float4 p = a.pos[S.jq[(qh + q / MJ) & 63u] * MJ + q % MJ];
-                    const float r = __fmul_rn(a.support, p.w);
-                    S.jp[q] = make_float4(p.x, p.y, p.z, __fmul_rn(r, r));
+                for (uint32_t q = lane; q < nq * HJ; q += 32) {
+                    const float4 *p = a.pos + S.jq[(qh + q / HJ) & 63u] * MJ + q % HJ;
+                    const float4 p0 = p[0], p1 = p[HJ];
+                    const float r0 = __fmul_rn(a.support, p0.w), r1 = __fmul_rn(a.support, p1.w);
+                    S.ja[q] = make_float4(p0.x, p1.x, p0.y, p1.y);
+                    S.jb[q] = make_float4(p0.z, p1.z, -__fmul_rn(r0, r0), -__fmul_rn(r1, r1));
                 }
                 __syncwarp();
+                // particle jj of batch slot sl
+                auto staged = [&](uint32_t sl, uint32_t jj) {
+                    const uint32_t q = sl * HJ + (jj & (HJ - 1u)), h = jj / HJ;
+                    const float *A = reinterpret_cast<const float *>(&S.ja[q]) + h;
+                    const float *B = reinterpret_cast<const float *>(&S.jb[q]) + h;
+                    return make_float4(A[0], A[2], B[0], -B[2]);
+                };
                 // 3. single pairs of every candidate tile, one j-cluster per
                 // lane: most tiles that hold a pair are found here (about half
                 // of all pairs of such tiles are neighbors)
-                uint32_t mask = 0;
                 if (cm) {
-#pragma unroll
+#pragma unroll (WR ? 1 : kProbes)
                     for (int q = 0; q < kProbes; ++q) {
-                        const float4 pj = S.jp[lane * MJ + ((lane + q * (MJ / 2)) & (MJ - 1))];
-#pragma unroll
+                        const float4 pj = staged(lane, (lane + q * HJ) & (MJ - 1));
+#pragma unroll (WR ? 1 : kSC)
                         for (int k = 0; k < kSC; ++k) {
                             const float4 pi = S.ip[k * M + (q * (M / 2) + M / 4)];
-                            const float d2 = pair_d2<PER>(pi, pj, box);
+                            const float d2 = pair_d2<WR>(pi, pj, box);
                             // (a self pair has d2 = 0)
                             if (d2 < fmaxf(pi.w, pj.w) && d2 > 0.f) mask |= 1u << k;
                         }
@@ -585,45 +622,70 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 const uint32_t T = __shfl_sync(0xffffffffu, incl, 31);
                 uint32_t at = incl - pc;
                 for (uint32_t b = cm; b; b &= b - 1u) S.tl[at++] = (uint8_t)(lane * kSC + __ffs(b) - 1);
+                ttests += T;
                 __syncwarp();
-                // 4. exact FP32 test of these tiles, G at a time: a lane holds
-                // one i particle of its group's tile and takes the MJ j
-                // particles in turn
-                auto tiles_test = [&](auto own) {
+                // 4. FP32 test of these tiles, G at a time: a lane holds one i
+                // particle of its group's tile and takes the MJ j particles in turn
+                const uint32_t J0 = S.jq[qh & 63u];
+                const bool own = J0 * MJ < base + kSC * M && S.jq[(qh + nq - 1u) & 63u] * MJ >= base;
+                {
                     for (uint32_t t0 = 0; t0 < T; t0 += G) {
                         const uint32_t e = S.tl[min(t0 + grp, T - 1u)];
                         const uint32_t sl = e >> 3, k = e & 7u;
                         const float4 pi = S.ip[k * M + II];
-                        const float4 *jb = S.jp + sl * MJ;
-                        // pair (i, j) is a self pair iff jj == delta
-                        const uint32_t delta = own ? base + k * M + II - S.jq[(qh + sl) & 63u] * MJ : 0u;
-                        const f32x2 ixy = pk2(pi.x, pi.y);
-                        bool hit = false;
+                        bool hit = false, exact = WR || own;
+                        if (!exact) {
+                            // min of d2 - max(ri^2, rj^2), two j particles at a
+                            // time in fused arithmetic.  It and the canonical
+                            // predicate's sum are each within 2^-22 of the radius
+                            // squared of the true value near zero: only a
+                            // minimum within tol of zero needs the exact test.
+                            const float nri = -pi.w;
+                            const f32x2 ix = pk2(pi.x, pi.x), iy = pk2(pi.y, pi.y), iz = pk2(pi.z, pi.z);
+                            float mn = INFINITY;
 #pragma unroll
-                        for (uint32_t t = 0; t < (uint32_t)MJ; ++t) {
-                            const uint32_t jj = t ^ swz;
-                            const float4 pj = jb[jj];
-                            float d2;
-                            if constexpr (PER) {
-                                d2 = pair_d2<true>(pi, pj, box);
-                            } else {
-                                const f32x2 dxy = sub2_rn(pk2(pj.x, pj.y), ixy);
-                                const float dz = __fsub_rn(pj.z, pi.z);
-                                float x2, y2;
-                                unpk2(mul2_rn(dxy, dxy), x2, y2);
-                                d2 = __fadd_rn(__fadd_rn(x2, y2), __fmul_rn(dz, dz));
+                            for (uint32_t t = 0; t < HJ; ++t) {
+                                const uint32_t q = sl * HJ + (t ^ swz);
+                                const float4 A = S.ja[q], B = S.jb[q];
+                                const f32x2 dx = sub2_rn(pk2(A.x, A.y), ix), dy = sub2_rn(pk2(A.z, A.w), iy);
+                                const f32x2 dz = sub2_rn(pk2(B.x, B.y), iz);
+                                const f32x2 m = pk2(fminf(nri, B.z), fminf(nri, B.w));
+                                float d0, d1;
+                                unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, fma2_rn(dx, dx, m))), d0, d1);
+                                mn = fminf(mn, fminf(d0, d1));
                             }
-                            hit |= d2 < fmaxf(pi.w, pj.w) && (!own || jj != delta);
+                            const float tol = fmaf(fmaxf(pi.w, S.jrr[sl]), 2e-6f, 1e-37f);
+                            hit = mn < -tol;
+                            exact = __any_sync(0xffffffffu, !hit && mn <= tol);
+                        }
+                        if (exact) {
+                            // pair (i, j) is a self pair iff jj == delta
+                            const uint32_t delta = base + k * M + II - S.jq[(qh + sl) & 63u] * MJ;
+#pragma unroll (WR ? 1 : MJ)
+                            for (uint32_t t = 0; t < (uint32_t)MJ; ++t) {
+                                const uint32_t jj = t ^ swz;
+                                const float4 pj = staged(sl, jj);
+                                hit |= pair_d2<WR>(pi, pj, box) < fmaxf(pi.w, pj.w) && jj != delta;
+                            }
                         }
                         const uint32_t hb = __ballot_sync(0xffffffffu, hit) & gbits;
                         if (II == 0 && hb) atomicOr(&S.found[sl], 1u << k);
                     }
-                };
-                const uint32_t J0 = S.jq[qh & 63u];
-                if (J0 * MJ < base + kSC * M && S.jq[(qh + nq - 1u) & 63u] * MJ >= base)
-                    tiles_test(std::true_type{});
-                else
-                    tiles_test(std::false_type{});
+                }
+                return true;
+            };
+            bool any;
+            if constexpr (PER) {
+                // no pair of the batch wraps if none of the box corners does (the
+                // canonical difference is monotone in both coordinates)
+                const bool in = lane >= nq || (!wraps(slo.x, shi.x, blo.x, bhi.x, box.x) &&
+                                               !wraps(slo.y, shi.y, blo.y, bhi.y, box.y) &&
+                                               !wraps(slo.z, shi.z, blo.z, bhi.z, box.z));
+                any = __all_sync(0xffffffffu, in) ? test(std::false_type{}) : test(std::true_type{});
+            } else {
+                any = test(std::false_type{});
+            }
+            if (any) {
                 __syncwarp();
                 // 5. j-clusters with a tile holding a pair
                 mask = S.found[lane];
@@ -635,7 +697,6 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 }
                 cnt += __popc(has);
                 tiles += __popc(mask);
-                ttests += T;
                 __syncwarp();
             }
             if (SPLIT && lane == 0) B.first[nbatch] = (uint16_t)(cnt - cnt0);

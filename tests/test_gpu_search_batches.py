@@ -79,3 +79,22 @@ def test_deep_and_shallow_trees(bucket, periodic):
 def test_small_systems(n, half):
     for tile in ((8, 8), (4, 4), (16, 16)):
         _check(cloud(n, n % 2), tile, half)
+
+
+def lattice(scale, periodic):
+    """Spacings and ranges that differ by a few ulps: the fused sums of the tile
+    test cannot decide these pairs, which need the canonical predicate; at the
+    small scale squared distances are denormal."""
+    rng = np.random.default_rng(33)
+    m = 12
+    g = (np.indices((m, m, m)).reshape(3, -1).T + 0.5) / m
+    p = g * (1 + rng.integers(-3, 4, g.shape) * 6e-8)
+    h = (1 + rng.integers(-3, 4, len(g)) * 6e-8) / (2 * m)
+    return _system(scale * p, scale * h, periodic)
+
+
+@pytest.mark.parametrize("half", [0, 1])
+@pytest.mark.parametrize("tile", TILES)
+@pytest.mark.parametrize("scale,periodic", [(1.0, 0), (1.0, 1), (3e-21, 0)])
+def test_pairs_at_the_edge_of_the_range(scale, periodic, tile, half):
+    _check(lattice(scale, periodic), tile, half)
