@@ -15,18 +15,12 @@
 //   4. all M x MJ pairs of the tiles still undecided, 32 / M tiles at a time, in
 //      fused packed arithmetic whose sign decides them unless it is within its
 //      own rounding of zero: then by the exact predicate.
-// Periodic systems wrap differences only in batches that can hold a wrapped pair
-// (the boxes of their j-clusters against the super-cluster's); that code is kept
-// rolled, as both copies unrolled waited 2.2 cycles per instruction for the
-// instruction cache.
-// All box tests use monotone round-to-nearest gaps, so that no pair accepted by
-// the FP32 predicate can be pruned.  Depth-first order yields ascending
-// j-clusters (Sec. II-A), so the (J, mask) list is produced sorted; it is staged
-// per warp (L2 resident) and then encoded:
-// u32 count | u8 masks | nibble blocks of 32 differences (Sec. II-B, the
-// layout of Sec. II-C with w = 32), reserved with one atomicAdd in the list
-// buffer.  Super-clusters whose list exceeds the staging capacity or the
-// list buffer are queued in a redo list and re-run by the host after growth.
+// Periodic systems: only in batches that can hold a wrapped pair (the boxes of
+// their j-clusters against the super-cluster's) are the j particles moved to the
+// image next to the super-cluster, and the rounding of that is part of the margin
+// within which the exact predicate decides.  Differences wrapped pair by pair cost
+// twice the open arithmetic, and a second copy of the code for batches without
+// wraps waited 2.2 cycles per instruction for the instruction cache.
 //
 // What bounds it: instruction issue (0.65 to 0.76 per scheduler and cycle), not
 // DRAM; about half of the time goes to step 4, a quarter to the walk.  The
@@ -34,8 +28,8 @@
 // tile at a time with the whole warp: 78.7k -> 20k warp instructions per
 // super-cluster on the Evrard sphere at 2^21; search stage (half lists, CUDA events)
 // 1.18 -> 0.75 ms there, 15.9 -> 9.2 ms on 2^24 particles in 64 Plummer spheres, 3.36
-// -> 2.22 ms on the 4M-particle fluid.  Fused tile tests, and wraps only where they
-// can happen: 0.74, 9.1 and 1.90 ms.
+// -> 2.22 ms on the 4M-particle fluid.  Fused tile tests, and images instead of
+// wrapped differences: 0.71, 9.0 and 1.69 ms.
 #include <algorithm>
 #include <type_traits>
 
@@ -565,27 +559,82 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 blo = a.jlo[J];
                 bhi = a.jhi[J];
             }
-            uint32_t mask = 0;
-            // wr: pairs of the batch may lie across a periodic face
-            auto test = [&](auto wr) {
-                constexpr bool WR = decltype(wr)::value;
-                // 1. box tests, one j-cluster per lane against the 8 i-clusters
-                uint32_t cm = 0;
-                if (lane < nq) {
-                    const float brr = __fmul_rn(blo.w, blo.w);
-                    S.jrr[lane] = brr;
-#pragma unroll (WR ? 1 : kSC / 2)
+            uint32_t mask = 0, cm = 0;
+            const float brr = lane < nq ? __fmul_rn(blo.w, blo.w) : 0.f;
+            // Periodic: do pairs of the batch wrap?  Not if none of the box corners
+            // does (the canonical difference is monotone in both coordinates).  If
+            // some may, the j particles are staged in the image next to the
+            // super-cluster, where squared distances are within tx of the canonical
+            // ones: an image is then the nearest one or beyond every radius if the
+            // box and the radii leave room (else all tiles are tested exactly).
+            bool wr = false, room = true;
+            float tx = 0.f;
+            if constexpr (PER) {
+                const bool w = lane < nq && (wraps(slo.x, shi.x, blo.x, bhi.x, box.x) ||
+                                             wraps(slo.y, shi.y, blo.y, bhi.y, box.y) ||
+                                             wraps(slo.z, shi.z, blo.z, bhi.z, box.z));
+                wr = __any_sync(0xffffffffu, w);
+                if (wr) {
+                    // largest radius, and coordinate with its shift
+                    float rm = slo.w, am = 0.f;
+                    if (lane < nq && blo.x <= bhi.x) {
+                        rm = fmaxf(rm, blo.w);
+                        am = fmaxf(fmaxf(fmaxf(fabsf(blo.x), fabsf(bhi.x)), fmaxf(fabsf(blo.y), fabsf(bhi.y))),
+                                   fmaxf(fabsf(blo.z), fabsf(bhi.z)));
+                    }
+                    rm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rm)));
+                    am = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(am)));
+                    auto axis = [&](float lo, float hi, float len) {
+                        if (len < INFINITY) {
+                            am = fmaxf(am, fmaxf(fabsf(lo), fabsf(hi)) + len);
+                            room = room && rm + 0.5f * (hi - lo) < 0.499f * len;
+                        }
+                    };
+                    const float a0 = am;
+                    axis(slo.x, shi.x, box.x);
+                    axis(slo.y, shi.y, box.y);
+                    axis(slo.z, shi.z, box.z);
+                    am += a0;
+                    // three differences, each a few roundings of am off
+                    tx = room ? fmaf(am * 2e-6f, rm, am * am * 1e-12f) : 0.f;
+                }
+            }
+            // 1. box tests, one j-cluster per lane against the 8 i-clusters
+            if (lane < nq) {
+                S.jrr[lane] = brr;
+                if (PER && wr) {
+#pragma unroll 1
                     for (int k = 0; k < kSC; k += 2) {
                         bool n0, n1;
-                        box_pair_near<WR>(S.ibox[k >> 1], blo, bhi, brr, box, n0, n1);
+                        box_pair_near<PER>(S.ibox[k >> 1], blo, bhi, brr, box, n0, n1);
+                        cm |= (n0 ? 1u << k : 0u) | (n1 ? 2u << k : 0u);
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < kSC; k += 2) {
+                        bool n0, n1;
+                        box_pair_near<false>(S.ibox[k >> 1], blo, bhi, brr, box, n0, n1);
                         cm |= (n0 ? 1u << k : 0u) | (n1 ? 2u << k : 0u);
                     }
                 }
-                if (!__any_sync(0xffffffffu, cm != 0u)) return false;
+            }
+            if (__any_sync(0xffffffffu, cm != 0u)) {
                 // 2. stage the j particles
                 for (uint32_t q = lane; q < nq * HJ; q += 32) {
                     const float4 *p = a.pos + S.jq[(qh + q / HJ) & 63u] * MJ + q % HJ;
-                    const float4 p0 = p[0], p1 = p[HJ];
+                    float4 p0 = p[0], p1 = p[HJ];
+                    if (PER && wr && room) {
+                        auto image = [](float x, float lo, float hi, float len) {
+                            const float d = x - 0.5f * (lo + hi);
+                            return d > 0.5f * len ? x - len : d < -0.5f * len ? x + len : x;
+                        };
+                        p0.x = image(p0.x, slo.x, shi.x, box.x);
+                        p0.y = image(p0.y, slo.y, shi.y, box.y);
+                        p0.z = image(p0.z, slo.z, shi.z, box.z);
+                        p1.x = image(p1.x, slo.x, shi.x, box.x);
+                        p1.y = image(p1.y, slo.y, shi.y, box.y);
+                        p1.z = image(p1.z, slo.z, shi.z, box.z);
+                    }
                     const float r0 = __fmul_rn(a.support, p0.w), r1 = __fmul_rn(a.support, p1.w);
                     S.ja[q] = make_float4(p0.x, p1.x, p0.y, p1.y);
                     S.jb[q] = make_float4(p0.z, p1.z, -__fmul_rn(r0, r0), -__fmul_rn(r1, r1));
@@ -601,16 +650,17 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 // 3. single pairs of every candidate tile, one j-cluster per
                 // lane: most tiles that hold a pair are found here (about half
                 // of all pairs of such tiles are neighbors)
-                if (cm) {
-#pragma unroll (WR ? 1 : kProbes)
+                if (cm && room) {
+                    const float part = wr ? 1.f - 2e-6f : 1.f;  // (1: the canonical predicate)
+#pragma unroll
                     for (int q = 0; q < kProbes; ++q) {
                         const float4 pj = staged(lane, (lane + q * HJ) & (MJ - 1));
-#pragma unroll (WR ? 1 : kSC)
+#pragma unroll
                         for (int k = 0; k < kSC; ++k) {
                             const float4 pi = S.ip[k * M + (q * (M / 2) + M / 4)];
-                            const float d2 = pair_d2<WR>(pi, pj, box);
+                            const float d2 = pair_d2<false>(pi, pj, box);
                             // (a self pair has d2 = 0)
-                            if (d2 < fmaxf(pi.w, pj.w) && d2 > 0.f) mask |= 1u << k;
+                            if (d2 < fmaf(fmaxf(pi.w, pj.w), part, -tx) && d2 > 0.f) mask |= 1u << k;
                         }
                     }
                     cm &= ~mask;
@@ -628,64 +678,57 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                 // particle of its group's tile and takes the MJ j particles in turn
                 const uint32_t J0 = S.jq[qh & 63u];
                 const bool own = J0 * MJ < base + kSC * M && S.jq[(qh + nq - 1u) & 63u] * MJ >= base;
-                {
-                    for (uint32_t t0 = 0; t0 < T; t0 += G) {
-                        const uint32_t e = S.tl[min(t0 + grp, T - 1u)];
-                        const uint32_t sl = e >> 3, k = e & 7u;
-                        const float4 pi = S.ip[k * M + II];
-                        bool hit = false, exact = WR || own;
-                        if (!exact) {
-                            // min of d2 - max(ri^2, rj^2), two j particles at a
-                            // time in fused arithmetic.  It and the canonical
-                            // predicate's sum are each within 2^-22 of the radius
-                            // squared of the true value near zero: only a
-                            // minimum within tol of zero needs the exact test.
-                            const float nri = -pi.w;
-                            const f32x2 ix = pk2(pi.x, pi.x), iy = pk2(pi.y, pi.y), iz = pk2(pi.z, pi.z);
-                            float mn = INFINITY;
+                for (uint32_t t0 = 0; t0 < T; t0 += G) {
+                    const uint32_t e = S.tl[min(t0 + grp, T - 1u)];
+                    const uint32_t sl = e >> 3, k = e & 7u;
+                    const float4 pi = S.ip[k * M + II];
+                    // pair (i, j) is a self pair iff jj == delta
+                    const uint32_t Jt = S.jq[(qh + sl) & 63u];
+                    const uint32_t delta = base + k * M + II - Jt * MJ;
+                    bool hit = false;
+                    if (PER && !room) {
+#pragma unroll 4
+                        for (uint32_t t = 0; t < (uint32_t)MJ; ++t) {
+                            const uint32_t jj = t ^ swz;
+                            const float4 pj = staged(sl, jj);
+                            hit |= pair_d2<PER>(pi, pj, box) < fmaxf(pi.w, pj.w) && jj != delta;
+                        }
+                    } else {
+                        // min of d2 - max(ri^2, rj^2), two j particles at a time in
+                        // fused arithmetic.  It and the canonical predicate's sum
+                        // are each within 2^-22 of the radius squared (and tx) of the
+                        // true value near zero: only a minimum within tol of zero
+                        // needs the exact test; so do tiles holding self pairs.
+                        const float nri = -pi.w;
+                        const f32x2 ix = pk2(pi.x, pi.x), iy = pk2(pi.y, pi.y), iz = pk2(pi.z, pi.z);
+                        float mn = INFINITY;
 #pragma unroll
-                            for (uint32_t t = 0; t < HJ; ++t) {
-                                const uint32_t q = sl * HJ + (t ^ swz);
-                                const float4 A = S.ja[q], B = S.jb[q];
-                                const f32x2 dx = sub2_rn(pk2(A.x, A.y), ix), dy = sub2_rn(pk2(A.z, A.w), iy);
-                                const f32x2 dz = sub2_rn(pk2(B.x, B.y), iz);
-                                const f32x2 m = pk2(fminf(nri, B.z), fminf(nri, B.w));
-                                float d0, d1;
-                                unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, fma2_rn(dx, dx, m))), d0, d1);
-                                mn = fminf(mn, fminf(d0, d1));
-                            }
-                            const float tol = fmaf(fmaxf(pi.w, S.jrr[sl]), 2e-6f, 1e-37f);
-                            hit = mn < -tol;
-                            exact = __any_sync(0xffffffffu, !hit && mn <= tol);
+                        for (uint32_t t = 0; t < HJ; ++t) {
+                            const uint32_t q = sl * HJ + (t ^ swz);
+                            const float4 A = S.ja[q], B = S.jb[q];
+                            const f32x2 dx = sub2_rn(pk2(A.x, A.y), ix), dy = sub2_rn(pk2(A.z, A.w), iy);
+                            const f32x2 dz = sub2_rn(pk2(B.x, B.y), iz);
+                            const f32x2 m = pk2(fminf(nri, B.z), fminf(nri, B.w));
+                            float d0, d1;
+                            unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, fma2_rn(dx, dx, m))), d0, d1);
+                            mn = fminf(mn, fminf(d0, d1));
                         }
-                        if (exact) {
-                            // pair (i, j) is a self pair iff jj == delta
-                            const uint32_t delta = base + k * M + II - S.jq[(qh + sl) & 63u] * MJ;
-#pragma unroll (WR ? 1 : MJ)
-                            for (uint32_t t = 0; t < (uint32_t)MJ; ++t) {
-                                const uint32_t jj = t ^ swz;
-                                const float4 pj = staged(sl, jj);
-                                hit |= pair_d2<WR>(pi, pj, box) < fmaxf(pi.w, pj.w) && jj != delta;
+                        const float tol = fmaf(fmaxf(pi.w, S.jrr[sl]), 2e-6f, tx + 1e-37f);
+                        hit = mn < -tol;
+                        const bool exact = (!hit && mn <= tol) || (own && delta < (uint32_t)MJ);
+                        if (__any_sync(0xffffffffu, exact)) {  // (particles as they are, not their images)
+                            if (exact) hit = false;
+#pragma unroll 2
+                            for (uint32_t jj = 0; jj < (uint32_t)MJ; ++jj) {
+                                const float4 pj = a.pos[(size_t)Jt * MJ + jj];
+                                const float r = __fmul_rn(a.support, pj.w);
+                                hit |= pair_d2<PER>(pi, pj, box) < fmaxf(pi.w, __fmul_rn(r, r)) && jj != delta;
                             }
                         }
-                        const uint32_t hb = __ballot_sync(0xffffffffu, hit) & gbits;
-                        if (II == 0 && hb) atomicOr(&S.found[sl], 1u << k);
                     }
+                    const uint32_t hb = __ballot_sync(0xffffffffu, hit) & gbits;
+                    if (II == 0 && hb) atomicOr(&S.found[sl], 1u << k);
                 }
-                return true;
-            };
-            bool any;
-            if constexpr (PER) {
-                // no pair of the batch wraps if none of the box corners does (the
-                // canonical difference is monotone in both coordinates)
-                const bool in = lane >= nq || (!wraps(slo.x, shi.x, blo.x, bhi.x, box.x) &&
-                                               !wraps(slo.y, shi.y, blo.y, bhi.y, box.y) &&
-                                               !wraps(slo.z, shi.z, blo.z, bhi.z, box.z));
-                any = __all_sync(0xffffffffu, in) ? test(std::false_type{}) : test(std::true_type{});
-            } else {
-                any = test(std::false_type{});
-            }
-            if (any) {
                 __syncwarp();
                 // 5. j-clusters with a tile holding a pair
                 mask = S.found[lane];
