@@ -595,8 +595,12 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
                     axis(slo.y, shi.y, box.y);
                     axis(slo.z, shi.z, box.z);
                     am += a0;
-                    // three differences, each a few roundings of am off
-                    tx = room ? fmaf(am * 2e-6f, rm, am * am * 1e-12f) : 0.f;
+                    // three differences, each at most 2 roundings of am off (margin 2);
+                    // where that is not small against the radii (boxes far from the
+                    // origin or very large), too many tiles would be left undecided
+                    tx = fmaf(am * 1e-6f, rm, am * am * 1e-12f);
+                    room = room && tx <= 1e-3f * rm * rm;
+                    if (!room) tx = 0.f;
                 }
             }
             // 1. box tests, one j-cluster per lane against the 8 i-clusters

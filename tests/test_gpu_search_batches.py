@@ -15,9 +15,9 @@ pytestmark = pytest.mark.gpu
 F = np.float32
 
 
-def _system(pos, h, periodic, kind=1):
+def _system(pos, h, periodic, kind=1, lo=0.0):
     pos = np.ascontiguousarray(pos, F)
-    box = {"lo": np.zeros(3, F), "hi": np.ones(3, F), "periodic": np.full(3, periodic, np.int32)}
+    box = {"lo": np.full(3, lo, F), "hi": np.full(3, lo + 1.0, F), "periodic": np.full(3, periodic, np.int32)}
     n = len(pos)
     return {"x": pos[:, 0].copy(), "y": pos[:, 1].copy(), "z": pos[:, 2].copy(),
             "h": np.ascontiguousarray(h, F), "m": np.ones(n, F), "box": box, "kind": kind, "support": 2.0}
@@ -98,3 +98,14 @@ def lattice(scale, periodic):
 @pytest.mark.parametrize("scale,periodic", [(1.0, 0), (1.0, 1), (3e-21, 0)])
 def test_pairs_at_the_edge_of_the_range(scale, periodic, tile, half):
     _check(lattice(scale, periodic), tile, half)
+
+
+@pytest.mark.parametrize("lo", [-0.5, 3.0, 1024.0])
+@pytest.mark.parametrize("half", [0, 1])
+def test_periodic_boxes_off_the_origin(lo, half):
+    """Images of particles round to the size of the coordinates: far from the
+    origin the differences are wrapped one by one instead."""
+    rng = np.random.default_rng(35)
+    d = _system(lo + rng.random((6000, 3)) * 0.999, rng.uniform(0.02, 0.05, 6000), 1, lo=lo)
+    for tile in ((8, 8), (4, 4), (16, 16)):
+        _check(d, tile, half)
