@@ -759,12 +759,6 @@ inline bool pass_is_packed(int kind, int M, int MJ, float support)
 {
     return M * MJ >= 64 && ((kind != PASS_DENSITY && kind != PASS_SPH) || support == 2.f);
 }
-// The packed LJ kernel sums its terms in units of 24 eps / sigma^2 (sigma^2
-// rounded to FP32 as in the terms).
-__device__ __forceinline__ double lj_unit(int kind, const PassArgs &a)
-{
-    return kind == PASS_LJ && a.packed ? 24.0 * (double)a.p0 / (double)(a.p1 * a.p1) : 1.0;
-}
 // threads 0 = 256; blocks_per_sm 0 = default.  Sets a.packed and a.split.
 cudaError_t launch_pass(const PassArgs &a, int kind, int M, int any_periodic, int num_sms,
                         cudaStream_t s, int threads = 0, int blocks_per_sm = 0);

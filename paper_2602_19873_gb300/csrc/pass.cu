@@ -115,10 +115,9 @@ __global__ void __launch_bounds__(256) k_half_finish(PassArgs a, int kind, uint3
         return;
     }
     if (kind != PASS_DENSITY) {  // forces: the FP64 sums rounded once to FP32
-        const double u = lj_unit(kind, a);
-        a.out0[o] = (float)(a.hf[3 * (size_t)k + 0] * u);
-        a.out1[o] = (float)(a.hf[3 * (size_t)k + 1] * u);
-        a.out2[o] = (float)(a.hf[3 * (size_t)k + 2] * u);
+        a.out0[o] = (float)a.hf[3 * (size_t)k + 0];
+        a.out1[o] = (float)a.hf[3 * (size_t)k + 1];
+        a.out2[o] = (float)a.hf[3 * (size_t)k + 2];
         return;
     }
     const int ex = half_scale_exp(a.st->m_absmax);

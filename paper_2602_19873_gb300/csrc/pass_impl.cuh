@@ -1,4 +1,7 @@
-// Neighborhood passes over the compressed list (Sec. II-A: loop in parallel
+// Neighborhood passes in scalar arithmetic: tiles of fewer than 64 pairs (4x4,
+// 8x4), and density and pressure with a support other than 2.
+//
+// A pass over the compressed list (Sec. II-A: loop in parallel
 // over super-clusters, decode the list iteratively as needed, process each
 // cluster-cluster interaction; Sec. II-D: pure pair function + a sum or a
 // minimum).
@@ -156,8 +159,8 @@ constexpr size_t pass_smem_per_warp()
            (KIND == PASS_DENSITY ? (size_t)2 * kSC * 32 * sizeof(float) : 0);
 }
 
-// Resident blocks per SM the register budget is cut for (measured at the
-// benchmark sizes): the scalar passes run at 64 registers (4 blocks of 256;
+// Resident blocks per SM the register budget is cut for (measured with 8x8
+// tiles at 2^24 particles): the scalar passes run at 64 registers (4 blocks of 256;
 // 5 blocks were slower); the force passes at 128 (2 blocks) on half lists
 // and for LJ, at 85 (3 blocks) for SPH and LJ + Coulomb on full lists.
 template <int KIND, bool HL>
@@ -539,7 +542,7 @@ __global__ void __launch_bounds__(PS_THREADS, (ps_min_blocks<KIND, HL>())) k_pas
                             }
                     }
                 }
-                if constexpr (HL && NP == 2 && (KIND == PASS_DENSITY || KIND == PASS_COUNT)) {
+                if constexpr (HL && NP == 2 && KIND == PASS_DENSITY) {
                     if (js) {
                         // sum each j particle's share over the M lanes of its i
                         // particles in a fixed order: the first step trades the
@@ -547,23 +550,14 @@ __global__ void __launch_bounds__(PS_THREADS, (ps_min_blocks<KIND, HL>())) k_pas
                         // first j particle, odd lanes the second), two more steps
                         // finish; lanes II = 0 and 1 then add one integer each
                         const bool odd = II & 1u;
-                        if constexpr (KIND == PASS_DENSITY) {
-                            float v = (odd ? jsh[1] : jsh[0]) +
-                                      __shfl_xor_sync(0xffffffffu, odd ? jsh[0] : jsh[1], 1);
+                        float v = (odd ? jsh[1] : jsh[0]) + __shfl_xor_sync(0xffffffffu, odd ? jsh[0] : jsh[1], 1);
 #pragma unroll
-                            for (int o = 2; o < M; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                            // a share is a sum of m 4w >= 0 (up to a rounding of
-                            // the square root at the edge of the support, where
-                            // w is below 1e-20: clamped to 0)
-                            if (II < 2u && v > 0.f)
-                                atomicAdd(&a.hsum[Je * MJ + JJ0 + II * JSTEP], fixed_of_nonneg(v * hscale));
-                        } else {
-                            uint32_t v = (odd ? jcn[1] : jcn[0]) +
-                                         __shfl_xor_sync(0xffffffffu, odd ? jcn[0] : jcn[1], 1);
-#pragma unroll
-                            for (int o = 2; o < M; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                            if (II < 2u && v != 0u) atomicAdd(&a.hcnt[Je * MJ + JJ0 + II * JSTEP], v);
-                        }
+                        for (int o = 2; o < M; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                        // a share is a sum of m 4w >= 0 (up to a rounding of the
+                        // square root at the edge of the support, where w is
+                        // below 1e-20: clamped to 0)
+                        if (II < 2u && v > 0.f)
+                            atomicAdd(&a.hsum[Je * MJ + JJ0 + II * JSTEP], fixed_of_nonneg(v * hscale));
                     }
                 } else if constexpr (HL) {
                     if (js) {

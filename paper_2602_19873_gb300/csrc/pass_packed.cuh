@@ -33,7 +33,7 @@
 // a time.  A scalar form of the terms is left for tiles that hold self pairs which
 // have to be left out, and for all of them when an input is not finite (a status
 // word of the gather kernel).  (All entries of the own j-clusters and all wrapped
-// ones in the scalar form: LJ at 4M 3.8 ms instead of 3.39.)
+// ones in the scalar form: LJ at 4M 3.8 ms instead of 3.35.)
 //
 // What bounds it: instruction issue.  The half-list density pass issues 0.69, the
 // force passes 0.62 to 0.65 instructions per scheduler and cycle, with the FMA pipe
@@ -41,7 +41,7 @@
 // the wait for fixed latencies at 24 to 32 warps per SM, as many as the registers allow.
 // Pass stage, scalar kernel -> this one (CUDA events): half-list density on 2^24
 // particles 9.10 -> 6.77 ms, pressure force on the 2^21-particle Evrard sphere 2.85
-// -> 1.26, LJ at 4M particles 6.92 -> 3.39, LJ + Coulomb 4.83 -> 2.79; full lists:
+// -> 1.26, LJ at 4M particles 6.92 -> 3.35, LJ + Coulomb 4.83 -> 2.79; full lists:
 // density and nearest distance on 2M particles 1.38 -> 1.03, pressure force on 300k
 // 0.69 -> 0.29; small systems (split): density of 32k particles 0.48 -> 0.09 ms, of
 // 4096 0.32 -> 0.05 ms.
@@ -230,19 +230,20 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
     const float hscale = (HL && KIND == PASS_DENSITY)
                              ? __int_as_float((half_scale_exp(a.st->m_absmax) + 127) << 23) : 0.f;
     const float sig2 = a.p1 * a.p1, e24 = 24.f * a.p0;
-    // LJ terms are summed without this factor (half lists: left to the finishing
-    // kernel)
-    const double fscale = lj_unit(KIND, a);
-
     // running sums take one partial a stage.  Density and pressure (whose sums
     // cancel) compensated: plain adds left the pressure force of the Evrard
     // sphere 10 % further from FP64 than the scalar kernel, 3 % less time.  Lennard-
-    // Jones alone too (median error at 4M particles 3.60e-7 plain, 3.55e-7
-    // compensated, scalar kernel 3.57e-7; 4 % of the time); with Coulomb terms plain
-    // sums are as near as the scalar kernel's (4.73e-7).
+    // Jones sums are ruled by their nearest pairs: plain adds are as near as the
+    // scalar kernel's (median error at 4M particles 3.52e-7, scalar 3.57e-7; with
+    // Coulomb terms 4.72e-7, scalar 4.74e-7) and 4 % faster.
     auto sum_add = [](float &v, float &c, float b) {
-        if constexpr (KIND == PASS_DENSITY || KIND == PASS_SPH || KIND == PASS_LJ) kahan_add(v, c, b);
-        else v += b;
+        if constexpr (KIND == PASS_DENSITY || KIND == PASS_SPH) {
+            kahan_add(v, c, b);
+            // (a force that overflows stays infinite)
+            if (KIND != PASS_DENSITY && !(fabsf(v) < INFINITY)) c = 0.f;
+        } else {
+            v += b;
+        }
     };
     auto merge = [](uint32_t u, uint32_t v) { return KIND == PASS_COUNT ? u + v : min(u, v); };
 
@@ -373,17 +374,22 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                 float f0, f1;
                 if constexpr (KIND == PASS_LJ) {
                     // -1/d2 by the hardware reciprocal and one Newton step
+                    // (of denormal distances: overflows below like 1/d2)
+                    d0 = fmaxf(d0, 1.17549435e-38f);
+                    d1 = fmaxf(d1, 1.17549435e-38f);
                     const f32x2 r = pk2(rcp_ftz(-d0), rcp_ftz(-d1));
                     const f32x2 e = fma2_rn(pk2(d0, d1), r, dup2(1.f));
-                    const f32x2 s2 = mul2_rn(dup2(sig2), fma2_rn(r, e, r));
+                    const f32x2 ir2 = fma2_rn(r, e, r);
+                    const f32x2 s2 = mul2_rn(dup2(sig2), ir2);
                     const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);  // -(sigma/r)^6
-                    unpk2(mul2_rn(s2, fma2_rn(add2_rn(s6, s6), s6, s6)), f0, f1);
+                    // (overflows only where the product of all does)
+                    unpk2(mul2_rn(mul2_rn(mul2_rn(dup2(e24), ir2), s6), fma2_rn(dup2(2.f), s6, dup2(1.f))), f0, f1);
                 } else {
                     const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
                     const f32x2 ir2 = mul2_rn(ir, ir);
                     const f32x2 s2 = mul2_rn(dup2(-sig2), ir2);
                     const f32x2 s6 = mul2_rn(mul2_rn(s2, s2), s2);
-                    const f32x2 lj = mul2_rn(dup2(e24), fma2_rn(add2_rn(s6, s6), s6, s6));
+                    const f32x2 lj = mul2_rn(mul2_rn(dup2(e24), s6), fma2_rn(dup2(2.f), s6, dup2(1.f)));
                     const f32x2 qq = mul2_rn(I.u, pk2(C.x, C.y));
                     float t0, t1;
                     unpk2(mul2_rn(ir2, fma2_rn(qq, ir, lj)), t0, t1);
@@ -761,15 +767,16 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                                     } else if (ini || inj) {
                                         float f;
                                         if constexpr (KIND == PASS_LJ) {
-                                            const float s2 = sig2 * (1.f / e2);
+                                            const float ir2 = 1.f / e2;
+                                            const float s2 = sig2 * ir2;
                                             const float s6 = s2 * s2 * s2;
-                                            f = -(s2 * (s6 * (2.f * s6 - 1.f)));
+                                            f = -(e24 * ir2 * s6 * (2.f * s6 - 1.f));
                                         } else {
                                             const float ir = rsqrtf(e2);
                                             const float ir2 = ir * ir;
                                             const float s2 = sig2 * ir2;
                                             const float s6 = s2 * s2 * s2;
-                                            f = -(ir2 * (e24 * (s6 * (2.f * s6 - 1.f)) + iv.x * C[0] * ir));
+                                            f = -(ir2 * (e24 * s6 * (2.f * s6 - 1.f) + iv.x * C[0] * ir));
                                         }
                                         if (ini) fi = f;
                                         if (inj) fj = f;
@@ -935,10 +942,6 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                 atomicAdd(&a.hf[3 * (size_t)i + 0], f64_of(rx[q]));
                 atomicAdd(&a.hf[3 * (size_t)i + 1], f64_of(ry[q]));
                 atomicAdd(&a.hf[3 * (size_t)i + 2], f64_of(rz[q]));
-            } else if constexpr (KIND == PASS_LJ) {
-                a.out0[o] = (float)((double)rx[q] * fscale);
-                a.out1[o] = (float)((double)ry[q] * fscale);
-                a.out2[o] = (float)((double)rz[q] * fscale);
             } else {
                 a.out0[o] = rx[q];
                 a.out1[o] = ry[q];

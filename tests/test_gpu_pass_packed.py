@@ -100,3 +100,29 @@ def test_a_support_below_the_kernels_sums_its_own_pairs(support, half):
     rel = np.abs(gpu_density(L, t, n)[o["perm"]] - want) / want
     assert rel.max() <= DENSITY_RTOL, rel.max()
     L.free()
+
+
+@pytest.mark.parametrize("n", [900, 39001])
+@pytest.mark.parametrize("cluster,half", [(8, 0), (8, 1), (16, 0), (16, 1)])
+def test_lj_forces_overflow_where_their_coefficient_does(n, cluster, half):
+    """Pairs at 7e-4: 24 eps (2 s^12 - s^6) / r^2 exceeds FP32 (3.6e39), the force
+    itself (2.6e36) would not; at 1e-3 (2.5e37) it is finite."""
+    import torch
+    d = wl.lj_fluid(n, seed=330 + n % 89, rc=0.55)
+    for k, r in ((0, 7e-4), (2, 1e-3)):
+        for a in "xyz":
+            d[a][k] = np.float32(0.001 + 0.2 * k)
+            d[a][k + 1] = np.float32(d[a][k] + r / np.sqrt(3.0))
+    L, t = gpu_build(d, cluster=cluster, j_cluster=cluster, half_list=half)
+    out = [torch.empty(n, dtype=torch.float32, device="cuda") for _ in range(3)]
+    L.force_pass(nl.NL_FORCE_LJ, *out, eps=1.0, sigma=0.3)
+    got = np.stack([a.cpu().numpy() for a in out], 1)
+    assert np.all(got[0] == -np.inf) and np.all(got[1] == np.inf)
+    x = [np.array([d[a][k] for a in "xyz"], np.float64) for k in (2, 3)]
+    dv = x[1] - x[0]
+    r2 = dv @ dv
+    s6 = (0.09 / r2) ** 3
+    f = 24.0 / r2 * s6 * (2 * s6 - 1) * dv
+    assert np.allclose(got[3], f, rtol=1e-5) and np.allclose(got[2], -f, rtol=1e-5)
+    assert np.isfinite(got[2:]).all()
+    L.free()
