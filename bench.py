@@ -35,12 +35,11 @@ ALU_OPS_PER_DENSITY_SIDE = 12    # gather pair in range: square root, scale, spl
 ALGO_BYTES_PER_PARTICLE = 145    # keygen 20 + sort 24 + permute 49 + octree 2 + search 19 + density 31
 # DRAM bytes (read + write) of one k_search launch per particle, from an ncu
 # capture on this generator at 2^21 particles (8x8 clusters, leaf bucket 256,
-# half list: packed tile and node tests, the range test of the half search
-# ending at the first accepted leaf), 44.87 MB + 1.13 MB, scaled by the
-# particle count (the traffic grows with the particles).  Valid for that kernel
-# version only; a list kind without a capture of the current kernel reports no
-# traffic.
-SEARCH_DRAM_BYTES_PER_PARTICLE = {"half": 46.0e6 / 2097152}
+# half list: 32 nodes, j-clusters or tiles tested at a time), 44.89 MB + 1.54 MB,
+# scaled by the particle count (the traffic grows with the particles).  Valid for
+# that kernel version only; a list kind without a capture of the current kernel
+# reports no traffic.
+SEARCH_DRAM_BYTES_PER_PARTICLE = {"half": 46.43e6 / 2097152}
 
 
 def peaks():
@@ -486,7 +485,7 @@ def run_native(args):
                      "algorithmic": "%d FP32 ops per computed pair, %d computed pairs (tiles of "
                                     "the timed %s list with the mask bit set x M x MJ)"
                                     % (ALU_OPS_PER_PAIR_SEARCH, pairs, args.list)},
-        "roofline_pass": {"bound": "alu", "kernel": "k_pass (decode + density)",
+        "roofline_pass": {"bound": "alu", "kernel": "k_pass_packed (decode + density)",
                           "achieved": pass_achieved, "peak": alu_peak, "unit": "TFLOP/s",
                           "frac": pass_achieved / alu_peak,
                           "algorithmic": "%d FP32 ops per computed pair (%d) + %d per gather "

@@ -17,8 +17,8 @@
 // and written once for two tiles, and the two tiles' chains overlap.  (One
 // i-cluster at a time left the half-list force passes bound by shared memory, 12 of
 // 18 wavefronts per tile carrying the j shares: LJ at 4M particles 4.28 -> 3.8 ms,
-// LJ + Coulomb 3.73 -> 3.19, density and pressure of the 2^21-particle Evrard
-// sphere 1.51 -> 1.26 each; evaluating every entry for both would have cost 18 %
+// LJ + Coulomb 3.73 -> 3.19, pressure force of the 2^21-particle Evrard
+// sphere 1.51 -> 1.26; evaluating every entry for both would have cost 18 %
 // in pairs that are not listed.)
 //
 // The pair terms have no branches.  Kernels that vanish with the distance
