@@ -107,10 +107,10 @@ typedef struct {
     int32_t cluster;         /* M */
     int32_t compress;
     /* work of the last cluster-pair search (all rounds) */
-    int64_t node_visits;     /* octree nodes tested, summed over super-clusters */
+    int64_t node_visits;     /* octree nodes tested (32 at a time), summed over super-clusters */
     int64_t leaf_visits;     /* leaves reached */
     int64_t j_examined;      /* j-clusters box-tested against a super-cluster */
-    int64_t tile_tests;      /* (i-cluster, j-cluster) tiles decided by the exact predicate */
+    int64_t tile_tests;      /* (i-cluster, j-cluster) tiles decided by testing all their pairs */
     int32_t j_cluster;       /* MJ */
     int32_t pad0;
 } nl_sizes;
