@@ -276,6 +276,12 @@ DevBox make_devbox(const nl_box &b)
         d.qs[a] = num / len;
         d.per[a] = b.periodic[a] ? 1 : 0;
     }
+    // beyond the face nearer to the origin, by more than the coordinates' ulp; on a
+    // periodic axis two box lengths more, so that it is as far after wrapping (where
+    // FP32 ends before: such boxes have room for a wrapped difference of 0 only)
+    float away = std::max(1e30f, std::max(std::fabs(d.lo[0]), std::fabs(d.hi[0])) * 0x1p-21f);
+    if (d.per[0] && d.len[0] < 1e38f) away += 2.f * d.len[0];
+    d.far = d.hi[0] <= -d.lo[0] ? d.hi[0] + away : d.lo[0] - away;
     return d;
 }
 

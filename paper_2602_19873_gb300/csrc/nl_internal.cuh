@@ -29,6 +29,9 @@ constexpr uint32_t kSeek = 256;             // entries between the places a long
 struct DevBox {
     float lo[3], hi[3], len[3], half[3], qs[3];
     int per[3];
+    // x of the padding particles of the packed passes: so far outside the box that
+    // squared distances overflow (wrapped ones too), while differences stay finite
+    float far;
 };
 
 // Tables of a batch of independent systems (a single system is a batch of

@@ -60,7 +60,6 @@
 namespace nlg {
 
 constexpr int PK_THREADS = 256;
-constexpr float PK_FAR = 1e18f;     // position of padding particles: out of every range, finite
 
 __device__ __forceinline__ f32x2 add2_rn(f32x2 a, f32x2 b)
 {
@@ -167,7 +166,9 @@ struct PkSmem {
     float4 jc[JC ? NP : 1];
     f32x2 js[HL ? NC * SE * NT * 32 : NC * (kSC / G) * 16];
     float2 ib[IB ? NI : 2];
-    uint32_t seen, pad[3];
+    uint32_t seen;
+    float far;      // x of padding particles (DevBox::far)
+    uint32_t pad[2];
 };
 
 // Resident blocks of 256 threads the register budget is cut for (half-list
@@ -297,6 +298,18 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             }
         }
     };
+    // Padding particles: counts and nearest distances leave their NaN positions,
+    // which are in no range.  The sums need finite differences even of pairs that
+    // take no part: there padding lies at (far, 0, 0), where no squared distance is
+    // below a squared range, and 0 to density and pressure (mass and coefficient 0).
+    // A fixed point would be in range of some box or radius.
+    auto place_padding = [&](float4 &p, float far) {
+        if (!INTS && !(p.x == p.x)) {
+            p.x = far;
+            p.y = p.z = 0.f;
+        }
+    };
+
     // the terms of one i particle and the lane's two j particles; wrap: pairs
     // may lie across a periodic face
     auto terms = [&](const IPart<KIND> &I, JPart &j, ISum &T, auto wrap, const PerLen &box) {
@@ -503,11 +516,14 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             continue;
         }
         const uint32_t VW = W * np, vw = part * W + wig;  // warps that share the list
-        const PerLen box = per_len(a.sys.box[sys_of(a.sys.pad_off, a.sys.nsys, s * kSC * M)]);
+        const DevBox &sbox = a.sys.box[sys_of(a.sys.pad_off, a.sys.nsys, s * kSC * M)];
+        const PerLen box = per_len(sbox);
 
         // own particles; the box around them (periodic)
         float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
         __syncwarp();
+        const float far = INTS ? 0.f : sbox.far;
+        if (!INTS && lane == 0) S.far = far;
 #pragma unroll
         for (uint32_t t = lane; t < (uint32_t)Smem::NI; t += 32) {
             const uint32_t i = s * kSC * M + t;
@@ -534,7 +550,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                     lo[2] = fminf(lo[2], p.z); hi[2] = fmaxf(hi[2], p.z);
                 }
             }
-            if (!real) p.x = p.y = p.z = PK_FAR;
+            place_padding(p, far);
             S.ia[t] = make_float4(p.x, p.y, p.z, av);
         }
         if constexpr (PER) {
@@ -623,7 +639,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                                      __fsub_rn(p[h].y, lo[1]) > hy || __fsub_rn(p[h].y, hi[1]) < -hy ||
                                      __fsub_rn(p[h].z, lo[2]) > hz || __fsub_rn(p[h].z, hi[2]) < -hz;
                             }
-                            if (!(p[h].x == p[h].x)) p[h].x = p[h].y = p[h].z = PK_FAR;
+                            place_padding(p[h], INTS ? 0.f : S.far);
                         }
                         S.ja[q] = make_float4(p[0].x, p[1].x, p[0].y, p[1].y);
                         S.jb[q] = make_float4(p[0].z, p[1].z, bv[0], bv[1]);
