@@ -127,6 +127,9 @@ struct nl_list {
         leaf_lev, nodeoff, bsum;
     DevBuf nlo, nhi, nrng, nlevel, nparent, nchild, narrive;
     DevBuf stageJ, stageM, list, rec_off, redo, work, aux, status;
+    // inputs of the packed pressure pass; not in aux, which graphs of the density
+    // step hold the address of
+    DevBuf aux4;
     // half search: upper entries, transposed tuples (+ sort buffers), per super-cluster tables
     DevBuf uJ, uM, up_off, up_cnt, lower_cnt, seg_off, tkey, tkey_alt, tval, tval_alt, thist;
     // batches mixing periodic and open systems: their super-clusters, so that
@@ -203,7 +206,7 @@ struct nl_list {
                          &lcp, &lev,
                          &leaf_first, &leaf_lev, &nodeoff, &bsum, &nlo, &nhi, &nrng, &nlevel,
                          &nparent, &nchild, &narrive, &stageJ, &stageM, &list, &rec_off, &redo,
-                         &work, &aux, &status, &hx, &hy, &hz, &hh, &hm, &hrho, &perm_pad,
+                         &work, &aux, &aux4, &status, &hx, &hy, &hz, &hh, &hm, &hrho, &perm_pad,
                          &sys_off, &sys_pad, &sys_box, &sys_root, &sys_hcap, &it_hq,
                          &it_hlo, &it_hhi, &it_hs, &it_counts, &it_conv, &it_aflag, &it_alist,
                          &it_words, &it_tmp, &ml_X, &ml_e64, &ml_pred, &ml_slo, &ml_shi,
@@ -986,7 +989,7 @@ PassArgs pass_args(const nl_list *nl)
     a.rec_off = nl->rec_off.as<uint32_t>();
     a.perm = nl->perm_pad.as<uint32_t>();
     a.aux = nl->aux.as<float2>();
-    a.aux4 = nl->aux.as<float4>();
+    a.aux4 = nl->aux4.as<float4>();
     a.n = (uint32_t)nl->n;
     a.nsc = nl->nsc;
     a.sys = nl->tables();
@@ -1757,7 +1760,7 @@ nl_status nl_force_pass(const nl_list *cnl, int32_t kind, const float *params, c
     if (half) CK(nl->hf.ensure((size_t)nl->npad * 24));
     if (kind == NL_FORCE_SPH_PRESSURE) {
         if (!m || !rho || !pres) return fail(NL_ERR_ARG, "SPH force needs m, rho and pres");
-        CK(nl->aux.ensure((size_t)nl->npad * (sph4 ? 16 : 8)));
+        CK(sph4 ? nl->aux4.ensure((size_t)nl->npad * 16) : nl->aux.ensure((size_t)nl->npad * 8));
     }
     PassArgs a = pass_args(nl);  // after every buffer it points to exists
     a.out0 = ax;
@@ -1767,7 +1770,7 @@ nl_status nl_force_pass(const nl_list *cnl, int32_t kind, const float *params, c
         CK(nl->mark(6, s));
         CK(cudaMemsetAsync(&a.st->m_absmax, 0, sizeof(unsigned int), s));
         CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), nl->pos.as<float4>(), nl->p.support,
-                             m, pres, rho, sph4 ? AUX_SPH4 : AUX_SPH, nl->aux.p, s, &a.st->m_absmax));
+                             m, pres, rho, sph4 ? AUX_SPH4 : AUX_SPH, sph4 ? nl->aux4.p : nl->aux.p, s, &a.st->m_absmax));
         CK(nl->mark(7, s));
         if (half) CK(cudaMemsetAsync(nl->hf.p, 0, (size_t)nl->npad * 24, s));
         CK(run_pass(nl, a, PASS_SPH, s));
