@@ -713,7 +713,7 @@ nl_status do_search_half(nl_list *nl, cudaStream_t s)
         st = read_status(nl, s);
         if (st != NL_OK) return st;
         const uint32_t heavy[2] = {std::min(nl->hst->n_heavy[0], hcap), std::min(nl->hst->n_heavy[1], hcap)};
-        if (!work && (heavy[0] || heavy[1]) && !nl->hst->half_overflow) {
+        if (!work && (heavy[0] || heavy[1])) {
             uint32_t np[2];
             for (int per = 0; per < 2; ++per)
                 np[per] = std::min(kSearchPartsMax, std::max(kSearchPartsMin, kSearchItems / std::max(heavy[per], 1u)));

@@ -21,6 +21,7 @@ constexpr uint32_t kLongSearch = 1024, kLongList = 1024;
 // warp of the grid (one range can be all neighbors: with 64 ranges of a 2^20-particle
 // system, 2048 j-clusters, a part ran for 1 ms)
 constexpr uint32_t kSearchPartsMin = 64, kSearchPartsMax = 1024, kSearchItems = 155648;
+constexpr uint32_t kNoPlace = 0xffffffffu;  // a heavy super-cluster's part without room for its entries
 constexpr uint32_t kPassParts = 16;         // blocks that share a long list at most
 constexpr uint32_t kSeek = 256;             // entries between the places a long record can be entered (multiple of 32)
 

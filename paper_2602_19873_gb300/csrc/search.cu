@@ -485,9 +485,10 @@ __global__ void __launch_bounds__(SR_THREADS, 4) k_search(SearchArgs a, SearchCt
             pend = base + (uint32_t)((uint64_t)n8 * (part + 1) / ctl.nparts) * (kSC * M);
             cap = 0;
             if (ctl.phase == 2) {
-                if (a.st->half_overflow) continue;  // (the host starts over)
-                stJ = a.uJ + a.hpart[tk];
-                stM = a.uM + a.hpart[tk];
+                const uint32_t at = a.hpart[tk];
+                if (at == kNoPlace) continue;  // (the host starts over)
+                stJ = a.uJ + at;
+                stM = a.uM + at;
                 cap = 0xffffffffu;
             }
             if (pbeg == pend) {
@@ -1011,7 +1012,11 @@ cudaError_t launch_search_ctl(const SearchArgs &a, const uint32_t *work, uint32_
 }
 
 // Upper entries of a heavy super-cluster from the counts of its parts: one
-// reservation, then the place of every part (one warp per super-cluster).
+// reservation, then the place of every part (one warp per super-cluster).  Parts
+// with a place are searched to their end also when the tuples have no room left,
+// so that the host learns how many there are (stopping at the first that did not
+// fit made it start over with a little more room, again and again, until it gave up
+// on systems in which most super-clusters are heavy).
 __global__ void __launch_bounds__(128) k_heavy_place(SearchArgs a, const uint32_t *heavy, uint32_t count, uint32_t nparts)
 {
     const uint32_t h = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1024,6 +1029,7 @@ __global__ void __launch_bounds__(128) k_heavy_place(SearchArgs a, const uint32_
     if (lane == 0) off = atomicAdd(&a.st->up_used, (unsigned long long)cnt);
     off = __shfl_sync(0xffffffffu, off, 0);
     if (off + cnt > a.up_cap) {
+        for (uint32_t p = lane; p < nparts; p += 32) part[p] = kNoPlace;
         if (lane == 0) atomicExch(&a.st->half_overflow, 1u);
         return;
     }
