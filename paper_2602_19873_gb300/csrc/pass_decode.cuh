@@ -84,6 +84,13 @@ __device__ __forceinline__ unsigned long long fixed_of_nonneg(float x)
     return ((unsigned long long)hi << 32) | lo;
 }
 
+// The same for |x| < 2^63 of either sign, as two's complement.
+__device__ __forceinline__ unsigned long long fixed_of_signed(float x)
+{
+    const unsigned long long q = fixed_of_nonneg(fabsf(x));
+    return x < 0.f ? 0ull - q : q;
+}
+
 // The FP64 value of x with integer operations only (exact for normal x;
 // zero and subnormals, below 1.2e-38, give 0; inf and NaN stay so).
 __device__ __forceinline__ double f64_of(float x)

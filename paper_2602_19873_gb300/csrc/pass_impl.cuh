@@ -553,11 +553,10 @@ __global__ void __launch_bounds__(PS_THREADS, (ps_min_blocks<KIND, HL>())) k_pas
                         float v = (odd ? jsh[1] : jsh[0]) + __shfl_xor_sync(0xffffffffu, odd ? jsh[0] : jsh[1], 1);
 #pragma unroll
                         for (int o = 2; o < M; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                        // a share is a sum of m 4w >= 0 (up to a rounding of the
-                        // square root at the edge of the support, where w is
-                        // below 1e-20: clamped to 0)
-                        if (II < 2u && v > 0.f)
-                            atomicAdd(&a.hsum[Je * MJ + JJ0 + II * JSTEP], fixed_of_nonneg(v * hscale));
+                        // (a rounding of the square root at the edge of the support
+                        // can make w negative, by less than 1e-20: 0 units)
+                        if (II < 2u && v != 0.f)
+                            atomicAdd(&a.hsum[Je * MJ + JJ0 + II * JSTEP], fixed_of_signed(v * hscale));
                     }
                 } else if constexpr (HL) {
                     if (js) {

@@ -851,8 +851,8 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                             float v0, v1;
                             unpk2(v, v0, v1);
                             if constexpr (KIND == PASS_DENSITY) {  // units of w/2
-                                if (v0 > 0.f) atomicAdd(&a.hsum[j0], fixed_of_nonneg(__fmul_rn(v0, hscale) * 2.f));
-                                if (v1 > 0.f) atomicAdd(&a.hsum[j0 + HJ], fixed_of_nonneg(__fmul_rn(v1, hscale) * 2.f));
+                                if (v0 != 0.f) atomicAdd(&a.hsum[j0], fixed_of_signed(__fmul_rn(v0, hscale) * 2.f));
+                                if (v1 != 0.f) atomicAdd(&a.hsum[j0 + HJ], fixed_of_signed(__fmul_rn(v1, hscale) * 2.f));
                             } else if constexpr (KIND == PASS_COUNT) {
                                 if (__float_as_uint(v0)) atomicAdd(&a.hcnt[j0], __float_as_uint(v0));
                                 if (__float_as_uint(v1)) atomicAdd(&a.hcnt[j0 + HJ], __float_as_uint(v1));
