@@ -1768,7 +1768,7 @@ nl_status nl_force_pass(const nl_list *cnl, int32_t kind, const float *params, c
     a.out2 = az;
     if (kind == NL_FORCE_SPH_PRESSURE) {
         CK(nl->mark(6, s));
-        CK(cudaMemsetAsync(&a.st->m_absmax, 0, sizeof(unsigned int), s));
+        CK(cudaMemsetAsync(&a.st->m_absmax, 0, 2 * sizeof(unsigned int), s));  // and c_absmax
         CK(launch_gather_aux(nl->npad, nl->perm_pad.as<uint32_t>(), nl->pos.as<float4>(), nl->p.support,
                              m, pres, rho, sph4 ? AUX_SPH4 : AUX_SPH, sph4 ? nl->aux4.p : nl->aux.p, s, &a.st->m_absmax));
         CK(nl->mark(7, s));

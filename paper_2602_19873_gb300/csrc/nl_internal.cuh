@@ -97,9 +97,9 @@ struct Status {
     unsigned int pad2;
     // periodic super-clusters whose neighbors cannot wrap (interior) and the rest
     unsigned int n_int, n_bnd;
-    // density and pressure passes: bits of the largest |input| (half-list
-    // density: sets the fixed-point scale)
-    unsigned int m_absmax;
+    // density and pressure passes: bits of the largest |m| (half-list density:
+    // sets the fixed-point scale); pressure: of the largest |C|, 2 |C| / h
+    unsigned int m_absmax, c_absmax;
     // super-clusters whose lists grew past kLongSearch while searched (open and
     // periodic kernel), and lists longer than kLongList
     unsigned int n_heavy[2], n_long, n_seek;
@@ -769,8 +769,9 @@ cudaError_t launch_pass(const PassArgs &a, int kind, int M, int any_periodic, in
 // Pass inputs in SFC order, for real padded slots (values without effect for
 // dummies): AUX_CHARGE aux = (a, 0); AUX_MASS aux = (a, -1/(2h)), -inf when
 // (support h)^2 underflows; AUX_SPH aux = (a, b / c^2); AUX_SPH4 float4
-// (3 b / (pi c^2 h^4), a, -1/(2h), 0).  amax (AUX_MASS, AUX_SPH4): atomic
-// maximum of the bits of |inputs| (zero it first).
+// (C = 3 b / (pi c^2 h^4), a, -1/(2h), 0).  amax (AUX_MASS, AUX_SPH4): atomic
+// maximum of the bits of |a|; amax[1] (AUX_SPH4): of |C| and 2 |C| / h (zero
+// them first).
 enum AuxMode { AUX_CHARGE = 0, AUX_SPH = 1, AUX_MASS = 2, AUX_SPH4 = 3 };
 cudaError_t launch_gather_aux(uint32_t npad, const uint32_t *perm_pad, const float4 *pos, float support,
                               const float *a, const float *b, const float *c, int mode, void *aux,

@@ -56,9 +56,9 @@ __global__ void __launch_bounds__(256) k_gather_aux(uint32_t npad, const uint32_
                                                     unsigned int *amax)
 {
     constexpr bool MAXIMA = MODE == AUX_MASS || MODE == AUX_SPH4;
-    __shared__ unsigned int wm[8];
+    __shared__ unsigned int wm[8], wc[8];
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned int mb = 0;
+    unsigned int mb = 0, cb = 0;
     if (k < npad) {
         const uint32_t o = perm_pad[k];
         const bool real = o != 0xffffffffu;
@@ -76,21 +76,30 @@ __global__ void __launch_bounds__(256) k_gather_aux(uint32_t npad, const uint32_
         if constexpr (MODE == AUX_SPH4) {
             y = 0.954929658551372015f * y * hinv * hinv * hinv * hinv;  // 3/pi
             reinterpret_cast<float4 *>(aux)[k] = make_float4(y, x, hneg, 0.f);
-            mb = max(__float_as_uint(fabsf(x)), __float_as_uint(fabsf(y)));
+            cb = max(__float_as_uint(fabsf(y)), __float_as_uint(fabsf(2.f * y * hinv)));
         } else {
             reinterpret_cast<float2 *>(aux)[k] = make_float2(x, MODE == AUX_MASS ? hneg : y);
-            mb = __float_as_uint(fabsf(x));
         }
+        mb = __float_as_uint(fabsf(x));
     }
     if constexpr (MAXIMA) {
         // largest of the block, one atomic per block (non-negative floats
         // order like their bit patterns, NaN above all)
         mb = __reduce_max_sync(0xffffffffu, mb);
-        if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = mb;
+        if (MODE == AUX_SPH4) cb = __reduce_max_sync(0xffffffffu, cb);
+        if ((threadIdx.x & 31) == 0) {
+            wm[threadIdx.x >> 5] = mb;
+            wc[threadIdx.x >> 5] = cb;
+        }
         __syncthreads();
         if (threadIdx.x < 32) {
-            mb = __reduce_max_sync(0xffffffffu, threadIdx.x < (blockDim.x >> 5) ? wm[threadIdx.x] : 0u);
+            const bool on = threadIdx.x < (blockDim.x >> 5);
+            mb = __reduce_max_sync(0xffffffffu, on ? wm[threadIdx.x] : 0u);
             if (threadIdx.x == 0 && mb) atomicMax(amax, mb);
+            if constexpr (MODE == AUX_SPH4) {
+                cb = __reduce_max_sync(0xffffffffu, on ? wc[threadIdx.x] : 0u);
+                if (threadIdx.x == 0 && cb) atomicMax(amax + 1, cb);
+            }
         }
     }
 }

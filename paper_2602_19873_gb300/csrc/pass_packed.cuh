@@ -224,9 +224,13 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
     const uint32_t II = lane % M, g = lane / M;
     const uint32_t W = (uint32_t)a.split, wig = warp & (W - 1u), grp = warp / W;
     const uint32_t ngrp = (blockDim.x >> 5) / W;
-    // inputs that are not finite: a zero kernel must not multiply them
-    const bool careful = (KIND == PASS_DENSITY || KIND == PASS_SPH) &&
-                         __any_sync(0xffffffffu, a.st->m_absmax >= 0x7f800000u);
+    // inputs that are not finite: a zero kernel must not multiply them; nor a zero
+    // pair vector the pressure terms of coincident particles, at most m 2C/h
+    bool careful = false;
+    if constexpr (KIND == PASS_DENSITY) careful = a.st->m_absmax >= 0x7f800000u;
+    if constexpr (KIND == PASS_SPH)
+        careful = !(__uint_as_float(a.st->m_absmax) * __uint_as_float(a.st->c_absmax) < INFINITY);
+    careful = __any_sync(0xffffffffu, careful);
     // fixed-point scale of the half-list density
     const float hscale = (HL && KIND == PASS_DENSITY)
                              ? __int_as_float((half_scale_exp(a.st->m_absmax) + 127) << 23) : 0.f;
@@ -341,10 +345,12 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             if constexpr (HL)
                 j.x = fma2_rn(I.u, spline_half_w2(sat_fma1(r0, C.x), sat_fma1(r1, C.y), mul2_rn(r, pk2(C.z, C.w))), j.x);
         } else if constexpr (KIND == PASS_SPH) {
-            // (a self pair: dx = 0; the floor keeps 1/r finite)
+            // (a self pair: dx = 0, and careful passes aside b is finite; the floor,
+            // the smallest normal square, keeps 1/r finite and is so near that w'/r
+            // hardly depends on r)
             unpk2(fma2_rn(dz, dz, fma2_rn(dy, dy, mul2_rn(dx, dx))), d0, d1);
-            d0 = fmaxf(d0, 1e-30f);
-            d1 = fmaxf(d1, 1e-30f);
+            d0 = fmaxf(d0, 1.17549435e-38f);
+            d1 = fmaxf(d1, 1.17549435e-38f);
             const f32x2 ir = pk2(rsqrt_ftz(d0), rsqrt_ftz(d1));
             const f32x2 r = mul2_rn(pk2(d0, d1), ir);
             float r0, r1;
