@@ -140,7 +140,7 @@ struct nl_list {
     DevBuf sc_int, sc_bnd;
     // heavy super-clusters of the half search (two lists, and the parts of one),
     // lists of more than kLongList entries: their number at the last build
-    DevBuf heavy, hpart, long_list, seek, seek_of;
+    DevBuf heavy, hpart, long_list, long_asked, seek, seek_of;
     uint32_t n_long = 0;
     DevBuf perm_pad, sys_off, sys_pad, sys_box, sys_root, sys_hcap;
     int32_t nsys = 1;
@@ -212,7 +212,7 @@ struct nl_list {
                          &it_words, &it_tmp, &ml_X, &ml_e64, &ml_pred, &ml_slo, &ml_shi,
                          &uJ, &uM, &up_off, &up_cnt, &lower_cnt, &seg_off, &tkey, &tkey_alt,
                          &tval, &tval_alt, &thist, &sc_open, &sc_per, &sc_int, &sc_bnd,
-                         &pos_ref, &hsum, &hcnt, &hf, &heavy, &hpart, &long_list, &seek, &seek_of};
+                         &pos_ref, &hsum, &hcnt, &hf, &heavy, &hpart, &long_list, &long_asked, &seek, &seek_of};
         for (DevBuf *b : all) b->release();
         for (int i = 0; i <= kStages; ++i)
             if (ev[i]) cudaEventDestroy(ev[i]);
@@ -381,6 +381,7 @@ nl_status do_prep(nl_list *nl, const float *x, const float *y, const float *z, c
     CK(nl->redo.ensure((size_t)nsc * 4));
     CK(nl->work.ensure((size_t)nsc * 4));
     CK(nl->long_list.ensure((size_t)nsc * 8));
+    CK(nl->long_asked.ensure((size_t)nsc * 4));
     // seek points of the long records (those that find no room are decoded from
     // their start)
     CK(nl->seek.ensure(((size_t)N / 8 + nsc) * 8));
@@ -564,10 +565,16 @@ cudaError_t run_pass(const nl_list *nl, const PassArgs &a0, int kind, cudaStream
     PassArgs a = a0;
     if (nl->n_long && !nl->graph_mode && pass_is_packed(kind, M, a.mj, a.support)) {
         // the long lists, by many warps each, after the others (the device holds
-        // their list and number; those the caller did not ask for give the values
-        // they had)
+        // their list and number).  Of a caller's list of super-clusters the first
+        // launch marks the long ones: the outputs of the others stay as they are
+        cudaError_t e;
         a.skip_longer = kLongList;
-        cudaError_t e = run_pass_split(nl, a, kind, s);
+        if (a.work) {
+            a.long_asked = nl->long_asked.as<uint32_t>();
+            e = cudaMemsetAsync(a.long_asked, 0, (size_t)nl->nsc * 4, s);
+            if (e != cudaSuccess) return e;
+        }
+        e = run_pass_split(nl, a, kind, s);
         if (e != cudaSuccess) return e;
         a.work = nullptr;
         a.nwork = nl->nsc;

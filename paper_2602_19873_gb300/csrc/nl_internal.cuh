@@ -721,6 +721,7 @@ struct PassArgs {
     int packed;            // the packed kernel (pass_is_packed)
     int split;             // packed kernel: warps that share a super-cluster (1, 2, 4, 8)
     uint32_t skip_longer;  // packed kernel: leave lists of more entries to a pass over the long ones (0: none)
+    uint32_t *long_asked;  // packed kernel: per super-cluster, 1 when its list was left to that pass (NULL: all are)
     const uint2 *longs;    // packed kernel: the long lists (nwork of them), worked off in parts
     const uint2 *seek;
     uint32_t n, nsc;

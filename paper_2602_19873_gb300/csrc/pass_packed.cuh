@@ -488,6 +488,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             const uint2 l = a.longs[it % nwork];
             s = l.x;
             seek = l.y;
+            if (a.long_asked && !a.long_asked[s]) continue;
         } else {
             if (W == 1u) {
                 if (lane == 0) s = atomicAdd(&a.st->pass_ticket, 1u);
@@ -510,6 +511,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             if (part >= np) continue;
         }
         if (!LONG && a.skip_longer && cnt > a.skip_longer) {
+            if (a.long_asked && lane == 0) a.long_asked[s] = 1u;
             if constexpr (!HL && INTS) {  // empty results for the blocks to add to
                 for (uint32_t t = lane; t < (uint32_t)Smem::NI; t += 32) {
                     const uint32_t i = s * kSC * M + t, pc = a.perm[i];
