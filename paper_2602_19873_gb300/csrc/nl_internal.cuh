@@ -717,7 +717,7 @@ struct PassArgs {
     const uint32_t *rec_off;
     const uint32_t *perm;  // caller index of every padded slot, ~0 for dummies
     const float2 *aux;     // per padded particle: density (m, -1/(2h)); SPH (m, P/rho^2); LJ + Coulomb (q, 0)
-    const float4 *aux4;    // SPH, packed kernel: (3 P/(pi rho^2 h^4), m, -1/(2h), 0)
+    const float4 *aux4;    // SPH, packed kernel: (3 P/(pi rho^2 h^4), m, -1/(2h), P/rho^2)
     int packed;            // the packed kernel (pass_is_packed)
     int split;             // packed kernel: warps that share a super-cluster (1, 2, 4, 8)
     uint32_t skip_longer;  // packed kernel: leave lists of more entries to a pass over the long ones (0: none)
@@ -770,7 +770,7 @@ cudaError_t launch_pass(const PassArgs &a, int kind, int M, int any_periodic, in
 // Pass inputs in SFC order, for real padded slots (values without effect for
 // dummies): AUX_CHARGE aux = (a, 0); AUX_MASS aux = (a, -1/(2h)), -inf when
 // (support h)^2 underflows; AUX_SPH aux = (a, b / c^2); AUX_SPH4 float4
-// (C = 3 b / (pi c^2 h^4), a, -1/(2h), 0).  amax (AUX_MASS, AUX_SPH4): atomic
+// (C = 3 b / (pi c^2 h^4), a, -1/(2h), b / c^2).  amax (AUX_MASS, AUX_SPH4): atomic
 // maximum of the bits of |a|; amax[1] (AUX_SPH4): of |C| and 2 |C| / h (zero
 // them first).
 enum AuxMode { AUX_CHARGE = 0, AUX_SPH = 1, AUX_MASS = 2, AUX_SPH4 = 3 };

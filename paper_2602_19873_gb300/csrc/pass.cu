@@ -74,9 +74,9 @@ __global__ void __launch_bounds__(256) k_gather_aux(uint32_t npad, const uint32_
             y = b[o] / (rho * rho);
         }
         if constexpr (MODE == AUX_SPH4) {
-            y = 0.954929658551372015f * y * hinv * hinv * hinv * hinv;  // 3/pi
-            reinterpret_cast<float4 *>(aux)[k] = make_float4(y, x, hneg, 0.f);
-            cb = max(__float_as_uint(fabsf(y)), __float_as_uint(fabsf(2.f * y * hinv)));
+            const float c = 0.954929658551372015f * y * hinv * hinv * hinv * hinv;  // 3/pi
+            reinterpret_cast<float4 *>(aux)[k] = make_float4(c, x, hneg, y);
+            cb = max(__float_as_uint(fabsf(c)), __float_as_uint(fabsf(2.f * c * hinv)));
         } else {
             reinterpret_cast<float2 *>(aux)[k] = make_float2(x, MODE == AUX_MASS ? hneg : y);
         }

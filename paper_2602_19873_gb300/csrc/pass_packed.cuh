@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
             } else if constexpr (KIND == PASS_SPH) {
                 const float4 x = a.aux4[i];
                 av = x.z;
-                S.ib[t] = make_float2(x.x, x.y);
+                S.ib[t] = make_float2(careful ? x.w : x.x, x.y);
             } else if constexpr (KIND == PASS_LJC) {
                 av = fminf(av, a.p2);
                 S.ib[t] = make_float2(a.p3 * a.aux[i].x, 0.f);
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                             } else if constexpr (KIND == PASS_SPH) {
                                 const float4 x = a.aux4[j];
                                 bv[h] = x.z;
-                                cv[h] = x.x;
+                                cv[h] = careful ? x.w : x.x;
                                 dv[h] = x.y;
                             } else {
                                 if constexpr (HL) {
@@ -770,10 +770,16 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                                 } else if constexpr (KIND == PASS_SPH) {
                                     const float ir = e2 > 0.f ? rsqrtf(e2) : 0.f;  // grad W(0) = 0
                                     const float r = e2 * ir;
-                                    const float gi = spline_third_dw(sat_fma1(r, pi.w), r * pi.w);
-                                    const float gj = spline_third_dw(sat_fma1(r, pj.w), r * pj.w);
+                                    // (from P/rho^2: the coefficients may overflow
+                                    // where their products with w' do not)
+                                    auto grad = [&](float a) {
+                                        const float g = spline_third_dw(sat_fma1(r, a), r * a), q = -2.f * a;
+                                        return g != 0.f ? g * q * q * q * q : 0.f;
+                                    };
+                                    const float gi = grad(pi.w), gj = grad(pj.w);
                                     if ((gi != 0.f || gj != 0.f) && e2 > 0.f) {
-                                        const float b = ((gi != 0.f ? iv.x * gi : 0.f) + (gj != 0.f ? C[0] * gj : 0.f)) * ir;
+                                        const float b = ((gi != 0.f ? iv.x * gi : 0.f) + (gj != 0.f ? C[0] * gj : 0.f)) *
+                                                        0.954929658551372015f * ir;  // 3/pi
                                         fi = C[2] * b;
                                         fj = iv.y * b;
                                     }

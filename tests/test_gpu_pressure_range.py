@@ -61,3 +61,10 @@ def test_coincident_particles_of_large_mass(cluster, jcl, half):
     coefficients does not."""
     p = [(0.0, 0.0, 0.0), (1.3, 0.0, 0.0), (0.0, 0.0, -1.5), (0.0, 0.0, -1.5)]
     check(p, 1.0, 1e30, 2.2e8, cluster, jcl, half)
+
+
+@pytest.mark.parametrize("cluster,jcl,half", SHAPES)
+def test_coefficients_that_overflow_where_forces_do_not(cluster, jcl, half):
+    """3 P / (pi rho^2 h^4) is beyond FP32, its products with w' at 1.5 h are not."""
+    p = [(0.0, 0.0, 0.0), (0.75, 0.0, 0.0), (0.0, 0.8, 0.0), (0.0, 0.0, -0.85)]
+    check(p, 0.5, 1e-10, 2.6e37, cluster, jcl, half)
