@@ -31,8 +31,8 @@
 // Entries with pairs across a periodic face (an eighth of the tiles of LJ at 4M
 // particles) take the packed terms with the pair vector wrapped, one i-cluster at
 // a time.  A scalar form of the terms is left for tiles that hold self pairs which
-// have to be left out, and for all of them when an input is not finite (a status
-// word of the gather kernel).  (All entries of the own j-clusters and all wrapped
+// have to be left out, and for all of them when an input is not finite or pressure
+// coefficients may overflow (status words of the gather kernel).  (All entries of the own j-clusters and all wrapped
 // ones in the scalar form: LJ at 4M 3.8 ms instead of 3.35.)
 //
 // What bounds it: instruction issue.  The half-list density pass issues 0.69, the
@@ -41,7 +41,7 @@
 // the wait for fixed latencies at 24 to 32 warps per SM, as many as the registers allow.
 // Pass stage, scalar kernel -> this one (CUDA events): half-list density on 2^24
 // particles 9.10 -> 6.77 ms, pressure force on the 2^21-particle Evrard sphere 2.85
-// -> 1.26, LJ at 4M particles 6.92 -> 3.35, LJ + Coulomb 4.83 -> 2.79; full lists:
+// -> 1.27, LJ at 4M particles 6.92 -> 3.35, LJ + Coulomb 4.83 -> 2.79; full lists:
 // density and nearest distance on 2M particles 1.38 -> 1.03, pressure force on 300k
 // 0.69 -> 0.29; small systems (split): density of 32k particles 0.48 -> 0.09 ms, of
 // 4096 0.32 -> 0.05 ms.
@@ -226,11 +226,11 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
     const uint32_t ngrp = (blockDim.x >> 5) / W;
     // inputs that are not finite: a zero kernel must not multiply them; nor a zero
     // pair vector the pressure terms of coincident particles, at most m 2C/h
-    bool careful = false;
-    if constexpr (KIND == PASS_DENSITY) careful = a.st->m_absmax >= 0x7f800000u;
-    if constexpr (KIND == PASS_SPH)
-        careful = !(__uint_as_float(a.st->m_absmax) * __uint_as_float(a.st->c_absmax) < INFINITY);
-    careful = __any_sync(0xffffffffu, careful);
+    const bool careful =
+        KIND == PASS_DENSITY ? __any_sync(0xffffffffu, a.st->m_absmax >= 0x7f800000u)
+        : KIND == PASS_SPH
+            ? __any_sync(0xffffffffu, !(__uint_as_float(a.st->m_absmax) * __uint_as_float(a.st->c_absmax) < INFINITY))
+            : false;
     // fixed-point scale of the half-list density
     const float hscale = (HL && KIND == PASS_DENSITY)
                              ? __int_as_float((half_scale_exp(a.st->m_absmax) + 127) << 23) : 0.f;
@@ -303,13 +303,13 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
         }
     };
     // Padding particles: counts and nearest distances leave their NaN positions,
-    // which are in no range.  The sums need finite differences even of pairs that
-    // take no part: there padding lies at (far, 0, 0), where no squared distance is
-    // below a squared range, and 0 to density and pressure (mass and coefficient 0).
-    // A fixed point would be in range of some box or radius.
+    // which are in no range.  Sums of forces need finite differences even of pairs
+    // that take no part: there padding lies at (far, 0, 0), where no squared distance
+    // is below a squared range (a fixed point would be in range of some box or
+    // radius).  To the density, whose padding has no mass, any place will do.
     auto place_padding = [&](float4 &p, float far) {
         if (!INTS && !(p.x == p.x)) {
-            p.x = far;
+            p.x = FORCE ? far : 1e18f;
             p.y = p.z = 0.f;
         }
     };
@@ -392,8 +392,10 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                 // f: minus the coefficient of dx in the force on j
                 float f0, f1;
                 if constexpr (KIND == PASS_LJ) {
-                    // -1/d2 by the hardware reciprocal and one Newton step
-                    // (of denormal distances: overflows below like 1/d2)
+                    // -1/d2 by the hardware reciprocal and one Newton step.
+                    // Denormal d2 (separations below 1.1e-19) count as the
+                    // smallest normal one: the coefficient overflows there like
+                    // that of 1/d2 unless sigma is below about 1e-18
                     d0 = fmaxf(d0, 1.17549435e-38f);
                     d1 = fmaxf(d1, 1.17549435e-38f);
                     const f32x2 r = pk2(rcp_ftz(-d0), rcp_ftz(-d1));
@@ -530,8 +532,8 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
         // own particles; the box around them (periodic)
         float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
         __syncwarp();
-        const float far = INTS ? 0.f : sbox.far;
-        if (!INTS && lane == 0) S.far = far;
+        const float far = FORCE ? sbox.far : 0.f;
+        if (FORCE && lane == 0) S.far = far;
 #pragma unroll
         for (uint32_t t = lane; t < (uint32_t)Smem::NI; t += 32) {
             const uint32_t i = s * kSC * M + t;
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                                      __fsub_rn(p[h].y, lo[1]) > hy || __fsub_rn(p[h].y, hi[1]) < -hy ||
                                      __fsub_rn(p[h].z, lo[2]) > hz || __fsub_rn(p[h].z, hi[2]) < -hz;
                             }
-                            place_padding(p[h], INTS ? 0.f : S.far);
+                            place_padding(p[h], FORCE ? S.far : 0.f);
                         }
                         S.ja[q] = make_float4(p[0].x, p[1].x, p[0].y, p[1].y);
                         S.jb[q] = make_float4(p[0].z, p[1].z, bv[0], bv[1]);
@@ -865,8 +867,13 @@ __global__ void __launch_bounds__(PK_THREADS, (pk_min_blocks<KIND, HL>())) k_pas
                             float v0, v1;
                             unpk2(v, v0, v1);
                             if constexpr (KIND == PASS_DENSITY) {  // units of w/2
-                                if (v0 != 0.f) atomicAdd(&a.hsum[j0], fixed_of_signed(__fmul_rn(v0, hscale) * 2.f));
-                                if (v1 != 0.f) atomicAdd(&a.hsum[j0 + HJ], fixed_of_signed(__fmul_rn(v1, hscale) * 2.f));
+                                const float x0 = __fmul_rn(v0, hscale) * 2.f, x1 = __fmul_rn(v1, hscale) * 2.f;
+                                if (v0 > 0.f) atomicAdd(&a.hsum[j0], fixed_of_nonneg(x0));
+                                if (v1 > 0.f) atomicAdd(&a.hsum[j0 + HJ], fixed_of_nonneg(x1));
+                                if (fminf(v0, v1) < 0.f) {
+                                    if (v0 < 0.f) atomicAdd(&a.hsum[j0], fixed_of_signed(x0));
+                                    if (v1 < 0.f) atomicAdd(&a.hsum[j0 + HJ], fixed_of_signed(x1));
+                                }
                             } else if constexpr (KIND == PASS_COUNT) {
                                 if (__float_as_uint(v0)) atomicAdd(&a.hcnt[j0], __float_as_uint(v0));
                                 if (__float_as_uint(v1)) atomicAdd(&a.hcnt[j0 + HJ], __float_as_uint(v1));
