@@ -86,7 +86,7 @@ struct Status {
     unsigned long long node_visits;
     unsigned long long leaf_visits;
     unsigned long long j_examined;     // j-clusters box-tested against the 8 i-clusters
-    unsigned long long tile_tests;     // (i-cluster, j-cluster) tiles decided by the exact predicate
+    unsigned long long tile_tests;     // (i-cluster, j-cluster) tiles decided by testing all their pairs
     // half search (symmetric lists): reservations in the upper-entry and
     // transposed-tuple buffers (counted even when they do not fit)
     unsigned long long up_used;

@@ -1,5 +1,6 @@
 // Instantiation of the neighborhood pass kernel for PASS_MIN, the distance to
-// the nearest gather neighbor (a minimum reduction; see pass_impl.cuh).
+// the nearest gather neighbor (a minimum reduction; pass_packed.cuh; tiles of
+// fewer than 64 pairs: pass_impl.cuh).
 #include "pass_impl.cuh"
 #include "pass_packed.cuh"
 

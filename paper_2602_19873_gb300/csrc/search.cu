@@ -22,14 +22,14 @@
 // twice the open arithmetic, and a second copy of the code for batches without
 // wraps waited 2.2 cycles per instruction for the instruction cache.
 //
-// What bounds it: instruction issue (0.65 to 0.76 per scheduler and cycle), not
-// DRAM; about half of the time goes to step 4, a quarter to the walk.  The
-// lane-per-item steps replaced a walk that tested one node, four j-clusters and one
-// tile at a time with the whole warp: 78.7k -> 20k warp instructions per
-// super-cluster on the Evrard sphere at 2^21; search stage (half lists, CUDA events)
-// 1.18 -> 0.75 ms there, 15.9 -> 9.2 ms on 2^24 particles in 64 Plummer spheres, 3.36
-// -> 2.22 ms on the 4M-particle fluid.  Fused tile tests, and images instead of
-// wrapped differences: 0.71, 9.0 and 1.69 ms.
+// What bounds it: instruction issue (0.78 per scheduler and cycle on 2^21 particles
+// in 64 Plummer spheres), not DRAM; about half of the time goes to step 4, a quarter
+// to the walk.  The lane-per-item steps replaced a walk that tested one node, four
+// j-clusters and one tile at a time with the whole warp: with fused tile tests 78.7k
+// -> 50k warp instructions per super-cluster on those spheres; search stage (half
+// lists, CUDA events) 1.18 -> 0.75 ms on the Evrard sphere at 2^21, 15.9 -> 9.2 ms on
+// 2^24 particles in 64 Plummer spheres, 3.36 -> 2.22 ms on the 4M-particle fluid.
+// Fused tile tests, and images instead of wrapped differences: 0.71, 9.0 and 1.69 ms.
 #include <algorithm>
 #include <type_traits>
 
@@ -974,7 +974,7 @@ static cudaError_t launch_split(const SearchArgs &a, const SearchCtl &c, int per
                                 cudaStream_t s)
 {
     const uint64_t batches = ((uint64_t)a.nsc * kSC * (M / MJ)) / sr_batch<MJ>() + 2;
-        if (a.nsc <= 3u * (uint32_t)grid && batches <= kSplitBatches && a.stage_cap < 65536u / SR_WARPS)
+    if (a.nsc <= 3u * (uint32_t)grid && batches <= kSplitBatches && a.stage_cap < 65536u / SR_WARPS)
         return launch_m<M, MJ, MODE, true>(a, c, per, (int)std::min<uint32_t>(c.count, (uint32_t)grid), threads, s);
     return launch_m<M, MJ, MODE>(a, c, per, grid, threads, s);
 }
